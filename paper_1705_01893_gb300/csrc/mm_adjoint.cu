@@ -62,7 +62,7 @@ struct DstRowsAdj {           // inverse row DFT output with the conjugate four-
 // The filtered adjoint spectrum b v~ of rows rA, rB of yV; THETA: also the theta sums, with
 // the forward spectrum read from rspec.
 template <int M2, int T, bool THETA>
-__global__ void __launch_bounds__(T, 2) k_row_adjoint(AdjRowParams q) {
+__global__ void __launch_bounds__(T, pass_ctas(T, 8)) k_row_adjoint(AdjRowParams q) {
   extern __shared__ float2 sm[];
   using Lay = RowLayout<M2>;
   __shared__ double red[kAdjN - 1][32];
@@ -211,8 +211,8 @@ __device__ __forceinline__ float4 gather4_map(const ColParams& q, const void* ma
 // Inverse column DFTs of the adjoint spectrum -> t = irfft(b v~)/tau; bin P^T t (the next
 // gbar), accumulate dL/dd += v/tau - t and (THETA) <v, P m'> per chunk.
 template <int M1, int CB, int T, int NC, bool THETA>
-__global__ void __launch_bounds__(T, (T <= 512 ? 2 : 1)) k_col_inverse_adjoint(ColParams q,
-                                                                             AdjColExtra x) {
+__global__ void __launch_bounds__(T, pass_ctas(T, 8)) k_col_inverse_adjoint(ColParams q,
+                                                                          AdjColExtra x) {
   extern __shared__ float2 sm[];
   __shared__ double red[32];
   const int M2 = q.g.M2;

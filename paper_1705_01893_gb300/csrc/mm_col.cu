@@ -12,7 +12,7 @@ namespace mm {
 
 // Persistent over the batch's tiles (chunk ci, column block cb).
 template <int M1, int CB, int T, int NC, int SRC>
-__global__ void __launch_bounds__(T, (T <= 512 ? 2 : 1)) k_col_forward(ColParams q) {
+__global__ void __launch_bounds__(T, pass_ctas(T, 8)) k_col_forward(ColParams q) {
   extern __shared__ float2 sm[];
   const int M2 = q.g.M2;
   const int tpc = M2 / CB;
@@ -34,7 +34,7 @@ __global__ void __launch_bounds__(T, (T <= 512 ? 2 : 1)) k_col_forward(ColParams
 }
 
 template <int M1, int CB, int T, int NC>
-__global__ void __launch_bounds__(T, (T <= 512 ? 2 : 1)) k_col_inverse(ColParams q) {
+__global__ void __launch_bounds__(T, pass_ctas(T, 8)) k_col_inverse(ColParams q) {
   extern __shared__ float2 sm[];
   const int M2 = q.g.M2;
   const int tpc = M2 / CB;

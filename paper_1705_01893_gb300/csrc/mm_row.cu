@@ -6,7 +6,7 @@
 namespace mm {
 
 template <int M2, int T, int MODE>
-__global__ void __launch_bounds__(T, (T <= 512 ? 2 : 1)) k_row(RowParams q) {
+__global__ void __launch_bounds__(T, pass_ctas(T, 12)) k_row(RowParams q) {
   extern __shared__ float2 sm[];
   using Lay = RowLayout<M2>;
   __shared__ float red[32];
