@@ -72,45 +72,53 @@ __global__ void __launch_bounds__(T, pass_ctas(T, 8)) k_col_inverse(ColParams q)
 
 // Copy the caller's pointing into tile order: sample 2 (j1 M2 + j2) + h of a chunk goes to
 // cb (2 CB M1) + j1 (2 CB) + 2 (j2 - cb CB) + h with cb = j2 / CB (CB = col_cb(M1), the
-// column kernels' tile width).  Coalesced writes.
-template <int CB>
+// column kernels' tile width).  A tile's rows are runs of 2 CB >= 8 samples on both sides, so
+// four samples move at once, 16 bytes (8 for FP16 weights); all sizes are powers of two, so
+// the indices are shifts.  Reads the caller's arrays element by element when they don't start
+// on such a boundary.  8 x 2^22 samples with FP32 weights: 250 -> 135 us (one sample a thread
+// with 64-bit divisions before).
+template <typename V4, typename V>
+__device__ __forceinline__ V4 load4(const void* p, int64_t i, bool aligned) {
+  if (aligned) return *reinterpret_cast<const V4*>(static_cast<const V*>(p) + i);
+  V4 r;
+  V* e = reinterpret_cast<V*>(&r);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) e[k] = static_cast<const V*>(p)[i + k];
+  return r;
+}
+
 __global__ void k_tile_pointing(const int32_t* __restrict__ pix, const void* cosw, const void* sinw,
-                                int wbytes, int64_t off, int M1, int M2, int32_t* __restrict__ tpix,
-                                void* tcos, void* tsin) {
-  const int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (o >= 2ll * M1 * M2) return;
-  const int64_t tile = 2ll * CB * M1;
-  const int cb = (int)(o / tile);
-  const int r = (int)(o % tile);
-  const int j1 = r / (2 * CB), w = r % (2 * CB);
-  const int64_t src = off + 2ll * ((int64_t)j1 * M2 + cb * CB) + w;
-  tpix[off + o] = pix[src];
+                                int wbytes, int64_t off, int log_m1, int log_m2, int log_row,
+                                int aligned, int32_t* __restrict__ tpix, void* tcos, void* tsin) {
+  const int o = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+  if (o >= 2 << (log_m1 + log_m2)) return;
+  const int w = o & ((1 << log_row) - 1);
+  const int j1 = (o >> log_row) & ((1 << log_m1) - 1), cb = o >> (log_row + log_m1);
+  const int64_t src = off + (((int64_t)j1 << (log_m2 + 1)) + (cb << log_row) + w), dst = off + o;
+  *reinterpret_cast<int4*>(tpix + dst) = load4<int4, int>(pix, src, aligned & 1);
   if (cosw) {
     if (wbytes == 2) {
-      static_cast<__half*>(tcos)[off + o] = static_cast<const __half*>(cosw)[src];
-      static_cast<__half*>(tsin)[off + o] = static_cast<const __half*>(sinw)[src];
+      *reinterpret_cast<uint2*>(static_cast<__half*>(tcos) + dst) = load4<uint2, uint16_t>(cosw, src, aligned & 2);
+      *reinterpret_cast<uint2*>(static_cast<__half*>(tsin) + dst) = load4<uint2, uint16_t>(sinw, src, aligned & 2);
     } else {
-      static_cast<float*>(tcos)[off + o] = static_cast<const float*>(cosw)[src];
-      static_cast<float*>(tsin)[off + o] = static_cast<const float*>(sinw)[src];
+      *reinterpret_cast<float4*>(static_cast<float*>(tcos) + dst) = load4<float4, float>(cosw, src, aligned & 2);
+      *reinterpret_cast<float4*>(static_cast<float*>(tsin) + dst) = load4<float4, float>(sinw, src, aligned & 2);
     }
   }
 }
 
 cudaError_t launch_tile_pointing(const mm_plan_s* p, cudaStream_t st) {
   const int wb = p->wdtype == MM_W_F16 ? 2 : 4;
+  // chunks of the compile-time path start on multiples of 4 samples
+  const uintptr_t wm = wb == 2 ? 7 : 15;
+  const int aligned = (((uintptr_t)p->pix & 15) == 0 ? 1 : 0) |
+                      ((((uintptr_t)p->cosw | (uintptr_t)p->sinw) & wm) == 0 ? 2 : 0);
   for (int c = 0; c < p->n_chunks; ++c) {
     const ChunkDesc& d = p->h_desc[c];
-    if (p->groups[d.grp].general) continue;   // the general path reads the caller's order
-    const int64_t n = d.n;
-    if (col_cb(d.M1) == 4)
-      k_tile_pointing<4><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
-          p->pix, p->cosw, p->sinw, wb, d.off, d.M1, d.M2, p->tpix, p->tcos, p->tsin);
-    else if (col_cb(d.M1) == 8)
-      k_tile_pointing<8><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
-          p->pix, p->cosw, p->sinw, wb, d.off, d.M1, d.M2, p->tpix, p->tcos, p->tsin);
-    else
-      k_tile_pointing<kColCB><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
-          p->pix, p->cosw, p->sinw, wb, d.off, d.M1, d.M2, p->tpix, p->tcos, p->tsin);
+    if (p->groups[d.grp].general) continue;   // the general path has its own tile copy
+    k_tile_pointing<<<(unsigned)((d.n / 4 + 255) / 256), 256, 0, st>>>(
+        p->pix, p->cosw, p->sinw, wb, d.off, ilog2(d.M1), ilog2(d.M2), ilog2(2 * col_cb(d.M1)), aligned,
+        p->tpix, p->tcos, p->tsin);
   }
   return cudaGetLastError();
 }
