@@ -16,7 +16,8 @@
 #include <unordered_map>
 #include <vector>
 
-#include "mm_internal.cuh"
+#include "mm_colcommon.cuh"
+#include "mm_runbin.cuh"
 
 using namespace mm;
 
@@ -454,16 +455,25 @@ __global__ void k_twiddles(float2* out, int count, int denom_mul, int L) {
   out[m] = make_float2((float)c, (float)s);
 }
 
+// Hit counts and the range check.  A warp takes 32 consecutive samples and issues one add per
+// run of equal pixels (115 -> 45 us on 8 x 2^22 samples at 4 per pixel).
 __global__ void k_hits(const int32_t* __restrict__ pix, int64_t n, int64_t n_pix,
                        int32_t* __restrict__ hits, double* __restrict__ flag) {
-  const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (s >= n) return;
-  const int p = pix[s];
-  if (p < -1 || p >= n_pix) {
-    flag[0] = 1.0;  // any nonzero marks an out-of-range pixel index
-    return;
+  constexpr int U = 4;   // rounds of 32 samples a warp has in flight
+  const int lane = threadIdx.x & 31;
+  const int64_t s0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane) * U + lane;
+  int p[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) p[u] = s0 + 32 * u < n ? pix[s0 + 32 * u] : -1;
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    if (p[u] < -1 || p[u] >= n_pix) flag[0] = 1.0;   // any nonzero marks an index out of range
+    const int before = __shfl_up_sync(0xffffffffu, p[u], 1);
+    const bool head = lane == 0 || p[u] != before;
+    const unsigned later = __ballot_sync(0xffffffffu, head) & ~((2u << lane) - 1u);
+    if (head && p[u] >= 0 && p[u] < n_pix)
+      atomicAdd(hits + p[u], (later ? __ffs(later) - 1 : 32) - lane);
   }
-  if (p >= 0) atomicAdd(hits + p, 1);
 }
 
 struct NoiseArgs {
@@ -554,40 +564,6 @@ __global__ void k_min_psd(const ChunkDesc* desc, const double* psd, double* out)
   }
 }
 
-// Weight blocks: acc12[p][0..B) += (1/tau_c) w w^T, acc12[p][B..2B) += c0_c w w^T
-// (upper triangle 00 01 02 11 12 22 for IQU), w = (1, cos 2psi, sin 2psi).
-__global__ void k_weights_accum(const ChunkDesc* __restrict__ desc, int c,
-                                const int32_t* __restrict__ pix, const void* cosw,
-                                const void* sinw, int half_w, int ncomp,
-                                const double* __restrict__ c0, int64_t n0, int64_t n,
-                                double* __restrict__ acc12, double scale) {
-  const int64_t s = n0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (s >= n) return;
-  const int p = pix[s];
-  if (p < 0) return;
-  const double s1 = scale / desc[c].tau, s2 = c0[c];
-  if (ncomp == 1) {
-    atomicAdd(acc12 + 2 * (int64_t)p, s1);
-    atomicAdd(acc12 + 2 * (int64_t)p + 1, s2);
-    return;
-  }
-  double cw, sw;
-  if (half_w) {
-    cw = __half2float(reinterpret_cast<const __half*>(cosw)[s]);
-    sw = __half2float(reinterpret_cast<const __half*>(sinw)[s]);
-  } else {
-    cw = reinterpret_cast<const float*>(cosw)[s];
-    sw = reinterpret_cast<const float*>(sinw)[s];
-  }
-  const double pr[6] = {1.0, cw, sw, cw * cw, cw * sw, sw * sw};
-  double* a = acc12 + 12 * (int64_t)p;
-#pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    atomicAdd(a + i, s1 * pr[i]);
-    atomicAdd(a + 6 + i, s2 * pr[i]);
-  }
-}
-
 // Eigenvalues of a symmetric 3x3 matrix by the trigonometric closed form (Smith 1961).
 __device__ void sym3_eig(const double* m, double* emin, double* emax) {
   const double a00 = m[0], a01 = m[1], a02 = m[2], a11 = m[3], a12 = m[4], a22 = m[5];
@@ -637,9 +613,15 @@ __global__ void k_pixel_solve(int64_t n_pix, int ncomp, double rcond_min,
     W[p] = ok ? 1.0 / a : 0.0;
     Minv[p] = ok ? 1.0 / b : 0.0;
   } else {
-    const double* A = acc12 + 12 * p;
+    double A[12];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {   // 96 bytes per pixel, 16 at a time
+      const double2 v = reinterpret_cast<const double2*>(acc12 + 12 * p)[i];
+      A[2 * i] = v.x;
+      A[2 * i + 1] = v.y;
+    }
     double wi[6] = {0, 0, 0, 0, 0, 0}, mi[6] = {0, 0, 0, 0, 0, 0};
-    if (ok) {
+    if (ok && !sym3_surely_kept(A, rcond_min)) {
       double emin, emax;
       sym3_eig(A, &emin, &emax);
       ok = emax > 0.0 && emin / emax >= rcond_min;
@@ -647,13 +629,15 @@ __global__ void k_pixel_solve(int64_t n_pix, int ncomp, double rcond_min,
     if (ok) ok = sym3_inv(A, wi) && sym3_inv(A + 6, mi);
     if (!ok)
       for (int i = 0; i < 6; ++i) wi[i] = mi[i] = 0.0;
-    for (int i = 0; i < 6; ++i) {
-      W[6 * p + i] = wi[i];
-      Minv[6 * p + i] = mi[i];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      reinterpret_cast<double2*>(W + 6 * p)[i] = make_double2(wi[2 * i], wi[2 * i + 1]);
+      reinterpret_cast<double2*>(Minv + 6 * p)[i] = make_double2(mi[2 * i], mi[2 * i + 1]);
     }
   }
   valid[p] = ok ? 1 : 0;
-  if (ok) atomicAdd(n_valid, 1ull);
+  const unsigned act = __activemask(), kept = __ballot_sync(act, ok);
+  if ((threadIdx.x & 31) == 0 && kept) atomicAdd(n_valid, (unsigned long long)__popc(kept));
 }
 
 // ------------------------------------------------------------------ map-step kernels
@@ -742,10 +726,27 @@ __global__ void k_map_to4(int64_t n_pix, const double* __restrict__ map,
 }
 
 // ----------------------------------------------------------------- operator kernels
+// Four samples of P m a thread with 16-byte accesses (8-byte for FP16 weights), for arrays on
+// such boundaries; 8 x 2^22 samples of the 512^2 map: 159 -> 98 us (one sample a thread is
+// short of loads in flight).
 template <int NC>
-__global__ void k_gather(int64_t n, const int32_t* __restrict__ pix, const void* cosw,
+__global__ void k_gather_vec(int64_t n4, const int32_t* __restrict__ pix, const void* cosw,
+                             const void* sinw, int half_w, const void* map4, float* __restrict__ out) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= n4) return;
+  ColParams q{};
+  q.pix = pix;
+  q.cosw = cosw;
+  q.sinw = sinw;
+  q.half_w = half_w;
+  q.map4 = map4;
+  __stcs(reinterpret_cast<float4*>(out) + i, gather4<NC>(q, 4 * i));
+}
+
+template <int NC>
+__global__ void k_gather(int64_t s0, int64_t n, const int32_t* __restrict__ pix, const void* cosw,
                          const void* sinw, int half_w, const void* map4, float* __restrict__ out) {
-  const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t s = s0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (s >= n) return;
   const int p = pix[s];
   float v = 0.f;
@@ -766,31 +767,6 @@ __global__ void k_gather(int64_t n, const int32_t* __restrict__ pix, const void*
     }
   }
   out[s] = v;
-}
-
-template <int NC>
-__global__ void k_scatter(int64_t n, const int32_t* __restrict__ pix, const void* cosw,
-                          const void* sinw, int half_w, const float* __restrict__ tod,
-                          double* __restrict__ acc) {
-  const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (s >= n) return;
-  const int p = pix[s];
-  if (p < 0) return;
-  const double t = tod[s];
-  double* a = acc + (int64_t)p * NC;
-  atomicAdd(a, t);
-  if constexpr (NC == 3) {
-    float cw, sw;
-    if (half_w) {
-      cw = __half2float(reinterpret_cast<const __half*>(cosw)[s]);
-      sw = __half2float(reinterpret_cast<const __half*>(sinw)[s]);
-    } else {
-      cw = reinterpret_cast<const float*>(cosw)[s];
-      sw = reinterpret_cast<const float*>(sinw)[s];
-    }
-    atomicAdd(a + 1, t * (double)cw);
-    atomicAdd(a + 2, t * (double)sw);
-  }
 }
 
 template <int NC>
@@ -1322,9 +1298,9 @@ static mm_status plan_create(mm_plan* out, int n_chunks, const int64_t* offsets,
                            cudaMemcpyHostToDevice, s)) != cudaSuccess)
     return fail("fused item lists", e);
   if (L.n_total > 0)
-    k_hits<<<blocks_for(L.n_total, 256), 256, 0, s>>>(pix, L.n_total, n_pix, p->hits, p->scal + kScalTmp);
+    k_hits<<<blocks_for(L.n_total, 4 * 256), 256, 0, s>>>(pix, L.n_total, n_pix, p->hits, p->scal + kScalTmp);
   if (L.n_total > 0 && p->composite)
-    k_hits<<<blocks_for(L.n_total, 256), 256, 0, s>>>(p->pix_b, L.n_total, n_pix, p->hits, p->scal + kScalTmp);
+    k_hits<<<blocks_for(L.n_total, 4 * 256), 256, 0, s>>>(p->pix_b, L.n_total, n_pix, p->hits, p->scal + kScalTmp);
   if ((e = launch_tile_pointing(p, s)) != cudaSuccess) return fail("pointing tile copy", e);
   if ((e = cudaGetLastError()) != cudaSuccess) return fail("set-up kernels", e);
   double flag = 0.0;
@@ -1443,25 +1419,25 @@ extern "C" mm_status mm_set_noise_psd(mm_plan p, const double* psd_dev, const do
   // weight blocks, pixel cut, W and the PCG preconditioner
   const int blk = p->ncomp == 3 ? 6 : 1;
   MM_CUDA(cudaMemsetAsync(p->acc12, 0, sizeof(double) * 2 * blk * p->n_pix, s));
-  // one launch per chunk keeps the chunk's scales without a per-sample search
-  for (int c = 0; c < C; ++c) {
-    const ChunkDesc& d = p->h_desc[c];
+  {
+    const int half_w = p->wdtype == MM_W_F16;
+    const int64_t n0 = p->h_desc[0].off, n1 = p->h_desc[C - 1].off + p->h_desc[C - 1].n;
+    auto blocks = [&](const int32_t* pix, const void* cw, const void* sw, double scale) {
+      if (p->ncomp == 3)
+        return launch_run_bin(BinWeights<3>{p->d_desc, C, cw, sw, half_w, p->c0, scale, p->acc12, 0, 0, 0},
+                              pix, n0, n1, p->n_pix, s);
+      return launch_run_bin(BinWeights<1>{p->d_desc, C, cw, sw, half_w, p->c0, scale, p->acc12, 0, 0, 0},
+                            pix, n0, n1, p->n_pix, s);
+    };
     if (!p->composite) {
-      k_weights_accum<<<blocks_for(d.n, 256), 256, 0, s>>>(
-          p->d_desc, c, p->pix, p->cosw, p->sinw, p->wdtype == MM_W_F16, p->ncomp, p->c0, d.off,
-          d.off + d.n, p->acc12, 1.0);
+      MM_CUDA(blocks(p->pix, p->cosw, p->sinw, 1.0));
     } else {
       // D = P_A^T T_A^-1 P_A + P_B^T T_B^-1 P_B with T_A = T_B = tau / 2 (App. B); the gains
       // enter squared
-      k_weights_accum<<<blocks_for(d.n, 256), 256, 0, s>>>(
-          p->d_desc, c, p->pix, p->cosw, p->sinw, p->wdtype == MM_W_F16, p->ncomp, p->c0, d.off,
-          d.off + d.n, p->acc12, 2.0 * (double)p->gain_a * p->gain_a);
-      k_weights_accum<<<blocks_for(d.n, 256), 256, 0, s>>>(
-          p->d_desc, c, p->pix_b, p->cos_b, p->sin_b, p->wdtype == MM_W_F16, p->ncomp, p->c0,
-          d.off, d.off + d.n, p->acc12, 2.0 * (double)p->gain_b * p->gain_b);
+      MM_CUDA(blocks(p->pix, p->cosw, p->sinw, 2.0 * (double)p->gain_a * p->gain_a));
+      MM_CUDA(blocks(p->pix_b, p->cos_b, p->sin_b, 2.0 * (double)p->gain_b * p->gain_b));
     }
   }
-  LAUNCHED("k_weights_accum");
   unsigned long long* d_nvalid = reinterpret_cast<unsigned long long*>(p->scal + kScalTmp + 1);
   MM_CUDA(cudaMemsetAsync(d_nvalid, 0, 8, s));
   k_pixel_solve<<<blocks_for(p->n_pix, 256), 256, 0, s>>>(p->n_pix, p->ncomp, p->rcond_min, p->hits,
@@ -2348,10 +2324,21 @@ extern "C" mm_status mm_apply_pointing(mm_plan p, const double* map, float* tod_
   cudaStream_t s = S(stream);
   mm_status st = load_map(p, map, s);
   if (st != MM_OK) return st;
-  const unsigned nb = blocks_for(p->n_total, 256);
-  if (p->ncomp == 3) k_gather<3><<<nb, 256, 0, s>>>(p->n_total, p->pix, p->cosw, p->sinw, p->wdtype == MM_W_F16, p->map4, tod_out);
-  else k_gather<1><<<nb, 256, 0, s>>>(p->n_total, p->pix, p->cosw, p->sinw, p->wdtype == MM_W_F16, p->map4, tod_out);
-  LAUNCHED("k_gather");
+  const uintptr_t wmask = p->wdtype == MM_W_F16 ? 7 : 15;
+  const uintptr_t bits = ((uintptr_t)p->pix & 15) | ((uintptr_t)tod_out & 15) |
+                         ((uintptr_t)p->cosw & wmask) | ((uintptr_t)p->sinw & wmask);
+  const int half_w = p->wdtype == MM_W_F16;
+  const int64_t n4 = bits == 0 ? p->n_total / 4 : 0, rest = p->n_total - 4 * n4;
+  if (n4 > 0) {
+    if (p->ncomp == 3) k_gather_vec<3><<<blocks_for(n4, 256), 256, 0, s>>>(n4, p->pix, p->cosw, p->sinw, half_w, p->map4, tod_out);
+    else k_gather_vec<1><<<blocks_for(n4, 256), 256, 0, s>>>(n4, p->pix, nullptr, nullptr, 0, p->map4, tod_out);
+    LAUNCHED("k_gather_vec");
+  }
+  if (rest > 0) {
+    if (p->ncomp == 3) k_gather<3><<<blocks_for(rest, 256), 256, 0, s>>>(4 * n4, p->n_total, p->pix, p->cosw, p->sinw, half_w, p->map4, tod_out);
+    else k_gather<1><<<blocks_for(rest, 256), 256, 0, s>>>(4 * n4, p->n_total, p->pix, nullptr, nullptr, 0, p->map4, tod_out);
+    LAUNCHED("k_gather");
+  }
   return MM_OK;
 }
 
@@ -2363,10 +2350,11 @@ extern "C" mm_status mm_apply_pointing_T(mm_plan p, const float* tod, double* ac
   MM_ARG(p != nullptr && tod != nullptr && acc_out != nullptr, "NULL argument");
   cudaStream_t s = S(stream);
   MM_CUDA(cudaMemsetAsync(acc_out, 0, sizeof(double) * p->ncomp * p->n_pix, s));
-  const unsigned nb = blocks_for(p->n_total, 256);
-  if (p->ncomp == 3) k_scatter<3><<<nb, 256, 0, s>>>(p->n_total, p->pix, p->cosw, p->sinw, p->wdtype == MM_W_F16, tod, acc_out);
-  else k_scatter<1><<<nb, 256, 0, s>>>(p->n_total, p->pix, p->cosw, p->sinw, p->wdtype == MM_W_F16, tod, acc_out);
-  LAUNCHED("k_scatter");
+  const int half_w = p->wdtype == MM_W_F16;
+  if (p->ncomp == 3)
+    MM_CUDA(launch_run_bin(BinPT<3>{tod, p->cosw, p->sinw, half_w, acc_out}, p->pix, 0, p->n_total, p->n_pix, s));
+  else
+    MM_CUDA(launch_run_bin(BinPT<1>{tod, nullptr, nullptr, 0, acc_out}, p->pix, 0, p->n_total, p->n_pix, s));
   return MM_OK;
 }
 

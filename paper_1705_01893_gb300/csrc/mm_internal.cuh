@@ -539,6 +539,19 @@ __device__ __forceinline__ double f32_to_f64(float f) {
   return __longlong_as_double((long long)(e == 0u ? sgn : (sgn | mag)));
 }
 
+// Whether a positive semi-definite symmetric 3x3 block (upper triangle 00 01 02 11 12 22)
+// certainly has eigmin / eigmax >= rcond, without its eigenvalues: with e1 >= e2 >= e3,
+// e1 e2 <= (trace / 2)^2 and e1 <= trace, so e3 / e1 >= 4 det / trace^3.  The margin is far
+// above the rounding of det.  Well cross-linked pixels (about 0.1) pass it; only the others
+// take the trigonometric eigenvalues, whose FP64 acos and cos cost several times the rest of
+// the per-pixel solve.
+__device__ __forceinline__ bool sym3_surely_kept(const double* m, double rcond) {
+  const double tr = m[0] + m[3] + m[5];
+  const double det = m[0] * (m[3] * m[5] - m[4] * m[4]) - m[1] * (m[1] * m[5] - m[4] * m[2]) +
+                     m[2] * (m[1] * m[4] - m[3] * m[2]);
+  return tr > 0.0 && 4.0 * det >= (rcond + 1e-12) * (tr * tr * tr);
+}
+
 // w_M^e for 0 <= e < M from the two-level table (FP64-accurate entries, FP32 product).
 __device__ __forceinline__ float2 tw_big(const Group& g, int e) {
   return cmul(__ldg(&g.tw_hi[e >> g.log_lo]), __ldg(&g.tw_lo[e & ((1 << g.log_lo) - 1)]));

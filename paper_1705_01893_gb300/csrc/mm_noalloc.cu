@@ -5,7 +5,7 @@
 // only receives device pointers from elsewhere -- and still want the binned map.
 #include <mutex>
 
-#include "mm_internal.cuh"
+#include "mm_runbin.cuh"
 
 namespace {
 
@@ -51,39 +51,6 @@ __global__ void k_noalloc_clear(double* s, int64_t len) {
     s[i] = 0.0;
 }
 
-__global__ void k_noalloc_accum(const int32_t* __restrict__ pix, const void* cosw, const void* sinw,
-                                int half_w, const float* __restrict__ tod, int64_t n,
-                                int64_t n_pix, int ncomp, double* __restrict__ s) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int p = pix[i];
-  if (p < 0 || p >= n_pix) return;   // excluded sample (or an index outside the map)
-  const double d = (double)tod[i];
-  double* a = s + (int64_t)p * kNoallocPerPix;
-  if (ncomp == 1) {
-    atomicAdd(a, 1.0);
-    atomicAdd(a + 1, d);
-    return;
-  }
-  double c, w;
-  if (half_w) {
-    c = __half2float(static_cast<const __half*>(cosw)[i]);
-    w = __half2float(static_cast<const __half*>(sinw)[i]);
-  } else {
-    c = static_cast<const float*>(cosw)[i];
-    w = static_cast<const float*>(sinw)[i];
-  }
-  atomicAdd(a + 0, 1.0);
-  atomicAdd(a + 1, c);
-  atomicAdd(a + 2, w);
-  atomicAdd(a + 3, c * c);
-  atomicAdd(a + 4, c * w);
-  atomicAdd(a + 5, w * w);
-  atomicAdd(a + 6, d);
-  atomicAdd(a + 7, c * d);
-  atomicAdd(a + 8, w * d);
-}
-
 // Extreme eigenvalues of a symmetric 3x3 block (trigonometric closed form, Smith 1961).
 __device__ void noalloc_eig(const double* m, double* emin, double* emax) {
   const double a00 = m[0], a01 = m[1], a02 = m[2], a11 = m[3], a12 = m[4], a22 = m[5];
@@ -114,18 +81,26 @@ __global__ void k_noalloc_solve(const double* __restrict__ s, int64_t n_pix, int
   double* o = map + 3 * p;
   o[0] = o[1] = o[2] = 0.0;
   if (!(a[0] > 0.0)) return;
-  double emin, emax;
-  noalloc_eig(a, &emin, &emax);
-  if (!(emax > 0.0) || emin / emax < rcond_min) return;
+  if (!mm::sym3_surely_kept(a, rcond_min)) {
+    double emin, emax;
+    noalloc_eig(a, &emin, &emax);
+    if (!(emax > 0.0) || emin / emax < rcond_min) return;
+  }
   const double A = a[0], B = a[1], C = a[2], D = a[3], E = a[4], F = a[5];
   const double c00 = D * F - E * E, c01 = C * E - B * F, c02 = B * E - C * D;
   const double det = A * c00 + B * c01 + C * c02;
   if (!(det > 0.0) && !(det < 0.0)) return;
   const double c11 = A * F - C * C, c12 = B * C - A * E, c22 = A * D - B * B;
   const double b0 = a[6], b1 = a[7], b2 = a[8];
-  o[0] = (c00 * b0 + c01 * b1 + c02 * b2) / det;
-  o[1] = (c01 * b0 + c11 * b1 + c12 * b2) / det;
-  o[2] = (c02 * b0 + c12 * b1 + c22 * b2) / det;
+  // quotients by one reciprocal and a residual step each (FP64 divisions are several times that)
+  const double id = 1.0 / det;
+  auto over = [&](double v) {
+    const double r = v * id;
+    return fma(fma(-r, det, v), id, r);
+  };
+  o[0] = over(c00 * b0 + c01 * b1 + c02 * b2);
+  o[1] = over(c01 * b0 + c11 * b1 + c12 * b2);
+  o[2] = over(c02 * b0 + c12 * b1 + c22 * b2);
 }
 
 }  // namespace
@@ -171,9 +146,17 @@ extern "C" mm_status mm_binned_map_noalloc(const int32_t* pix, const void* cos2p
   const int64_t len = n_pix * kNoallocPerPix;   // the previous call's contents are cleared
   k_noalloc_clear<<<(unsigned)((len + 255) / 256 < 4096 ? (len + 255) / 256 : 4096), 256, 0, s>>>(
       scratch, len);
-  if (n > 0)
-    k_noalloc_accum<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(
-        pix, cos2psi, sin2psi, weight_dtype == MM_W_F16, tod, n, n_pix, ncomp, scratch);
+  const int half_w = weight_dtype == MM_W_F16;
+  if (ncomp == 3)
+    e = mm::launch_run_bin(mm::BinNormal<3, kNoallocPerPix>{tod, cos2psi, sin2psi, half_w, scratch},
+                           pix, 0, n, n_pix, s);
+  else
+    e = mm::launch_run_bin(mm::BinNormal<1, kNoallocPerPix>{tod, cos2psi, sin2psi, half_w, scratch},
+                           pix, 0, n, n_pix, s);
+  if (e != cudaSuccess) {
+    mm_set_error("mm_binned_map_noalloc: launch failed: %s", cudaGetErrorString(e));
+    return MM_ERR_CUDA;
+  }
   k_noalloc_solve<<<(unsigned)((n_pix + 255) / 256), 256, 0, s>>>(scratch, n_pix, ncomp,
                                                                   rcond_min, map_out);
   e = cudaGetLastError();
