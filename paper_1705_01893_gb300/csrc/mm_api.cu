@@ -180,9 +180,12 @@ static size_t tw_count(int M, int M1, int M2, bool general) {
   return (size_t)tw_size(M1) + tw_size(M2) + (size_t(1) << lo) + (size_t)(M >> lo) + M1 + M2;
 }
 
+// Pairs in a chunk's power-law table (see k_noise_table).
+constexpr int kNoiseTable = 1024 + 32;
+
 // -------------------------------------------------------------------- workspace layout
 struct Layout {
-  size_t desc, chunks, params, tw, hits, valid, W, Minv, acc, acc12, map4, bvec, dtab, nbar, nyq, c0,
+  size_t desc, chunks, params, ntab, tw, hits, valid, W, Minv, acc, acc12, map4, bvec, dtab, nbar, nyq, c0,
       ybuf, scal, tpix, tcos, tsin, lam, iter, map64, groups, gen, gen_rec, gen_ctab, gen_rtab,
       adapt, queue, fitems, fctr, fault, total, ybytes;
   int64_t gen_ccap, gen_rcap;
@@ -316,6 +319,7 @@ static mm_status make_layout(int n_chunks, const int64_t* off, int64_t n_pix, in
   L->desc = take(sizeof(ChunkDesc) * n_chunks);
   L->chunks = take(sizeof(int) * n_chunks);
   L->params = take(sizeof(double) * 4 * n_chunks);
+  L->ntab = take(sizeof(double2) * kNoiseTable * (size_t)n_chunks);
   L->tw = take(sizeof(float2) * tw);
   L->hits = take(sizeof(int32_t) * np);
   L->valid = take(np);
@@ -484,7 +488,35 @@ struct NoiseArgs {
   float* nyq;
   double* c0;
   double* scal;            // lambda max bits, min(Nbar) check at kScalTmp
+  const double2* table;    // power-law tables of every chunk (k_noise_table), or nullptr
 };
+
+// Power law (f_knee / f)^alpha at f = k f_sample / n without a pow per mode.  With k = 2^e m,
+// 1 <= m < 2, and m's leading 11 bits t (1024 <= t < 2048), m = (t / 1024) (1 + d), d < 2^-10:
+//   sigma^2 (f_knee / f)^alpha = A_e B_t (1 + d)^-alpha,
+//   A_e = sigma^2 (f_knee / (2^e f_1))^alpha,  B_t = (t / 1024)^-alpha,  f_1 = f_sample / n,
+// and (1 + d)^-alpha by its binomial series to d^5 (the next term is below 3e-17 for
+// |alpha| <= 4, the range the tables are used in).  A chunk's table: 1024 pairs
+// (B_t, 1024 / t), then A_e for e = 0 .. 31 in the x parts of 32 more.  A pow and two
+// divisions per mode on the narrow FP64 pipe took 4.13 ms for 8 x 2^22 samples.
+__global__ void k_noise_table(const ChunkDesc* __restrict__ desc, const double* __restrict__ params,
+                              double2* __restrict__ table) {
+  const int c = blockIdx.y;
+  const double* q = params + 4 * c;
+  const double alpha = q[2], f1 = q[3] / (double)desc[c].n;
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j < kNoiseTable) {
+    double2 v;
+    if (j < 1024) {
+      v.x = pow((double)(1024 + j) * 0x1p-10, -alpha);
+      v.y = 1024.0 / (double)(1024 + j);
+    } else {
+      v.x = q[0] * q[0] * pow(q[1] / (f1 * (double)(1u << (j - 1024))), alpha);
+      v.y = 0.0;
+    }
+    table[(int64_t)c * kNoiseTable + j] = v;
+  }
+}
 
 __device__ __forceinline__ double psd_value(const NoiseArgs& a, int c, const ChunkDesc& d, int k) {
   if (a.psd) return a.psd[d.nat + k];
@@ -499,39 +531,91 @@ __device__ __forceinline__ double psd_value(const NoiseArgs& a, int c, const Chu
   return q[0] * q[0] * (1.0 + xa);
 }
 
+// 1 / v for normal v in FP32's range: an FP32 reciprocal refined by one cubic Newton step
+// (r + r (e + e^2), e = 1 - v r, |e| < 2^-22, leaves e^3), 3 FP64 instructions.
+__device__ __forceinline__ double recip_refined(double v) {
+  const double r = f32_to_f64(__frcp_rn((float)v));
+  const double e = fma(-v, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
 // Nbar = N - tau on every rfft bin of chunk blockIdx.y, stored on the row-layout slots;
 // also c0 = (1/n) sum_k w_k / N_k, lambda_max and min(Nbar) (Sec. 2.1 needs Nbar >= 0).
+// About 18 FP64 instructions a mode with the tables; the extremes of Nbar are kept as integers
+// (the bits of a double order like the value, negative ones are settled apart) and divided by
+// tau once, so that no comparison takes the FP64 pipe.  8 x 2^22 samples: 4.13 -> 0.58 ms.
+template <bool kTable>
 __global__ void k_noise(NoiseArgs a) {
   const int c = blockIdx.y;
   const ChunkDesc d = a.desc[c];
-  double sum = 0.0, mx = 0.0, mn = 1e300;
+  double A0 = 0.0, b1 = 0.0, b2 = 0.0, b3 = 0.0, b4 = 0.0, b5 = 0.0;
+  const double2* tab = nullptr;
+  bool series = false, small = false;
+  if constexpr (kTable) {
+    const double* q = a.params + 4 * c;
+    const double al = q[2];
+    tab = a.table + (int64_t)c * kNoiseTable;
+    series = fabs(al) <= 4.0 && q[1] > 0.0;
+    A0 = q[0] * q[0];
+    small = A0 > 1e-30 && A0 < 1e30;
+    b1 = -al;
+    b2 = b1 * (-al - 1.0) / 2.0;
+    b3 = b2 * (-al - 2.0) / 3.0;
+    b4 = b3 * (-al - 3.0) / 4.0;
+    b5 = b4 * (-al - 4.0) / 5.0;
+  }
+  auto value = [&](int k) -> double {
+    if constexpr (kTable) {
+      if (series) {
+        const unsigned kk = k == 0 ? 1u : (unsigned)k;   // DC bin floored to bin 1
+        const int e = 31 - __clz((int)kk), sh = e - 10;
+        const unsigned t = sh >= 0 ? kk >> sh : kk << -sh;
+        const unsigned rest = sh > 0 ? kk & ((1u << sh) - 1u) : 0u;
+        const double2 B = __ldg(tab + (t - 1024u));
+        const double Ae = __ldg(&tab[1024 + e].x);
+        // d = rest / (t 2^sh): rest < 2^13 and the power of two are exact in FP32
+        const double x = f32_to_f64((float)rest * __uint_as_float((unsigned)(127 - e) << 23)) * B.y;
+        const double s = fma(x, fma(x, fma(x, fma(x, fma(x, b5, b4), b3), b2), b1), 1.0);
+        return fma(Ae * B.x, s, A0);
+      }
+    }
+    return psd_value(a, c, d, k);
+  };
+  double sum = 0.0, mn = 1e300;
+  long long mx = 0;                  // bits of the largest Nbar >= 0
+  auto extreme = [&](double nb) {
+    const long long u = __double_as_longlong(nb);
+    if (u <= 0x7ff0000000000000ll) mx = u > mx ? u : mx;   // a NaN of a caller's table is passed over
+    if (u < 0) mn = fmin(mn, nb);
+  };
   for (int slot = blockIdx.x * blockDim.x + threadIdx.x; slot < d.M; slot += gridDim.x * blockDim.x) {
-    const int k1 = slot / d.M2, k2 = slot % d.M2;
+    const int k1 = slot / d.M2, k2 = slot - k1 * d.M2;
     const int k = k1 + d.M1 * k2;
     // complex chunks hold every frequency 0..n-1; frequency k is rfft bin min(k, n - k)
     const int kb = d.cplx && 2 * k > d.n ? d.n - k : k;
-    const double N = psd_value(a, c, d, kb);
+    const double N = value(kb);
     const double nb = N - d.tau;
     a.nbar[d.spec + slot] = (float)nb;
-    double w = k == 0 || d.cplx ? 1.0 : 2.0;
-    sum += w / N;
-    mx = fmax(mx, nb / d.tau);
-    mn = fmin(mn, nb);
+    const double r = small && __double2hiint(N) < 0x46293e59 /* 1e30 */ ? recip_refined(N) : 1.0 / N;
+    sum += r;
+    extreme(nb);
     if (k == 0 && d.cplx) a.nyq[c] = 0.f;
     if (k == 0 && !d.cplx) {
-      const double NM = psd_value(a, c, d, d.M);
+      const double NM = value(d.M);
       const double nbM = NM - d.tau;
       a.nyq[c] = (float)nbM;
-      sum += 1.0 / NM;
-      mx = fmax(mx, nbM / d.tau);
-      mn = fmin(mn, nbM);
+      sum -= 0.5 * (r - 1.0 / NM);   // both bins have multiplicity 1, the others 2
+      extreme(nbM);
     }
   }
-  __shared__ double rs[32], rx[32], rn[32];
+  if (!d.cplx) sum += sum;
+  __shared__ double rs[32], rn[32];
+  __shared__ long long rx[32];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     sum += __shfl_down_sync(0xffffffffu, sum, o);
-    mx = fmax(mx, __shfl_down_sync(0xffffffffu, mx, o));
+    const long long ox = __shfl_down_sync(0xffffffffu, mx, o);
+    mx = ox > mx ? ox : mx;
     mn = fmin(mn, __shfl_down_sync(0xffffffffu, mn, o));
   }
   if ((threadIdx.x & 31) == 0) {
@@ -540,11 +624,11 @@ __global__ void k_noise(NoiseArgs a) {
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int i = 1; i < (int)(blockDim.x >> 5); ++i) {
-      sum += rs[i]; mx = fmax(mx, rx[i]); mn = fmin(mn, rn[i]);
+      sum += rs[i]; mx = rx[i] > mx ? rx[i] : mx; mn = fmin(mn, rn[i]);
     }
     atomicAdd(a.c0 + c, sum / (double)d.n);
     atomicMax(reinterpret_cast<unsigned long long*>(a.scal + kScalLambdaMax),
-              (unsigned long long)__double_as_longlong(fmax(mx, 0.0)));
+              (unsigned long long)__double_as_longlong(__longlong_as_double(mx) / d.tau));
     if (mn < 0.0) a.scal[kScalTmp] = fmin(a.scal[kScalTmp], mn);
   }
 }
@@ -1139,6 +1223,7 @@ static mm_status plan_create(mm_plan* out, int n_chunks, const int64_t* offsets,
   p->h_fused_n = nullptr;
   p->scal = reinterpret_cast<double*>(ws + L.scal);
   p->params = reinterpret_cast<double*>(ws + L.params);
+  p->noise_tab = reinterpret_cast<double2*>(ws + L.ntab);
   p->tpix = reinterpret_cast<int32_t*>(ws + L.tpix);
   p->tcos = ncomp == 3 ? static_cast<void*>(ws + L.tcos) : nullptr;
   p->tsin = ncomp == 3 ? static_cast<void*>(ws + L.tsin) : nullptr;
@@ -1399,12 +1484,20 @@ extern "C" mm_status mm_set_noise_psd(mm_plan p, const double* psd_dev, const do
   }
   MM_CUDA(cudaMemsetAsync(p->c0, 0, sizeof(double) * C, s));
   MM_CUDA(cudaMemsetAsync(p->scal, 0, sizeof(double) * kScalCount, s));
-  NoiseArgs na{p->d_desc, psd_dev, d_params, p->nbar, p->nyq, p->c0, p->scal};
+  NoiseArgs na{p->d_desc, psd_dev, d_params, p->nbar, p->nyq, p->c0, p->scal, p->noise_tab};
   {
     int maxM = 0;
     for (int c = 0; c < C; ++c) maxM = p->h_desc[c].M > maxM ? p->h_desc[c].M : maxM;
     const int per = 256 * 16;
-    k_noise<<<dim3((maxM + per - 1) / per, C), 256, 0, s>>>(na);
+    const dim3 grid((maxM + per - 1) / per, C);
+    // tables pay from about their own length on (1056 pow a chunk)
+    if (d_params && maxM >= 8 * kNoiseTable) {
+      k_noise_table<<<dim3(blocks_for(kNoiseTable, 64), C), 64, 0, s>>>(p->d_desc, d_params, p->noise_tab);
+      LAUNCHED("k_noise_table");
+      k_noise<true><<<grid, 256, 0, s>>>(na);
+    } else {
+      k_noise<false><<<grid, 256, 0, s>>>(na);
+    }
     LAUNCHED("k_noise");
   }
   // scal[kScalTmp] holds min(Nbar) if it went negative

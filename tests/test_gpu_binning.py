@@ -72,3 +72,32 @@ def test_weight_blocks_across_chunks(lens, skip):
     plan.apply_pointing(torch.from_numpy(m).cuda(), out)
     ref = np.concatenate([prob.P(m, a, b) for a, b in prob.chunks()])
     assert np.linalg.norm(out.cpu().numpy() - ref) <= 1e-6 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("alpha,fknee", [(0.0, 1.0), (-0.5, 0.3), (0.7, 2.0), (2.0, 0.5), (4.0, 0.01),
+                                         (4.5, 0.01), (2.5, 0.0)])
+@pytest.mark.parametrize("n", [1 << 14, 16875, 20000, 1 << 16])
+def test_noise_tables(n, alpha, fknee):
+    """lambda_max to FP64 accuracy and a step at lambda = 3 (reads every Nbar), plus PCG's second
+    iterate (reads c0), chunks long enough for the tables and slopes in and out of their range."""
+    import torch
+    npix = 64
+    pix, _, _, tod = _pointing(n, npix, 3, 7)
+    params = np.array([[1.3, fknee, alpha, 100.0]])
+    prob = O.problem_from_synth(dict(pix=pix, cos=None, sin=None, tod=tod, offsets=np.array([0, n]),
+                                     npix=npix, ncomp=1, params=params))
+    plan = _plan([0, n], pix, None, None, npix)
+    plan.set_noise(torch.from_numpy(tod).cuda(), params=params)
+    lam = O.lambda_max(prob)
+    assert abs(plan.lambda_max() - lam) <= 1e-12 * max(lam, 1.0)
+    m0 = np.random.default_rng(2).standard_normal((npix, 1))
+    ref, chi = O.messenger_step(prob, m0, 3.0)
+    m = torch.from_numpy(m0.copy()).cuda()
+    x2 = torch.zeros(1, dtype=torch.float64, device="cuda")
+    plan.messenger(m, [3.0], x2)
+    assert np.linalg.norm(m.cpu().numpy() - ref) <= 1e-5 * np.linalg.norm(ref)
+    assert abs(x2.item() - chi) <= 1e-5 * chi
+    x = torch.zeros(npix, 1, dtype=torch.float64, device="cuda")
+    plan.pcg(x, 2)
+    pref, _ = O.pcg(prob, 2)
+    assert np.linalg.norm(x.cpu().numpy() - pref) <= 1e-4 * np.linalg.norm(pref)
