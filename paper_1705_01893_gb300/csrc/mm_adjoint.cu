@@ -299,13 +299,16 @@ __global__ void k_adj_prep(int64_t n_pix, const double* __restrict__ W, const do
 }
 
 // gbar for the previous step: the binned adjoint, on kept pixels; clears the accumulators.
-__global__ void k_adj_take_g(int64_t len, int ncomp, double* __restrict__ acc,
-                             const uint8_t* __restrict__ valid, double* __restrict__ g) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= len) return;
-  const int64_t a = (i % ncomp) * acc_stride_of(len / ncomp, ncomp) + i / ncomp;   // planar
-  g[i] = valid[i / ncomp] ? acc[a] : 0.0;
-  acc[a] = 0.0;
+template <int NC>
+__global__ void k_adj_take_g(int64_t n_pix, double* __restrict__ acc, const uint8_t* __restrict__ valid,
+                             double* __restrict__ g) {
+  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (p >= n_pix) return;
+  double a[NC];
+  take_acc<NC>(acc, n_pix, p, a);
+  const bool ok = valid[p] != 0;
+#pragma unroll
+  for (int i = 0; i < NC; ++i) g[NC * p + i] = ok ? a[i] : 0.0;
 }
 
 // dL/dtheta from the per-chunk sums (tau = sigma^2, Nbar = sigma^2 (f_knee / f)^alpha).
@@ -542,7 +545,7 @@ static mm_status adjoint_backward(mm_plan p, const double* lambdas, int n_iter,
   ADJ_CUDA(cudaMemcpyAsync(g, grad_map_out, mapb, cudaMemcpyDeviceToDevice, s));
   ADJ_CUDA(cudaMemsetAsync(grad_tod, 0, sizeof(float) * (size_t)p->n_total, s));
   ADJ_CUDA(cudaMemsetAsync(acc, 0, sizeof(double) * kAdjN * p->n_chunks, s));
-  const unsigned nbp = (unsigned)((p->n_pix + 255) / 256), nbl = (unsigned)((len + 255) / 256);
+  const unsigned nbp = (unsigned)((p->n_pix + 255) / 256);
   // transposed step i (mi = m_i, mo = m_{i+1}, rs = (P m_i)~: read only for the theta terms)
   auto step = [&](int i, const double* mi, const double* mo, const float2* rs) -> mm_status {
     if (p->ncomp == 3)
@@ -557,7 +560,8 @@ static mm_status adjoint_backward(mm_plan p, const double* lambdas, int n_iter,
       ADJ_CUDA(launch_row_adjoint(p, B, p->ybuf, theta ? rs : nullptr, lambdas[i], acc, s));
       ADJ_CUDA(launch_col_adjoint(p, B, x, theta, s));
     }
-    k_adj_take_g<<<nbl, 256, 0, s>>>(len, p->ncomp, p->acc, p->valid, g);
+    if (p->ncomp == 3) k_adj_take_g<3><<<nbp, 256, 0, s>>>(p->n_pix, p->acc, p->valid, g);
+    else k_adj_take_g<1><<<nbp, 256, 0, s>>>(p->n_pix, p->acc, p->valid, g);
     ADJ_CUDA(cudaGetLastError());
     return MM_OK;
   };

@@ -751,12 +751,7 @@ __global__ void k_bin_apply(int64_t n_pix, double* __restrict__ acc, const doubl
   if (p >= n_pix) return;
   constexpr int B = NC == 3 ? 6 : 1;
   double a[NC], w[B], m[NC];
-#pragma unroll
-  for (int i = 0; i < NC; ++i) {
-    const int64_t j_ = i * acc_stride_of(n_pix, NC) + p;   // planar accumulators
-    a[i] = acc[j_];
-    acc[j_] = 0.0;
-  }
+  take_acc<NC>(acc, n_pix, p, a);
 #pragma unroll
   for (int i = 0; i < B; ++i) w[i] = W[B * p + i];
   sym_apply<NC>(w, a, m);
@@ -776,12 +771,7 @@ __global__ void k_bin_resid(int64_t n_pix, double* __restrict__ acc, const doubl
   if (p >= n_pix) return;
   constexpr int B = NC == 3 ? 6 : 1;
   double a[NC], w[B], u[NC], m[NC];
-#pragma unroll
-  for (int i = 0; i < NC; ++i) {
-    const int64_t j_ = i * acc_stride_of(n_pix, NC) + p;   // planar accumulators
-    a[i] = acc[j_];
-    acc[j_] = 0.0;
-  }
+  take_acc<NC>(acc, n_pix, p, a);
 #pragma unroll
   for (int i = 0; i < B; ++i) w[i] = W[B * p + i];
   sym_apply<NC>(w, a, u);
@@ -869,13 +859,16 @@ __global__ void k_expand_weights(int64_t n_pix, const double* __restrict__ W, do
 }
 
 // b = P^T N^-1 d on valid pixels; acc cleared.
-__global__ void k_finish_b(int64_t len, int ncomp, double* __restrict__ acc,
-                           const uint8_t* __restrict__ valid, double* __restrict__ b) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= len) return;
-  const int64_t a = (i % ncomp) * acc_stride_of(len / ncomp, ncomp) + i / ncomp;   // planar
-  b[i] = valid[i / ncomp] ? acc[a] : 0.0;
-  acc[a] = 0.0;
+template <int NC>
+__global__ void k_finish_b(int64_t n_pix, double* __restrict__ acc, const uint8_t* __restrict__ valid,
+                           double* __restrict__ b) {
+  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (p >= n_pix) return;
+  double a[NC];
+  take_acc<NC>(acc, n_pix, p, a);
+  const bool ok = valid[p] != 0;
+#pragma unroll
+  for (int i = 0; i < NC; ++i) b[NC * p + i] = ok ? a[i] : 0.0;
 }
 
 // ------------------------------------------------------------------------ PCG kernels
@@ -916,14 +909,10 @@ __global__ void k_pcg_init(int64_t n_pix, double* __restrict__ acc, const double
   double rz = 0, xb = 0, xr = 0;
   if (p < n_pix) {
     const bool ok = valid[p] != 0;
-    double rr[NC], zz[NC];
+    double aa[NC], rr[NC], zz[NC];
+    take_acc<NC>(acc, n_pix, p, aa);
 #pragma unroll
-    for (int i = 0; i < NC; ++i) {
-      const int64_t j = NC * p + i;
-      const int64_t ja = i * acc_stride_of(n_pix, NC) + p;   // planar accumulators
-      rr[i] = ok ? bvec[j] - acc[ja] : 0.0;
-      acc[ja] = 0.0;
-    }
+    for (int i = 0; i < NC; ++i) rr[i] = ok ? bvec[NC * p + i] - aa[i] : 0.0;
     block_apply<NC>(Minv, p, rr, zz);
 #pragma unroll
     for (int i = 0; i < NC; ++i) {
@@ -948,18 +937,23 @@ __global__ void k_pcg_init(int64_t n_pix, double* __restrict__ acc, const double
 
 // q = A p on valid pixels (acc cleared), p.q; block 0 records chi^2 of the current iterate
 // and clears the accumulators the update kernel fills.
-__global__ void k_pcg_q(int64_t len, int ncomp, double* __restrict__ acc, const uint8_t* __restrict__ valid,
+template <int NC>
+__global__ void k_pcg_q(int64_t n_pix, double* __restrict__ acc, const uint8_t* __restrict__ valid,
                         const double* __restrict__ pv, double* __restrict__ q, double* sc, int rz_next,
                         const double* cdd, double* chi2_slot) {
   __shared__ double red[32];
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   double s = 0.0;
-  if (i < len) {
-    const int64_t a = (i % ncomp) * acc_stride_of(len / ncomp, ncomp) + i / ncomp;   // planar
-    const double qq = valid[i / ncomp] ? acc[a] : 0.0;
-    acc[a] = 0.0;
-    q[i] = qq;
-    s = pv[i] * qq;
+  if (p < n_pix) {
+    double a[NC];
+    take_acc<NC>(acc, n_pix, p, a);
+    const bool ok = valid[p] != 0;
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+      const double qq = ok ? a[i] : 0.0;
+      q[NC * p + i] = qq;
+      s += pv[NC * p + i] * qq;
+    }
   }
   s = block_sum(s, red);
   if (threadIdx.x == 0) atomicAdd(sc + kPcgPq, s);
@@ -1547,8 +1541,8 @@ extern "C" mm_status mm_set_noise_psd(mm_plan p, const double* psd_dev, const do
     MM_CUDA(cudaMemsetAsync(p->acc, 0, sizeof(double) * p->ncomp * acc_stride_of(p->n_pix, p->ncomp), s));
     RowArgs a{kRowPcgRhs, 1.0, p->scal + kScalCdd, nullptr};
     FOR_BATCHES(L_(launch_row(p, B, a, s)); L_(launch_col_inverse(p, B, s)));
-    const int64_t len = p->ncomp * p->n_pix;
-    k_finish_b<<<blocks_for(len, 256), 256, 0, s>>>(len, p->ncomp, p->acc, p->valid, p->bvec);
+    if (p->ncomp == 3) k_finish_b<3><<<blocks_for(p->n_pix, 256), 256, 0, s>>>(p->n_pix, p->acc, p->valid, p->bvec);
+    else k_finish_b<1><<<blocks_for(p->n_pix, 256), 256, 0, s>>>(p->n_pix, p->acc, p->valid, p->bvec);
     LAUNCHED("k_finish_b");
   }
   unsigned long long nvalid = 0;
@@ -1665,12 +1659,7 @@ __global__ void k_bin_md(int64_t n_pix, double* __restrict__ acc, const double* 
   if (p < n_pix) {
     constexpr int B = NC == 3 ? 6 : 1;
     double a[NC], w[B], m[NC];
-#pragma unroll
-    for (int i = 0; i < NC; ++i) {
-    const int64_t j_ = i * acc_stride_of(n_pix, NC) + p;   // planar accumulators
-    a[i] = acc[j_];
-    acc[j_] = 0.0;
-  }
+    take_acc<NC>(acc, n_pix, p, a);
 #pragma unroll
     for (int i = 0; i < B; ++i) w[i] = W[B * p + i];
     sym_apply<NC>(w, a, m);
@@ -2148,7 +2137,7 @@ extern "C" mm_status mm_pcg_iterate(mm_plan p, int n_iter, double* map_inout, vo
   double* pv = z + len;
   double* q = pv + len;
   double* sc = reinterpret_cast<double*>(static_cast<char*>(state) + up(sizeof(double) * 4 * len));
-  const unsigned nb = blocks_for(p->n_pix, 256), nbl = blocks_for(len, 256);
+  const unsigned nb = blocks_for(p->n_pix, 256);
   const bool tri = p->ncomp == 3;
   if (restart) {
     MM_CUDA(cudaMemsetAsync(sc, 0, sizeof(double) * kPcgNs, s));
@@ -2172,8 +2161,9 @@ extern "C" mm_status mm_pcg_iterate(mm_plan p, int n_iter, double* map_inout, vo
     if (st != MM_OK) return st;
     int cur = kPcgRz0, nxt = kPcgRz1;
     // parity bookkeeping on the host: each call restarts parity at slot 0 after copying
-    k_pcg_q<<<nbl, 256, 0, s>>>(len, p->ncomp, p->acc, p->valid, pv, q, sc, nxt,
-                                p->scal + kScalCdd, chi2_out ? chi2_out + it : nullptr);
+    double* slot = chi2_out ? chi2_out + it : nullptr;
+    if (tri) k_pcg_q<3><<<nb, 256, 0, s>>>(p->n_pix, p->acc, p->valid, pv, q, sc, nxt, p->scal + kScalCdd, slot);
+    else k_pcg_q<1><<<nb, 256, 0, s>>>(p->n_pix, p->acc, p->valid, pv, q, sc, nxt, p->scal + kScalCdd, slot);
     LAUNCHED("k_pcg_q");
     if (tri) k_pcg_update<3><<<nb, 256, 0, s>>>(p->n_pix, map_inout, r, z, pv, q, p->bvec, p->Minv, sc, cur, nxt);
     else k_pcg_update<1><<<nb, 256, 0, s>>>(p->n_pix, map_inout, r, z, pv, q, p->bvec, p->Minv, sc, cur, nxt);

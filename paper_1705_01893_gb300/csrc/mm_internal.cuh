@@ -240,6 +240,17 @@ __host__ __device__ __forceinline__ int64_t acc_stride_of(int64_t n_pix, int nco
   return ncomp == 1 ? n_pix : ((n_pix + 31) / 32) * 32 + 32;
 }
 
+// Read pixel p's sums from the planar accumulators and clear them for the next pass.
+template <int NC>
+__device__ __forceinline__ void take_acc(double* acc, int64_t n_pix, int64_t p, double* a) {
+#pragma unroll
+  for (int i = 0; i < NC; ++i) {
+    double* q = acc + i * acc_stride_of(n_pix, NC) + p;
+    a[i] = *q;
+    *q = 0.0;
+  }
+}
+
 // ------------------------------------------------------------------------- butterflies
 // In-register DFTs of length 2, 4, 8 with kernel exp(DIR * 2 pi i jk / R).
 template <int DIR>
