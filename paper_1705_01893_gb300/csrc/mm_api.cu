@@ -187,7 +187,7 @@ constexpr int kNoiseTable = 1024 + 32;
 struct Layout {
   size_t desc, chunks, params, ntab, tw, hits, valid, W, Minv, acc, acc12, map4, bvec, dtab, nbar, nyq, c0,
       ybuf, scal, tpix, tcos, tsin, lam, iter, map64, groups, gen, gen_rec, gen_ctab, gen_rtab,
-      adapt, queue, fitems, fctr, fault, total, ybytes;
+      adapt, queue, fitems, fctr, fault, small, total, ybytes;
   int64_t gen_ccap, gen_rcap;
   int lam_cap;
   int n_groups;
@@ -370,6 +370,7 @@ static mm_status make_layout(int n_chunks, const int64_t* off, int64_t n_pix, in
   L->fitems = take(sizeof(int2) * (fitems > 0 ? fitems : 1));
   L->fctr = take(sizeof(unsigned) * (2 + 2 * (size_t)n_chunks));
   L->fault = take(16);
+  L->small = take(256 + sizeof(GenChunk) * (size_t)n_chunks);
   L->total = o;
   return MM_OK;
 }
@@ -1100,6 +1101,32 @@ static cudaError_t gen_upload(mm_plan_s* p, cudaStream_t s) {
   return cudaStreamSynchronize(s);
 }
 
+// Per-chunk records of the one-launch path: the group's tables with the radix sequences they
+// were built for (compile-time lengths: pick_radix; general ones: the schedule's order).
+static cudaError_t small_upload(mm_plan_s* p, cudaStream_t s) {
+  if (p->small.clusters == 0) return cudaSuccess;
+  std::vector<GenChunk> rec(p->n_chunks);
+  for (int c = 0; c < p->n_chunks; ++c) {
+    const Group& G = p->groups[p->h_desc[c].grp];
+    GenChunk& R = rec[c];
+    memset(&R, 0, sizeof(R));
+    R.d = p->h_desc[c];
+    R.c = c;
+    R.log_lo = G.log_lo;
+    R.tw_col = G.tw_col; R.tw_row = G.tw_row; R.tw_lo = G.tw_lo; R.tw_hi = G.tw_hi;
+    R.pack_a = G.tw_pack_a; R.pack_b = G.tw_pack_b;
+    if (G.general) {
+      R.nr1 = radix_plan(G.M1, R.rad1, p->gen_tune.radix_order);
+      R.nr2 = radix_plan(G.M2, R.rad2, p->gen_tune.radix_order);
+    } else {
+      for (int ns = 1; ns < G.M1; ns *= R.rad1[R.nr1++]) R.rad1[R.nr1] = (int8_t)pick_radix(G.M1 / ns);
+      for (int ns = 1; ns < G.M2; ns *= R.rad2[R.nr2++]) R.rad2[R.nr2] = (int8_t)pick_radix(G.M2 / ns);
+    }
+  }
+  cudaError_t e = cudaMemcpyAsync(p->small_rec, rec.data(), sizeof(GenChunk) * rec.size(), cudaMemcpyHostToDevice, s);
+  return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
+}
+
 // Second pointing component of a composite plan (App. B).
 struct CompArgs {
   const int32_t* pix_b;
@@ -1217,6 +1244,8 @@ static mm_status plan_create(mm_plan* out, int n_chunks, const int64_t* offsets,
   p->h_fused_n = nullptr;
   p->scal = reinterpret_cast<double*>(ws + L.scal);
   p->params = reinterpret_cast<double*>(ws + L.params);
+  p->small_bar = reinterpret_cast<unsigned*>(ws + L.small);
+  p->small_rec = reinterpret_cast<GenChunk*>(ws + L.small + 256);
   p->noise_tab = reinterpret_cast<double2*>(ws + L.ntab);
   p->tpix = reinterpret_cast<int32_t*>(ws + L.tpix);
   p->tcos = ncomp == 3 ? static_cast<void*>(ws + L.tcos) : nullptr;
@@ -1363,6 +1392,10 @@ static mm_status plan_create(mm_plan* out, int n_chunks, const int64_t* offsets,
                            cudaMemcpyHostToDevice, s)) != cudaSuccess) return fail("group upload", e);
   if (p->n_gen > 0) {
     if ((e = gen_upload(p, s)) != cudaSuccess) return fail("general chunk tables", e);
+  }
+  if (!p->composite) {
+    if ((e = small_shape(p, &p->small)) != cudaSuccess) return fail("one-launch shape", e);
+    if ((e = small_upload(p, s)) != cudaSuccess) return fail("one-launch records", e);
   }
   if ((e = cudaMemsetAsync(p->hits, 0, sizeof(int32_t) * n_pix, s)) != cudaSuccess) return fail("memset", e);
   if ((e = cudaMemsetAsync(p->scal, 0, sizeof(double) * kScalCount, s)) != cudaSuccess) return fail("memset", e);
@@ -1610,6 +1643,10 @@ extern "C" mm_status mm_messenger_iterate(mm_plan p, const double* lambdas, int 
     }
     return MM_OK;
   }
+  if (p->small.clusters > 0) {
+    MM_CUDA(launch_small(p, lambdas, n_iter, map_inout, chi2_out, s));
+    return check_waits(p, s, "mm_messenger_iterate");
+  }
   for (int it = 0; it < n_iter; ++it) {
     RowArgs a{kRowMessenger, lambdas[it], chi2_out ? chi2_out + it : nullptr, nullptr};
     FOR_BATCHES(if (fused_eligible(p, B)) { L_(launch_fused(p, B, a, s)); } else {
@@ -1778,6 +1815,12 @@ extern "C" mm_status mm_messenger_iterate_md(mm_plan p, const double* lambdas, i
   return check_waits(p, s, "mm_messenger_iterate_md");
 }
 
+// The accumulators are zero between launches; a one-launch solve whose grid barrier expired may
+// have left sums in them.
+static cudaError_t clear_after_fault(mm_plan p, cudaStream_t s) {
+  return cudaMemsetAsync(p->acc, 0, sizeof(double) * p->ncomp * acc_stride_of(p->n_pix, p->ncomp), s);
+}
+
 extern "C" mm_status mm_plan_fault_flags(mm_plan p, int* flags, void* stream) {
   MM_ARG(p != nullptr && flags != nullptr, "NULL argument");
   cudaStream_t s = S(stream);
@@ -1785,6 +1828,7 @@ extern "C" mm_status mm_plan_fault_flags(mm_plan p, int* flags, void* stream) {
   MM_CUDA(cudaMemcpyAsync(&f, p->fault, sizeof(int), cudaMemcpyDeviceToHost, s));
   MM_CUDA(cudaStreamSynchronize(s));
   MM_CUDA(cudaMemsetAsync(p->fault, 0, sizeof(int), s));
+  if (f) MM_CUDA(clear_after_fault(p, s));
   *flags = f;
   return MM_OK;
 }
@@ -1798,6 +1842,7 @@ static mm_status check_waits(mm_plan p, cudaStream_t s, const char* who) {
   MM_CUDA(cudaStreamSynchronize(s));
   if (f) {
     MM_CUDA(cudaMemsetAsync(p->fault, 0, sizeof(int), s));
+    MM_CUDA(clear_after_fault(p, s));
     mm_set_error("%s: a bounded wait of the fused launch ran out (its results are wrong)", who);
     return MM_ERR_TIMEOUT;
   }
@@ -2090,9 +2135,16 @@ extern "C" mm_status mm_messenger_graph(mm_plan p, const double* lambdas, int n_
   for (int i = 0; i < n_iter; ++i)
     MM_ARG(lambdas[i] >= 1.0 || isinf(lambdas[i]), "lambdas[%d] = %g must be >= 1 or inf", i, lambdas[i]);
   if (n_iter == 0) return MM_OK;
+  cudaStream_t s = S(stream);
+  if (p->small.clusters > 0) {   // the whole schedule is one launch already
+    if (chi2_out) MM_CUDA(cudaMemsetAsync(chi2_out, 0, sizeof(double) * n_iter, s));
+    mm_status sm = load_map(p, map_inout, s);
+    if (sm != MM_OK) return sm;
+    MM_CUDA(launch_small(p, lambdas, n_iter, map_inout, chi2_out, s));
+    return check_waits(p, s, "mm_messenger_graph");
+  }
   mm_status st = capture_iteration_graph(p);
   if (st != MM_OK) return st;
-  cudaStream_t s = S(stream);
   MM_CUDA(cudaMemcpyAsync(p->lam_table, lambdas, sizeof(double) * n_iter, cudaMemcpyHostToDevice, s));
   MM_CUDA(cudaMemsetAsync(p->iter, 0, sizeof(int), s));
   MM_CUDA(cudaMemcpyAsync(p->chi2_base, &chi2_out, sizeof(double*), cudaMemcpyHostToDevice, s));
@@ -2272,6 +2324,7 @@ extern "C" mm_status mm_chi2_modes(mm_plan p, const double* map, double lambda, 
 static mm_status apply_tune(mm_plan p, const GenTune& t, cudaStream_t s) {
   p->gen_tune = t;
   cudaError_t e = gen_upload(p, s);
+  if (e == cudaSuccess) e = small_upload(p, s);
   if (e != cudaSuccess) {
     mm_set_error("general schedule upload: %s", cudaGetErrorString(e));
     return MM_ERR_CUDA;

@@ -112,6 +112,13 @@ struct GenChunk {
   int8_t rad1[kMaxRadices], rad2[kMaxRadices];
 };
 
+// Shape of the one-launch path of small plans (mm_small.cu): clusters of S CTAs, `tile` words a
+// work buffer, `tables` words of tables; cache: pointing, spectra and tables kept on chip;
+// clusters = 0: not taken.
+struct SmallShape {
+  int S = 0, clusters = 0, tile = 0, tables = 0, cache = 0;
+};
+
 }  // namespace mm
 
 struct mm_plan_s {
@@ -194,6 +201,9 @@ struct mm_plan_s {
   int64_t gen_ccap;
   mm::Group* d_groups;
   mm::GenTune gen_tune;
+  mm::SmallShape small;    // one-launch path: shape, per-chunk records, barrier counter
+  mm::GenChunk* small_rec;
+  unsigned* small_bar;
   int32_t* tpix;    // pointing copied into column-tile order (see k_tile_pointing)
   void* tcos;
   void* tsin;
@@ -620,6 +630,11 @@ bool fused_eligible(const mm_plan_s* p, const Batch& b);
 int fused_items_per_chunk(int M1, int M2, bool general);
 int fused_build_items(int M1, int M2, int count, int2* out);
 cudaError_t launch_fused(const mm_plan_s* p, const Batch& b, const RowArgs& a, cudaStream_t st);
+// The whole schedule of a small plan in one launch per 128 iterations (mm_small.cu); the map
+// is in map4 at launch, chi2 (when given) is zero.
+cudaError_t small_shape(const mm_plan_s* p, SmallShape* out);
+cudaError_t launch_small(const mm_plan_s* p, const double* lambdas, int n_iter, double* map_out,
+                         double* chi2, cudaStream_t st);
 cudaError_t launch_col_inverse(const mm_plan_s* p, const Batch& b, cudaStream_t st);
 cudaError_t launch_tile_pointing(const mm_plan_s* p, cudaStream_t st);
 // General path (mm_gen.cu): the same three stages for a batch of general-length chunks,
