@@ -78,29 +78,38 @@ __device__ __forceinline__ void kernel_body_job(const RowParams& q, float2* sm, 
                     mode == kRowMessengerKeep;
   const bool inv = mess || mode == kRowPcgApply || mode == kRowPcgRhs;
 
+  // The job's constants come from thread 0: FP64 products and conversions in every warp, and a
+  // chain of them in thread 0 that all others wait for, held up each job by 2 to 3 of 46
+  // thousand cycles.  They are ready by the first barrier of the forward row DFTs.
+  __shared__ float s_con[2];    // tau, lambda tau
+  double* chi2 = q.a.chi2;
+  bool lam_inf = false;
+  {
+    double lambda = q.a.lambda;
+    if (q.a.lam_table) {          // graph mode: schedule and chi^2 slot from device memory
+      const int it = *q.a.iter;
+      lambda = q.a.lam_table[it];
+      chi2 = q.a.chi2_base[0] ? q.a.chi2_base[0] + it : nullptr;
+    }
+    lam_inf = (__double2hiint(lambda) & 0x7fffffff) == 0x7ff00000;
+    if (threadIdx.x == 0) {
+      s_con[0] = (float)d.tau;
+      s_con[1] = mess && lam_inf ? 0.f : (float)(lambda * d.tau);
+    }
+    if (!fwd) __syncthreads();
+  }
+
   if (fwd) {
     const SrcRows<kStream> src{y, rA * M2, rB * M2};
     smem_fft<M2, 2, Lay, T, -1>(sm, tws, src);
   }
 
   // per-mode constants
-  const float tau = (float)d.tau;
+  const float tau = s_con[0], lt = s_con[1];
   const float inv_n = 1.0f / (float)d.n;
-  double lambda = q.a.lambda;
-  double* chi2 = q.a.chi2;
-  if (q.a.lam_table) {          // graph mode: schedule and chi^2 slot from device memory
-    const int it = *q.a.iter;
-    lambda = q.a.lam_table[it];
-    chi2 = q.a.chi2_base[0] ? q.a.chi2_base[0] + it : nullptr;
-  }
-  float lt = 0.f;               // lambda * tau
-  bool lam_inf = false;
-  if (mess) {
-    lam_inf = isinf(lambda);
-    lt = lam_inf ? 0.f : (float)(lambda * d.tau);
-  }
+  if (!mess) lam_inf = false;
   // N' = Nbar + cn for chi^2: tau (Eq. 3) or lambda tau (chi^2(m, lambda))
-  const float cn = (mode == kRowChi2 || mode == kRowChi2Modes) ? (float)(lambda * d.tau) : tau;
+  const float cn = (mode == kRowChi2 || mode == kRowChi2Modes) ? lt : tau;
   // output scale: irfft normalisation 1/n, and T^-1 = 1/tau for the messenger map step
   const float sc = mess ? inv_n / tau : inv_n;
   const float2* dt = q.dtab + d.spec;
@@ -252,15 +261,16 @@ __device__ __forceinline__ void kernel_body_job(const RowParams& q, float2* sm, 
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) x2 += __shfl_down_sync(0xffffffffu, x2, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x2;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double s = 0.0;
-      for (int i = 0; i < T / 32; ++i) s += red[i];
-      atomicAdd(chi2, s / (double)d.n);
-    }
+  }
+  if (inv || want_x2) __syncthreads();
+  if (want_x2 && threadIdx.x >= T - 32) {   // one warp; the others go on
+    const int lane = threadIdx.x & 31;
+    double s = lane < T / 32 ? f32_to_f64(red[lane]) : 0.0;
+#pragma unroll
+    for (int o = T / 64; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) atomicAdd(chi2, s * (double)inv_n);   // n is a power of two: 1/n is exact
   }
   if (!inv) return;
-  __syncthreads();
   smem_fft<M2, 2, Lay, T, +1>(sm, tws, SmemIO{}, DstRows<kStream>{y, &q.g, rA, rB, self});
 }
 
