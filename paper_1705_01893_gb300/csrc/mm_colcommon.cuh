@@ -39,14 +39,26 @@ __device__ __forceinline__ float4 load_w4(const void* w, int half_w, int64_t s) 
   return __ldcs(reinterpret_cast<const float4*>(static_cast<const float*>(w) + s));
 }
 
+// (P m) of two consecutive samples.  They share a pixel more often than not, and then one map
+// load serves both: the gathers are short of L1 requests (a vertical sweep touches a line per
+// pixel), not of bytes.  256^2, 4 x 2^20: 1523 -> 1461 us per
+// 21 iterations; the 20-step gradient 6424 -> 6009 us; 512^2, 8 x 2^22: 435 -> 432 us an iteration.
 template <int NC>
-__device__ __forceinline__ float gather_one(const ColParams& q, int p, float cw, float sw) {
-  if (p < 0) return 0.f;
+__device__ __forceinline__ float2 gather_two(const ColParams& q, int p0, int p1, float c0, float c1,
+                                             float s0, float s1) {
   if constexpr (NC == 1) {
-    return __ldg(reinterpret_cast<const float*>(q.map4) + p);
+    const float* map = reinterpret_cast<const float*>(q.map4);
+    const float a = p0 < 0 ? 0.f : __ldg(map + p0);
+    float b = a;
+    if (p1 != p0) b = p1 < 0 ? 0.f : __ldg(map + p1);
+    return make_float2(a, b);
   } else {
-    const float4 m = __ldg(reinterpret_cast<const float4*>(q.map4) + p);
-    return fmaf(sw, m.z, fmaf(cw, m.y, m.x));
+    const float4* map = reinterpret_cast<const float4*>(q.map4);
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (p0 >= 0) a = __ldg(map + p0);
+    float4 b = a;
+    if (p1 != p0) b = p1 < 0 ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(map + p1);
+    return make_float2(fmaf(s0, a.z, fmaf(c0, a.y, a.x)), fmaf(s1, b.z, fmaf(c1, b.y, b.x)));
   }
 }
 
@@ -59,8 +71,9 @@ __device__ __forceinline__ float4 gather4(const ColParams& q, int64_t s) {
     c = load_w4(q.cosw, q.half_w, s);
     w = load_w4(q.sinw, q.half_w, s);
   }
-  return make_float4(gather_one<NC>(q, p.x, c.x, w.x), gather_one<NC>(q, p.y, c.y, w.y),
-                     gather_one<NC>(q, p.z, c.z, w.z), gather_one<NC>(q, p.w, c.w, w.w));
+  const float2 lo = gather_two<NC>(q, p.x, p.y, c.x, c.y, w.x, w.y);
+  const float2 hi = gather_two<NC>(q, p.z, p.w, c.z, c.w, w.z, w.w);
+  return make_float4(lo.x, lo.y, hi.x, hi.y);
 }
 
 // One FP64 add per component into the planar accumulators.  Planar, because the lanes of a
@@ -177,7 +190,7 @@ struct SrcGather {   // z = ((P m)_s, (P m)_s+1), Eq. 1; tile-ordered pointing f
         cw0 = c.x; cw1 = c.y; sw0 = w.x; sw1 = w.y;
       }
     }
-    return make_float2(gather_one<NC>(*q, p.x, cw0, sw0), gather_one<NC>(*q, p.y, cw1, sw1));
+    return gather_two<NC>(*q, p.x, p.y, cw0, cw1, sw0, sw1);
   }
 };
 
