@@ -120,6 +120,23 @@ __device__ __forceinline__ void scatter4(const ColParams& q, int64_t s, float4 t
     v[2][i] = tv[i] * sw[i];
   }
   const bool b1 = p[1] != p[0], b2 = p[2] != p[1], b3 = p[3] != p[2];
+  const int prev3 = __shfl_up_sync(0xffffffffu, p[3], 1);
+  const bool cont = qpos != 0 && p[0] == prev3;
+  if (__all_sync(0xffffffffu, !b1 && !b3 && !cont)) {
+    // every lane holds one pixel, or two of two samples each, and none runs on into the next
+    // lane (an even number of samples per pixel): no scan, at most two runs.  4 samples per
+    // pixel, 512^2, 8 x 2^22: 432 -> 414 us an iteration; PCG on it 4137 -> 3978 us per 8.
+    float h[2][3];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      h[0][k] = v[k][0] + v[k][1];
+      h[1][k] = v[k][2] + v[k][3];
+      if (!b2) h[0][k] += h[1][k];
+    }
+    emit_run<NC>(q.acc, q.acc_stride, p[0], h[0][0], h[0][1], h[0][2], pol);
+    if (b2) emit_run<NC>(q.acc, q.acc_stride, p[2], h[1][0], h[1][1], h[1][2], pol);
+    return;
+  }
   const bool single = !(b1 || b2 || b3);
   const int f = b1 ? 1 : (b2 ? 2 : (b3 ? 3 : 4));   // leading run [0, f)
   const int l = b3 ? 3 : (b2 ? 2 : (b1 ? 1 : 0));   // trailing run [l, 4)
@@ -134,8 +151,6 @@ __device__ __forceinline__ void scatter4(const ColParams& q, int64_t s, float4 t
       trail[k] += i >= l ? v[k][i] : 0.f;
     }
   }
-  const int prev3 = __shfl_up_sync(0xffffffffu, p[3], 1);
-  const bool cont = qpos != 0 && p[0] == prev3;
   float S[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) S[k] = cont ? lead[k] : 0.f;
