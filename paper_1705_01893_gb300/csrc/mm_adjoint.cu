@@ -17,6 +17,7 @@
 #include <math.h>
 
 #include "mm_colcommon.cuh"
+#include "mm_rowcommon.cuh"
 
 namespace mm {
 
@@ -47,18 +48,6 @@ struct Src2Rows {             // rows rA (b = 0) and rB (b = 1) of yV
   }
 };
 
-struct DstRowsAdj {           // inverse row DFT output with the conjugate four-step twiddle
-  float2* y;
-  const Group* g;
-  int rA, rB;
-  bool self;
-  __device__ __forceinline__ void operator()(int b, int i, float2 v) const {
-    if (b && self) return;
-    const int r = b ? rB : rA;
-    y[(int64_t)r * g->M2 + i] = cmulc(v, tw_big(*g, r * i));
-  }
-};
-
 // The filtered adjoint spectrum b v~ of rows rA, rB of yV; THETA: also the theta sums, with
 // the forward spectrum read from rspec.
 template <int M2, int T, bool THETA>
@@ -66,6 +55,7 @@ __global__ void __launch_bounds__(T, pass_ctas(T, 8)) k_row_adjoint(AdjRowParams
   extern __shared__ float2 sm[];
   using Lay = RowLayout<M2>;
   __shared__ double red[kAdjN - 1][32];
+  __shared__ float2 s4[2 * four_step_n(M2, kRowLo)];
   float2* tws = sm + 2 * M2;
   for (int i = threadIdx.x; i < tw_size(M2); i += T) tws[i] = q.g.tw_row[i];
   __syncthreads();
@@ -81,6 +71,7 @@ __global__ void __launch_bounds__(T, pass_ctas(T, 8)) k_row_adjoint(AdjRowParams
     const int rB = (M1 - rA) & (M1 - 1);
     const bool self = rA == rB;
     float2* yV = q.yV + (int64_t)ci * M;
+    load_row_twiddles<M2, T>(s4, q.g, rA, rB);
     smem_fft<M2, 2, Lay, T, -1>(sm, tws, Src2Rows{yV, rA * M2, rB * M2});
 
     const float tau = (float)d.tau;
@@ -189,7 +180,7 @@ __global__ void __launch_bounds__(T, pass_ctas(T, 8)) k_row_adjoint(AdjRowParams
     } else {
       __syncthreads();
     }
-    smem_fft<M2, 2, Lay, T, +1>(sm, tws, SmemIO{}, DstRowsAdj{yV, &q.g, rA, rB, self});
+    smem_fft<M2, 2, Lay, T, +1>(sm, tws, SmemIO{}, DstRows<M2>{yV, s4, rA, rB, self});
     __syncthreads();
   }
 }

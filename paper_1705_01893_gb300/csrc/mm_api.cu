@@ -177,7 +177,8 @@ static size_t tw_count(int M, int M1, int M2, bool general) {
   if (general)
     return (size_t)2 * M1 + 2 * M2 + (size_t(1) << kGenLogLo) + (size_t)(M >> kGenLogLo) + 1 + M1 + M2;
   const int lo = log_lo_of(M);
-  return (size_t)tw_size(M1) + tw_size(M2) + (size_t(1) << lo) + (size_t)(M >> lo) + M1 + M2;
+  return (size_t)tw_size(M1) + tw_size(M2) + (size_t(1) << lo) + (size_t)(M >> lo) + M1 + M2 +
+         (size_t)M2 * four_step_n(M1, kColLo) + (size_t)M1 * four_step_n(M2, kRowLo);
 }
 
 // Pairs in a chunk's power-law table (see k_noise_table).
@@ -458,6 +459,26 @@ __global__ void k_twiddles(float2* out, int count, int denom_mul, int L) {
   double s, c;
   sincospi(-2.0 * (double)m * (double)denom_mul / (double)L, &s, &c);
   out[m] = make_float2((float)c, (float)s);
+}
+
+// The per-tile and per-row four-step twiddles (Group::tw_c4, tw_r4) of one shape, in FP64: the
+// cos and sin of an exact fraction e / M of a turn, e = x y mod M.
+__global__ void k_four_step(float2* __restrict__ c4, float2* __restrict__ r4, int M, int M1, int M2, int cb) {
+  const int nc = four_step_n(M1, kColLo), nr = four_step_n(M2, kRowLo);
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t cols = (int64_t)M2 * nc;
+  if (i >= cols + (int64_t)M1 * nr) return;
+  int64_t e;
+  if (i < cols) {
+    const int b = (int)(i % cb), x = (int)(i / cb % nc), t = (int)(i / ((int64_t)cb * nc));
+    e = (int64_t)(x < kColLo ? x : (x - kColLo) * kColLo) * (t * cb + b);
+  } else {
+    const int x = (int)((i - cols) % nr), r = (int)((i - cols) / nr);
+    e = (int64_t)(x < kRowLo ? x : (x - kRowLo) * kRowLo) * r;
+  }
+  double sn, cs;
+  sincospi(-2.0 * (double)(e & (M - 1)) / (double)M, &sn, &cs);
+  (i < cols ? c4[i] : r4[i - cols]) = make_float2((float)cs, (float)sn);
 }
 
 // Hit counts and the range check.  A warp takes 32 consecutive samples and issues one add per
@@ -1314,6 +1335,11 @@ static mm_status plan_create(mm_plan* out, int n_chunks, const int64_t* offsets,
     G.tw_row = t; t += G.general ? 2 * G.M2 : tw_size(G.M2);
     G.tw_lo = t; t += (1 << G.log_lo);
     G.tw_hi = t; t += (G.M >> G.log_lo) + (G.general ? 1 : 0);
+    G.tw_c4 = G.tw_r4 = nullptr;
+    if (!G.general) {
+      G.tw_c4 = t; t += (size_t)G.M2 * four_step_n(G.M1, kColLo);
+      G.tw_r4 = t; t += (size_t)G.M1 * four_step_n(G.M2, kRowLo);
+    }
     G.tw_pack_a = t; t += G.M1;
     G.tw_pack_b = t; t += G.M2;
     tw_off += tw_count(G.M, G.M1, G.M2, G.general);
@@ -1379,6 +1405,8 @@ static mm_status plan_create(mm_plan* out, int n_chunks, const int64_t* offsets,
     } else {
       k_pass_twiddles<<<blocks_for(tw_size(G.M1), 256), 256, 0, s>>>(G.tw_col, G.M1);
       k_pass_twiddles<<<blocks_for(tw_size(G.M2), 256), 256, 0, s>>>(G.tw_row, G.M2);
+      const int64_t cnt = (int64_t)G.M2 * four_step_n(G.M1, kColLo) + (int64_t)G.M1 * four_step_n(G.M2, kRowLo);
+      k_four_step<<<blocks_for(cnt, 256), 256, 0, s>>>(G.tw_c4, G.tw_r4, G.M, G.M1, G.M2, col_cb(G.M1));
     }
     const int nhi = (G.M >> G.log_lo) + (G.general ? 1 : 0);
     struct { float2* o; int cnt, mul, L; } tabs[4] = {

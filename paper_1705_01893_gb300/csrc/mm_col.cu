@@ -14,6 +14,7 @@ namespace mm {
 template <int M1, int CB, int T, int NC, int SRC>
 __global__ void __launch_bounds__(T, pass_ctas(T, 8)) k_col_forward(ColParams q) {
   extern __shared__ float2 sm[];
+  __shared__ float2 s4[SRC == kSrcTod ? 1 : four_step_n(M1, kColLo) * CB];
   const int M2 = q.g.M2;
   const int tpc = M2 / CB;
   const int ntiles = q.count * tpc;
@@ -22,13 +23,15 @@ __global__ void __launch_bounds__(T, pass_ctas(T, 8)) k_col_forward(ColParams q)
     const ChunkDesc d = q.desc[q.chunks[ci]];
     const int cb = t % tpc;
     const int j2_0 = cb * CB;
-    const DstY<true> dst{q.ybuf + (int64_t)ci * d.M, &q.g, j2_0, M2};
-    if constexpr (SRC == kSrcTod)
-      smem_fft<M1, CB, ColLayout<CB>, T, -1>(sm, q.g.tw_col,
-                                             SrcTod{q.tod, d.off + 2ll * j2_0, M2}, dst);
-    else
+    if constexpr (SRC == kSrcTod) {
+      smem_fft<M1, CB, ColLayout<CB>, T, -1>(sm, q.g.tw_col, SrcTod{q.tod, d.off + 2ll * j2_0, M2},
+                                             DstYData{q.ybuf + (int64_t)ci * d.M, &q.g, j2_0, M2});
+    } else {
+      load_col_twiddles<M1, CB, T>(s4, q.g, cb);
       smem_fft<M1, CB, ColLayout<CB>, T, -1>(
-          sm, q.g.tw_col, SrcGather<NC, CB>{&q, d.off + (int64_t)cb * (2 * CB * M1)}, dst);
+          sm, q.g.tw_col, SrcGather<NC, CB>{&q, d.off + (int64_t)cb * (2 * CB * M1)},
+          DstY<M1, CB, true>{q.ybuf + (int64_t)ci * d.M, s4, j2_0, M2});
+    }
     __syncthreads();
   }
 }

@@ -218,20 +218,47 @@ struct SrcTod {      // z = (d_s, d_s+1)
   }
 };
 
+// The four-step twiddles of column tile cb into shared memory (four_step_n(M1, kColLo) x CB
+// entries); ready after the next barrier.
+template <int M1, int CB, int T>
+__device__ __forceinline__ void load_col_twiddles(float2* s4, const Group& g, int cb) {
+  constexpr int N = four_step_n(M1, kColLo) * CB;
+  const float2* src = g.tw_c4 + (int64_t)cb * N;
+#pragma unroll
+  for (int i = threadIdx.x; i < N; i += T) s4[i] = __ldg(src + i);
+  // a one-pass column DFT has no barrier of its own before its output
+  if constexpr (M1 <= 16) __syncthreads();
+}
+
 // y[k1][j2] = Z * w_M^(k1 j2): the four-step twiddle on the way out.  kStream: the
 // intermediate is written with evict-first priority (separate pass kernels, whose next
 // reader comes a whole batch later), leaving L2 to the map and the accumulators.
-template <bool kStream = false>
+template <int M1, int CB, bool kStream = false>
 struct DstY {
+  float2* y;
+  const float2* s4;    // load_col_twiddles
+  int j2_0;
+  int M2;
+  __device__ __forceinline__ void operator()(int b, int k1, float2 v) const {
+    float2 w = s4[(k1 & (four_step_lo(M1, kColLo) - 1)) * CB + b];
+    if constexpr (M1 > kColLo) w = cmul(s4[(kColLo + k1 / kColLo) * CB + b], w);
+    const float2 o = cmul(v, w);
+    if constexpr (kStream) __stcs(y + (int64_t)k1 * M2 + j2_0 + b, o);
+    else y[(int64_t)k1 * M2 + j2_0 + b] = o;
+  }
+};
+
+// The same with the plan-wide two-level table, for the transform of the data: it runs once per
+// data set, and its rounding reaches every later iterate through d~ (1/f noise spreads it over
+// the high frequencies), so it stays as it was.
+struct DstYData {
   float2* y;
   const Group* g;
   int j2_0;
   int M2;
   __device__ __forceinline__ void operator()(int b, int k1, float2 v) const {
     const int j2 = j2_0 + b;
-    const float2 o = cmul(v, tw_big(*g, k1 * j2));
-    if constexpr (kStream) __stcs(y + (int64_t)k1 * M2 + j2, o);
-    else y[(int64_t)k1 * M2 + j2] = o;
+    __stcs(y + (int64_t)k1 * M2 + j2, cmul(v, tw_big(*g, k1 * j2)));
   }
 };
 

@@ -51,6 +51,9 @@ template <int M1, int M2, int CB, int T, int NC, int MODE>
 __global__ void __launch_bounds__(T, 2) k_fused(FusedParams q) {
   extern __shared__ float2 sm[];
   __shared__ float red[32];
+  // four-step twiddles of the current column tile or row pair
+  constexpr int kC4 = four_step_n(M1, kColLo) * CB, kR4 = 2 * four_step_n(M2, kRowLo);
+  __shared__ float2 s4[kC4 > kR4 ? kC4 : kR4];
   __shared__ int2 s_it;
   // chunks this CTA has already seen complete (A tiles, B jobs): no second acquire poll
   constexpr int kMaskWords = 64;
@@ -93,7 +96,8 @@ __global__ void __launch_bounds__(T, 2) k_fused(FusedParams q) {
     __syncthreads();
     const ChunkDesc d = q.c.desc[q.c.chunks[ci]];
     if (kind == kItemA) {
-      const DstY<> dst{q.c.ybuf + (int64_t)ci * d.M, &q.c.g, idx * CB, M2};
+      load_col_twiddles<M1, CB, T>(s4, q.c.g, idx);
+      const DstY<M1, CB> dst{q.c.ybuf + (int64_t)ci * d.M, s4, idx * CB, M2};
       smem_fft<M1, CB, ColLayout<CB>, T, -1>(
           sm, q.c.g.tw_col, SrcGather<NC, CB>{&q.c, d.off + (int64_t)idx * (2 * CB * M1)}, dst);
     } else if (kind == kItemB) {
@@ -107,7 +111,7 @@ __global__ void __launch_bounds__(T, 2) k_fused(FusedParams q) {
           prefetch_l2(q.r.nbar + d.spec + (int64_t)rb * M2, 4 * M2);
         }
       }
-      kernel_body_job<M2, T, MODE>(q.r, sm, tws, red, ci, idx);
+      kernel_body_job<M2, T, MODE>(q.r, sm, tws, red, s4, ci, idx);
     } else {
       constexpr int RUN = 2 * CB, NS = M1 * RUN, ROWL = RUN / 4;
       using Lay = ColLayout<CB>;

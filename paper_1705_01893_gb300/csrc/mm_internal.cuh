@@ -46,6 +46,10 @@ struct Group {
   float2* tw_row;          // per-pass twiddles of the length-M2 DFT (general: [< 2 M2])
   float2* tw_lo;           // [2^log_lo]          exp(-2 pi i m / M)
   float2* tw_hi;           // [M >> log_lo (+1)]   exp(-2 pi i m 2^log_lo / M)
+  // four-step twiddles by tile and row (power-of-two lengths; see four_step_lo): column tile t:
+  // [N][CB] of exp(-2 pi i e j2 / M), e = 0 .. lo - 1, then multiples of lo; row r: [N] likewise
+  float2* tw_c4;
+  float2* tw_r4;
   float2* tw_pack_a;       // [M1]  exp(-2 pi i m / (2M))     (real-pack twiddle, k1 part)
   float2* tw_pack_b;       // [M2]  exp(-2 pi i m M1 / (2M))  (real-pack twiddle, k2 part)
 };
@@ -573,6 +577,20 @@ __device__ __forceinline__ bool sym3_surely_kept(const double* m, double rcond) 
                      m[2] * (m[1] * m[4] - m[3] * m[2]);
   return tr > 0.0 && 4.0 * det >= (rcond + 1e-12) * (tr * tr * tr);
 }
+
+// Four-step twiddles w_M^{k1 j2} of a column tile (fixed j2, k1 < M1) or of a row (fixed k1,
+// j2 < M2): w^{x y} with x split into low bits and the rest, from lo + L / lo FP64-accurate
+// entries per column or row that a tile or job copies into shared memory.  The plan-wide
+// two-level table (48 KB at M = 2^23) took two L1 or L2 loads and index arithmetic an element,
+// beside the streams that empty L1; without those loads the fused launch of 32 x 2^24 samples
+// ran 8% faster; with the entries from shared memory 32 x 2^24
+// samples take 34.7 -> 32.1 ms per 4 iterations, 8 x 2^22 414 -> 390 us an iteration, 4 x 2^20
+// 67 -> 63 us.
+__host__ __device__ constexpr int four_step_lo(int L, int most) { return L < most ? L : most; }
+__host__ __device__ constexpr int four_step_n(int L, int most) {
+  return four_step_lo(L, most) + (L > most ? L / most : 0);
+}
+constexpr int kColLo = 32, kRowLo = 64;
 
 // w_M^e for 0 <= e < M from the two-level table (FP64-accurate entries, FP32 product).
 __device__ __forceinline__ float2 tw_big(const Group& g, int e) {

@@ -10,6 +10,7 @@ __global__ void __launch_bounds__(T, pass_ctas(T, 12)) k_row(RowParams q) {
   extern __shared__ float2 sm[];
   using Lay = RowLayout<M2>;
   __shared__ float red[32];
+  __shared__ float2 s4[2 * four_step_n(M2, kRowLo)];
   const int jobs_pc = q.g.M1 / 2 + 1;
   const int njobs = q.count * jobs_pc;
   const int mode = MODE >= 0 ? MODE : q.a.mode;
@@ -52,7 +53,7 @@ __global__ void __launch_bounds__(T, pass_ctas(T, 12)) k_row(RowParams q) {
         prefetch_l2(q.nbar + dn.spec + (int64_t)rb * M2, 4 * M2);
       }
     }
-    kernel_body_job<M2, T, MODE, true>(q, sm, tws, red, ci, job % jobs_pc);
+    kernel_body_job<M2, T, MODE, true>(q, sm, tws, red, s4, ci, job % jobs_pc);
     __syncthreads();
     job = s_next;
     __syncthreads();

@@ -46,24 +46,37 @@ struct SrcRows {
   }
 };
 
-template <bool kStream = false>
+// The four-step twiddles of rows rA and rB into shared memory (four_step_n(M2, kRowLo) entries
+// each); ready after the next barrier.
+template <int M2, int T>
+__device__ __forceinline__ void load_row_twiddles(float2* s4, const Group& g, int rA, int rB) {
+  constexpr int N = four_step_n(M2, kRowLo);
+#pragma unroll
+  for (int i = threadIdx.x; i < 2 * N; i += T)
+    s4[i] = __ldg(g.tw_r4 + (int64_t)(i < N ? rA : rB) * N + (i < N ? i : i - N));
+}
+
+template <int M2, bool kStream = false>
 struct DstRows {
   float2* y;
-  const Group* g;
+  const float2* s4;    // load_row_twiddles
   int rA, rB;
   bool self;
   __device__ __forceinline__ void operator()(int b, int i, float2 v) const {
     if (b && self) return;
-    const int r = b ? rB : rA;
-    const float2 o = cmulc(v, tw_big(*g, r * i));
-    if constexpr (kStream) __stcs(y + (int64_t)r * g->M2 + i, o);
-    else y[(int64_t)r * g->M2 + i] = o;
+    const float2* t = s4 + b * four_step_n(M2, kRowLo);
+    float2 w = t[i & (four_step_lo(M2, kRowLo) - 1)];
+    if constexpr (M2 > kRowLo) w = cmul(t[kRowLo + i / kRowLo], w);
+    const float2 o = cmulc(v, w);
+    const int64_t at = (int64_t)(b ? rB : rA) * M2 + i;
+    if constexpr (kStream) __stcs(y + at, o);
+    else y[at] = o;
   }
 };
 
 template <int M2, int T, int MODE, bool kStream = false>
 __device__ __forceinline__ void kernel_body_job(const RowParams& q, float2* sm, const float2* tws,
-                                                float* red, int ci, int rA_) {
+                                                float* red, float2* s4, int ci, int rA_) {
   using Lay = RowLayout<M2>;
   const int c = q.chunks[ci];
   const ChunkDesc d = q.desc[c];
@@ -96,6 +109,7 @@ __device__ __forceinline__ void kernel_body_job(const RowParams& q, float2* sm, 
       s_con[0] = (float)d.tau;
       s_con[1] = mess && lam_inf ? 0.f : (float)(lambda * d.tau);
     }
+    if (inv) load_row_twiddles<M2, T>(s4, q.g, rA, rB);
     if (!fwd) __syncthreads();
   }
 
@@ -271,7 +285,7 @@ __device__ __forceinline__ void kernel_body_job(const RowParams& q, float2* sm, 
     if (lane == 0) atomicAdd(chi2, s * (double)inv_n);   // n is a power of two: 1/n is exact
   }
   if (!inv) return;
-  smem_fft<M2, 2, Lay, T, +1>(sm, tws, SmemIO{}, DstRows<kStream>{y, &q.g, rA, rB, self});
+  smem_fft<M2, 2, Lay, T, +1>(sm, tws, SmemIO{}, DstRows<M2, kStream>{y, s4, rA, rB, self});
 }
 
 // The row kernel's parameters for batch b and row mode a.
