@@ -9,6 +9,7 @@
 
 #include <algorithm>
 #include <cstddef>
+#include <functional>
 #include <map>
 #include <tuple>
 #include <mutex>
@@ -144,7 +145,7 @@ static bool gen_shape(int64_t n, int* M, int* M1, int* M2, int* cplx) {
   return true;
 }
 
-// Radix sequence of a general DFT length (any order is a valid Stockham schedule; larger
+// Radix sequence of a general DFT length for the data transform, radices up to 8 (any order is a valid Stockham schedule; larger
 // radices mean fewer passes).  order 0: radix 8 while 8 divides, then 4 or 2, then 5s, then
 // 3s; order 1: radix 4 in place of 8; order 2: the 3s and 5s first, then 8, 4, 2.
 static int radix_plan(int L, int8_t* rad, int order = 0) {
@@ -163,6 +164,44 @@ static int radix_plan(int L, int8_t* rad, int order = 0) {
   return L == 1 ? n : -1;
 }
 
+// Radix sequence of a general DFT length for the iterations: the fewest passes with radices 2, 3,
+// 4, 5, 6, 8, 9, 10, 15 and 16 (three for nearly every length up to 4096, where radices up to 8
+// take four to six), the smallest sum of radices among those.  A pass costs a trip of the tile
+// through shared memory, its barrier and index arithmetic.  order 0: large radices first; 1:
+// small ones first; 2: the odd ones first.  @WIDE@
+static int radix_plan_wide(int L, int8_t* rad, int order) {
+  static const int set[] = {16, 15, 10, 9, 8, 6, 5, 4, 3, 2};
+  struct Best { int n, sum, first; };
+  std::map<int, Best> best;
+  std::function<Best(int)> solve = [&](int x) -> Best {
+    if (x == 1) return Best{0, 0, 0};
+    auto it = best.find(x);
+    if (it != best.end()) return it->second;
+    Best b{1000, 0, 0};
+    for (int r : set) {
+      if (x % r) continue;
+      const Best t = solve(x / r);
+      if (t.n >= 1000) continue;
+      const Best c{t.n + 1, t.sum + r, r};
+      if (c.n < b.n || (c.n == b.n && c.sum < b.sum)) b = c;
+    }
+    best[x] = b;
+    return b;
+  };
+  int n = 0;
+  for (int x = L; x > 1;) {
+    const Best b = solve(x);
+    if (b.n >= 1000 || n == kMaxRadices) return -1;
+    rad[n++] = (int8_t)b.first;
+    x /= b.first;
+  }
+  auto odd_first = [](int8_t a, int8_t b) { return (a & 1) != (b & 1) ? (a & 1) > (b & 1) : a > b; };
+  if (order == 0) std::sort(rad, rad + n, [](int8_t a, int8_t b) { return a > b; });
+  else if (order == 1) std::sort(rad, rad + n);
+  else std::sort(rad, rad + n, odd_first);
+  return n;
+}
+
 static int log_lo_of(int M) {
   int p = 0;
   while ((1 << p) < M) ++p;
@@ -172,10 +211,10 @@ static int log_lo_of(int M) {
 static const int kGenLogLo = 10;
 
 static size_t tw_count(int M, int M1, int M2, bool general) {
-  // general lengths: per-pass tables of the column and row DFTs (fewer than 2 L entries for
-  // any radix plan of L), then the four-step and packing tables
+  // general lengths: per-pass tables of the column and row DFTs for the iterations' and the
+  // data's plan (fewer than 2 L entries for any radix plan of L), then the four-step and packing tables
   if (general)
-    return (size_t)2 * M1 + 2 * M2 + (size_t(1) << kGenLogLo) + (size_t)(M >> kGenLogLo) + 1 + M1 + M2;
+    return (size_t)4 * M1 + 4 * M2 + (size_t(1) << kGenLogLo) + (size_t)(M >> kGenLogLo) + 1 + M1 + M2;
   const int lo = log_lo_of(M);
   return (size_t)tw_size(M1) + tw_size(M2) + (size_t(1) << lo) + (size_t)(M >> lo) + M1 + M2 +
          (size_t)M2 * four_step_n(M1, kColLo) + (size_t)M1 * four_step_n(M2, kRowLo);
@@ -197,7 +236,7 @@ struct Layout {
   std::vector<int> chunk_group;
   std::vector<int> gen_list;            // general chunks in plan order
   std::vector<Batch> gen_batches;
-  int64_t spec_total, n_total;
+  int64_t spec_total, n_total, tile_base;
 };
 
 static size_t up(size_t x) { return (x + 255) & ~size_t(255); }
@@ -339,9 +378,14 @@ static mm_status make_layout(int n_chunks, const int64_t* off, int64_t n_pix, in
   L->scal = take(sizeof(double) * kScalCount);
   // pointing copied into column-tile order for the streaming passes
   const size_t wb = ncomp == 3 ? (wdtype == MM_W_F16 ? 2 : 4) : 0;
-  L->tpix = take(sizeof(int32_t) * (size_t)L->n_total);
-  L->tcos = take(wb * (size_t)L->n_total);
-  L->tsin = take(wb * (size_t)L->n_total);
+  // (general chunks on multiples of 4, after the compile-time ones when there are any)
+  L->tile_base = ngen < (size_t)n_chunks ? (L->n_total + 3) & ~int64_t(3) : 0;
+  int64_t tile_n = L->tile_base;
+  for (int c : L->gen_list) tile_n += (off[c + 1] - off[c] + 3) & ~int64_t(3);
+  if (ngen == 0) tile_n = L->n_total;
+  L->tpix = take(sizeof(int32_t) * (size_t)tile_n);
+  L->tcos = take(wb * (size_t)tile_n);
+  L->tsin = take(wb * (size_t)tile_n);
   // graph mode: schedule table, iteration counter + chi^2 pointer slot, FP64 map
   L->lam_cap = 65536;
   L->lam = take(sizeof(double) * L->lam_cap);
@@ -1081,8 +1125,14 @@ static cudaError_t gen_upload(mm_plan_s* p, cudaStream_t s) {
     R.yoff = yo;
     R.tw_col = G.tw_col; R.tw_row = G.tw_row; R.tw_lo = G.tw_lo; R.tw_hi = G.tw_hi;
     R.pack_a = G.tw_pack_a; R.pack_b = G.tw_pack_b;
-    R.nr1 = radix_plan(d.M1, R.rad1, p->gen_tune.radix_order);
-    R.nr2 = radix_plan(d.M2, R.rad2, p->gen_tune.radix_order);
+    R.toff = p->h_gen_toff[i];
+    R.inv_n = 1.0 / (double)d.n;
+    R.tw_col_d = G.tw_col_d; R.tw_row_d = G.tw_row_d;
+    R.nr1 = radix_plan_wide(d.M1, R.rad1, p->gen_tune.radix_order);
+    R.nr2 = radix_plan_wide(d.M2, R.rad2, p->gen_tune.radix_order);
+    R.nr1d = radix_plan(d.M1, R.rad1d, p->gen_tune.radix_order);
+    R.nr2d = radix_plan(d.M2, R.rad2d, p->gen_tune.radix_order);
+    if (R.nr1 < 0 || R.nr2 < 0 || R.nr1d < 0 || R.nr2d < 0) return cudaErrorInvalidValue;
     ct_n += tiles;
     rj += jobs;
     yo += d.M;
@@ -1095,15 +1145,18 @@ static cudaError_t gen_upload(mm_plan_s* p, cudaStream_t s) {
   for (int g = 0; g < p->n_groups; ++g) {
     const Group& G = p->groups[g];
     if (!G.general) continue;
-    for (int dim = 0; dim < 2; ++dim) {
+    for (int t = 0; t < 4; ++t) {
       PassPlan pl;
       memset(&pl, 0, sizeof(pl));
-      pl.nr = radix_plan(dim ? G.M2 : G.M1, pl.rad, p->gen_tune.radix_order);
+      const int len = t & 1 ? G.M2 : G.M1;
+      pl.nr = t < 2 ? radix_plan_wide(len, pl.rad, p->gen_tune.radix_order)
+                    : radix_plan(len, pl.rad, p->gen_tune.radix_order);
       if (pl.nr < 0) return cudaErrorInvalidValue;
       const int cnt = plan_twiddle_count(pl);
-      if (cnt > 2 * (dim ? G.M2 : G.M1)) return cudaErrorInvalidValue;
+      if (cnt > 2 * len) return cudaErrorInvalidValue;
+      float2* out[4] = {G.tw_col, G.tw_row, G.tw_col_d, G.tw_row_d};
       if (cnt > 0)   // a length-1 DFT has no pass
-        k_plan_twiddles<<<blocks_for(cnt, 256), 256, 0, s>>>(dim ? G.tw_row : G.tw_col, pl);
+        k_plan_twiddles<<<blocks_for(cnt, 256), 256, 0, s>>>(out[t], pl);
     }
   }
   cudaError_t ek = cudaGetLastError();
@@ -1137,6 +1190,7 @@ static cudaError_t small_upload(mm_plan_s* p, cudaStream_t s) {
     R.tw_col = G.tw_col; R.tw_row = G.tw_row; R.tw_lo = G.tw_lo; R.tw_hi = G.tw_hi;
     R.pack_a = G.tw_pack_a; R.pack_b = G.tw_pack_b;
     if (G.general) {
+      R.tw_col = G.tw_col_d; R.tw_row = G.tw_row_d;
       R.nr1 = radix_plan(G.M1, R.rad1, p->gen_tune.radix_order);
       R.nr2 = radix_plan(G.M2, R.rad2, p->gen_tune.radix_order);
     } else {
@@ -1285,7 +1339,7 @@ static mm_status plan_create(mm_plan* out, int n_chunks, const int64_t* offsets,
   p->gen_ctab = reinterpret_cast<int2*>(ws + L.gen_ctab);
   p->gen_rtab = reinterpret_cast<int4*>(ws + L.gen_rtab);
   p->gen_ccap = L.gen_ccap;
-  p->h_gen_ctile = p->h_gen_rjob = p->h_gen_yoff = nullptr;
+  p->h_gen_ctile = p->h_gen_rjob = p->h_gen_yoff = p->h_gen_toff = nullptr;
   p->h_gen_chunks = nullptr;
   p->gen_tune = GenTune{8, 256, 256, 0};
 
@@ -1320,11 +1374,6 @@ static mm_status plan_create(mm_plan* out, int n_chunks, const int64_t* offsets,
     G.general = L.ggen[g];
     G.cplx = L.gcplx[g];
     G.log_lo = G.general ? kGenLogLo : log_lo_of(G.M);
-    G.nr1 = G.nr2 = 0;
-    if (G.general) {
-      G.nr1 = radix_plan(G.M1, G.rad1);
-      G.nr2 = radix_plan(G.M2, G.rad2);
-    }
     G.chunks = d_chunks + order.size();
     G.n_chunks = 0;
     G.batch = L.gbatch[g];
@@ -1333,6 +1382,11 @@ static mm_status plan_create(mm_plan* out, int n_chunks, const int64_t* offsets,
     float2* t = p->tw_pool + tw_off;
     G.tw_col = t; t += G.general ? 2 * G.M1 : tw_size(G.M1);
     G.tw_row = t; t += G.general ? 2 * G.M2 : tw_size(G.M2);
+    G.tw_col_d = G.tw_row_d = nullptr;
+    if (G.general) {
+      G.tw_col_d = t; t += 2 * G.M1;
+      G.tw_row_d = t; t += 2 * G.M2;
+    }
     G.tw_lo = t; t += (1 << G.log_lo);
     G.tw_hi = t; t += (G.M >> G.log_lo) + (G.general ? 1 : 0);
     G.tw_c4 = G.tw_r4 = nullptr;
@@ -1381,11 +1435,17 @@ static mm_status plan_create(mm_plan* out, int n_chunks, const int64_t* offsets,
   if (p->n_gen > 0) {
     const int ng = p->n_gen;
     p->h_gen_chunks = new (std::nothrow) int[ng];
-    p->h_gen_ctile = new (std::nothrow) int64_t[3 * (ng + 1)];
+    p->h_gen_ctile = new (std::nothrow) int64_t[4 * (ng + 1)];
     if (!p->h_gen_chunks || !p->h_gen_ctile) { mm_plan_destroy(p); mm_set_error("host allocation failed"); return MM_ERR_NOMEM; }
     p->h_gen_rjob = p->h_gen_ctile + (ng + 1);
     p->h_gen_yoff = p->h_gen_rjob + (ng + 1);
-    for (int i = 0; i < ng; ++i) p->h_gen_chunks[i] = L.gen_list[i];
+    p->h_gen_toff = p->h_gen_yoff + (ng + 1);
+    int64_t to = L.tile_base;
+    for (int i = 0; i < ng; ++i) {
+      p->h_gen_chunks[i] = L.gen_list[i];
+      p->h_gen_toff[i] = to;
+      to += (p->h_desc[L.gen_list[i]].n + 3) & ~3;
+    }
   }
   cudaStream_t s = S(stream);
   auto fail = [&](const char* what, cudaError_t e) {

@@ -99,19 +99,14 @@ __device__ __forceinline__ void emit_run(double* acc, int64_t stride, int p, flo
 // X_u = the lane's leading run when it continues the previous lane's trailing run, G_u = the
 // lane is one such run and the next lane continues it).  Each run's first sample's lane
 // issues one FP64 add per component.
-template <int NC, int ROWL = 8>
-__device__ __forceinline__ void scatter4(const ColParams& q, int64_t s, float4 t4, int qpos) {
+template <int NC, int ROWL>
+__device__ __forceinline__ void bin4(double* acc, int64_t acc_stride, int4 p4, float4 t4, float4 c, float4 w,
+                                     int qpos) {
   static_assert(ROWL == 2 || ROWL == 4 || ROWL == 8, "rows of 2, 4 or 8 lanes");
   const uint64_t pol = l2_policy_evict_last();
-  const int4 p4 = __ldcs(reinterpret_cast<const int4*>(q.pix + s));
   const int p[4] = {p4.x, p4.y, p4.z, p4.w};
   const float tv[4] = {t4.x, t4.y, t4.z, t4.w};
   float v[3][4];
-  float4 c = make_float4(0.f, 0.f, 0.f, 0.f), w = c;
-  if constexpr (NC == 3) {
-    c = load_w4(q.cosw, q.half_w, s);
-    w = load_w4(q.sinw, q.half_w, s);
-  }
   const float cw[4] = {c.x, c.y, c.z, c.w}, sw[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -133,8 +128,8 @@ __device__ __forceinline__ void scatter4(const ColParams& q, int64_t s, float4 t
       h[1][k] = v[k][2] + v[k][3];
       if (!b2) h[0][k] += h[1][k];
     }
-    emit_run<NC>(q.acc, q.acc_stride, p[0], h[0][0], h[0][1], h[0][2], pol);
-    if (b2) emit_run<NC>(q.acc, q.acc_stride, p[2], h[1][0], h[1][1], h[1][2], pol);
+    emit_run<NC>(acc, acc_stride, p[0], h[0][0], h[0][1], h[0][2], pol);
+    if (b2) emit_run<NC>(acc, acc_stride, p[2], h[1][0], h[1][1], h[1][2], pol);
     return;
   }
   const bool single = !(b1 || b2 || b3);
@@ -174,14 +169,25 @@ __device__ __forceinline__ void scatter4(const ColParams& q, int64_t s, float4 t
     carry[k] = qpos != ROWL - 1 ? cd : 0.f;
   }
   if (!(single && cont))
-    emit_run<NC>(q.acc, q.acc_stride, p[3], trail[0] + carry[0], trail[1] + carry[1], trail[2] + carry[2], pol);
-  if (!cont && !single) emit_run<NC>(q.acc, q.acc_stride, p[0], lead[0], lead[1], lead[2], pol);
+    emit_run<NC>(acc, acc_stride, p[3], trail[0] + carry[0], trail[1] + carry[1], trail[2] + carry[2], pol);
+  if (!cont && !single) emit_run<NC>(acc, acc_stride, p[0], lead[0], lead[1], lead[2], pol);
   if (b1 && l > 1) {   // middle run [1, e)
     const bool two = b2;
-    emit_run<NC>(q.acc, q.acc_stride, p[1], two ? v[0][1] : v[0][1] + v[0][2], two ? v[1][1] : v[1][1] + v[1][2],
+    emit_run<NC>(acc, acc_stride, p[1], two ? v[0][1] : v[0][1] + v[0][2], two ? v[1][1] : v[1][1] + v[1][2],
                  two ? v[2][1] : v[2][1] + v[2][2], pol);
   }
-  if (b2 && l > 2) emit_run<NC>(q.acc, q.acc_stride, p[2], v[0][2], v[1][2], v[2][2], pol);
+  if (b2 && l > 2) emit_run<NC>(acc, acc_stride, p[2], v[0][2], v[1][2], v[2][2], pol);
+}
+
+template <int NC, int ROWL = 8>
+__device__ __forceinline__ void scatter4(const ColParams& q, int64_t s, float4 t4, int qpos) {
+  const int4 p4 = __ldcs(reinterpret_cast<const int4*>(q.pix + s));
+  float4 c = make_float4(0.f, 0.f, 0.f, 0.f), w = c;
+  if constexpr (NC == 3) {
+    c = load_w4(q.cosw, q.half_w, s);
+    w = load_w4(q.sinw, q.half_w, s);
+  }
+  bin4<NC, ROWL>(q.acc, q.acc_stride, p4, t4, c, w, qpos);
 }
 
 // First-pass sources and last-pass sink of the column DFTs.  Element (b, i) of a tile is

@@ -46,6 +46,7 @@ struct GenParams {
   const float* __restrict__ nbar;
   const float* __restrict__ nyq;
   RowArgs a;
+  unsigned* queue;      // [2] row jobs handed out, finished CTAs (zero between launches)
   // composite pointing (App. B): P = ga P_1 + gb P_2, the second component below
   int composite;
   float ga, gb;
@@ -54,12 +55,14 @@ struct GenParams {
   const void* sin2;
 };
 
-// k mod d for 0 <= k < 2^22 with d uniform: float reciprocal, then one correction step
+// k mod d for 0 <= k < 2^22 with d uniform: approximate reciprocal, then one correction step
 // each way (the float quotient is within one of the true one).
 struct FastDiv {
   int d;
   float inv;
-  __device__ __forceinline__ explicit FastDiv(int dd) : d(dd), inv(1.0f / (float)dd) {}
+  __device__ __forceinline__ explicit FastDiv(int dd) : d(dd) {
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"((float)dd));
+  }
   __device__ __forceinline__ int mod(int k) const {
     const int q = __float2int_rz((float)k * inv);
     int r = k - q * d;
@@ -76,19 +79,42 @@ struct FastDiv {
   }
 };
 
-// Row tiles hold nseq sequences of length L (sequence s at s L) in one of two layouts:
-// plain, or padded with one spare slot per 16 elements.  Each pass writes the layout that
-// suits it (padded after an even radix, whose stride-R stores would otherwise hit the same
-// banks), and the next pass reads that layout.
-__device__ __forceinline__ int lay(int e, bool pad) { return pad ? e + (e >> 4) : e; }
+// Row tiles: one spare slot after every 16 elements, so that the stride-R stores of the early
+// passes spread over the banks.
+__device__ __forceinline__ int lay(int e) { return e + (e >> 4); }
+
+__device__ __forceinline__ float2 gen_tw_big(const GenChunk& g, int e) {
+  return cmul(__ldg(&g.tw_hi[e >> g.log_lo]), __ldg(&g.tw_lo[e & ((1 << g.log_lo) - 1)]));
+}
 
 // ----------------------------------------------------------------- Stockham passes
+// Where a pass reads and writes: the shared-memory tile, or (first pass of the rows and of the
+// inverse columns, last pass of the inverse rows and of the columns) the intermediate itself,
+// with the four-step twiddle on the way out.  That saves a tile's trip through shared memory
+// and a barrier at either end.
+enum { kSmem = 0, kGlobal = 1 };
+
+struct ColIO {      // columns j2_0 .. j2_0 + width - 1 of one chunk
+  float2* y;
+  const GenChunk* g;
+  int M2, j2_0, width;
+};
+struct RowIO {      // the rows of one job: sequence sq holds row(sq)
+  float2* y;
+  const GenChunk* g;
+  int M1, M2, first;
+  bool self;
+  __device__ __forceinline__ int row(int sq) const {
+    return self ? first : ((sq & 1) ? M1 - first - (sq >> 1) : first + (sq >> 1));
+  }
+};
+
 // Column tiles: element (j, c) of the tile's NB interleaved sequences at j * NB + c.  A
 // thread keeps its column c and walks butterflies i = i0, i0 + T/NB, ...; k = i mod Ns is
 // advanced by the same step instead of being recomputed.
-template <int R, int DIR>
+template <int R, int DIR, int SRC, int DST>
 __device__ __forceinline__ void gpass_cols(const float2* src, float2* dst, int L, int Ns, int NB,
-                                           int lnb, const float2* __restrict__ tw, int T) {
+                                           int lnb, const float2* __restrict__ tw, int T, const ColIO& io) {
   const int nb = L / R;
   const int c = threadIdx.x & (NB - 1);
   const int di = T >> lnb;
@@ -100,7 +126,10 @@ __device__ __forceinline__ void gpass_cols(const float2* src, float2* dst, int L
   for (; i < nb; i += di) {
     float2 v[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = src[(i + r * nb) * NB + c];
+    for (int r = 0; r < R; ++r) {
+      if constexpr (SRC == kSmem) v[r] = src[(i + r * nb) * NB + c];
+      else v[r] = c < io.width ? io.y[(int64_t)(i + r * nb) * io.M2 + io.j2_0 + c] : make_float2(0.f, 0.f);
+    }
     if (Ns > 1) {
 #pragma unroll
       for (int r = 1; r < R; ++r) {
@@ -111,18 +140,25 @@ __device__ __forceinline__ void gpass_cols(const float2* src, float2* dst, int L
     dftR<R, DIR>(v);
     const int o = (i - k) * R + k;
 #pragma unroll
-    for (int r = 0; r < R; ++r) dst[(o + r * Ns) * NB + c] = v[r];
+    for (int r = 0; r < R; ++r) {
+      if constexpr (DST == kSmem) {
+        dst[(o + r * Ns) * NB + c] = v[r];
+      } else if (c < io.width) {
+        const int k1 = o + r * Ns, j2 = io.j2_0 + c;
+        io.y[(int64_t)k1 * io.M2 + j2] = cmul(v[r], gen_tw_big(*io.g, k1 * j2));
+      }
+    }
     k += dk;
     if (k >= Ns) k -= Ns;
   }
 }
 
-// Row jobs: nseq contiguous sequences of length L; PS / PD: the source / destination tile is
-// in the padded layout.  Butterfly b = sq nb + i advances by T per step as (sq, i, k) with
-// carries (nb is a multiple of Ns, so wrapping i keeps k = i mod Ns).
-template <int R, int DIR, bool PS, bool PD>
+// Row jobs: nseq sequences of length L, element i of sequence sq at lay(sq L + i).  Butterfly
+// b = sq nb + i advances by T per step as (sq, i, k) with carries (nb is a multiple of Ns, so
+// wrapping i keeps k = i mod Ns).
+template <int R, int DIR, int SRC, int DST>
 __device__ __forceinline__ void gpass_rows(const float2* src, float2* dst, int L, int Ns, int nseq,
-                                           const float2* __restrict__ tw, int T) {
+                                           const float2* __restrict__ tw, int T, const RowIO& io) {
   const int nb = L / R;
   const int total = nb * nseq;
   int b = threadIdx.x;
@@ -134,9 +170,13 @@ __device__ __forceinline__ void gpass_rows(const float2* src, float2* dst, int L
   const int dsq = fs.div(T), di = T - dsq * nb, dk = fd.mod(di);
   for (; b < total; b += T) {
     const int base = sq * L;
+    const int row = SRC == kGlobal || DST == kGlobal ? io.row(sq) : 0;
     float2 v[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = src[lay(base + i + r * nb, PS)];
+    for (int r = 0; r < R; ++r) {
+      if constexpr (SRC == kSmem) v[r] = src[lay(base + i + r * nb)];
+      else v[r] = io.y[(int64_t)row * io.M2 + i + r * nb];
+    }
     if (Ns > 1) {
 #pragma unroll
       for (int r = 1; r < R; ++r) {
@@ -145,9 +185,16 @@ __device__ __forceinline__ void gpass_rows(const float2* src, float2* dst, int L
       }
     }
     dftR<R, DIR>(v);
-    const int o = base + (i - k) * R + k;
+    const int o = (i - k) * R + k;
 #pragma unroll
-    for (int r = 0; r < R; ++r) dst[lay(o + r * Ns, PD)] = v[r];
+    for (int r = 0; r < R; ++r) {
+      if constexpr (DST == kSmem) {
+        dst[lay(base + o + r * Ns)] = v[r];
+      } else {
+        const int p = o + r * Ns;
+        io.y[(int64_t)row * io.M2 + p] = cmulc(v[r], gen_tw_big(*io.g, row * p));
+      }
+    }
     i += di;
     sq += dsq;
     k += dk;
@@ -156,53 +203,88 @@ __device__ __forceinline__ void gpass_rows(const float2* src, float2* dst, int L
   }
 }
 
-// All passes of the row DFTs of a job, starting from layout `pad` in tile a; returns the
-// tile holding the result and sets `pad` to its layout (padded after an even radix).
-template <int DIR>
-__device__ float2* gen_dft_rows(float2* a, float2* b, bool& pad, int L, int nr, const int8_t* rad,
-                                const float2* tw, int nseq, int T) {
+#define GEN_RADICES(X) X(2) X(3) X(4) X(5) X(6) X(8) X(9) X(10) X(15) X(16)
+
+// All passes of the row DFTs of a job.  kFirst: the first pass reads the intermediate (nothing
+// is in the tiles), otherwise tile a holds the input; kLast: the last pass writes the
+// intermediate.  Returns the tile that holds the result (kLast smem).
+template <int DIR, int kFirst, int kLast>
+__device__ float2* gen_dft_rows(float2* a, float2* b, int L, int nr, const int8_t* rad, const float2* tw,
+                                int nseq, int T, const RowIO& io) {
   int Ns = 1;
+  if (nr == 0) {      // L = 1
+    for (int sq = threadIdx.x; sq < nseq; sq += T) {
+      if (kFirst == kGlobal) a[lay(sq)] = io.y[(int64_t)io.row(sq) * io.M2];
+      if (kLast == kGlobal) io.y[(int64_t)io.row(sq) * io.M2] = a[lay(sq)];   // w_M^0
+    }
+    __syncthreads();
+    return a;
+  }
   for (int p = 0; p < nr; ++p) {
     const int R = rad[p];
-    if (pad) {
+    const bool g_in = kFirst == kGlobal && p == 0, g_out = kLast == kGlobal && p == nr - 1;
+    if (g_in) {      // into b: the swap below makes it the next source
       switch (R) {
-        case 2: gpass_rows<2, DIR, true, true>(a, b, L, Ns, nseq, tw, T); break;
-        case 3: gpass_rows<3, DIR, true, false>(a, b, L, Ns, nseq, tw, T); break;
-        case 4: gpass_rows<4, DIR, true, true>(a, b, L, Ns, nseq, tw, T); break;
-        case 5: gpass_rows<5, DIR, true, false>(a, b, L, Ns, nseq, tw, T); break;
-        default: gpass_rows<8, DIR, true, true>(a, b, L, Ns, nseq, tw, T); break;
+#define X(r) case r: gpass_rows<r, DIR, kGlobal, kSmem>(a, b, L, Ns, nseq, tw, T, io); break;
+        GEN_RADICES(X)
+#undef X
+      }
+    } else if (g_out) {
+      switch (R) {
+#define X(r) case r: gpass_rows<r, DIR, kSmem, kGlobal>(a, b, L, Ns, nseq, tw, T, io); break;
+        GEN_RADICES(X)
+#undef X
       }
     } else {
       switch (R) {
-        case 2: gpass_rows<2, DIR, false, true>(a, b, L, Ns, nseq, tw, T); break;
-        case 3: gpass_rows<3, DIR, false, false>(a, b, L, Ns, nseq, tw, T); break;
-        case 4: gpass_rows<4, DIR, false, true>(a, b, L, Ns, nseq, tw, T); break;
-        case 5: gpass_rows<5, DIR, false, false>(a, b, L, Ns, nseq, tw, T); break;
-        default: gpass_rows<8, DIR, false, true>(a, b, L, Ns, nseq, tw, T); break;
+#define X(r) case r: gpass_rows<r, DIR, kSmem, kSmem>(a, b, L, Ns, nseq, tw, T, io); break;
+        GEN_RADICES(X)
+#undef X
       }
     }
     __syncthreads();
     float2* t = a; a = b; b = t;
-    pad = (R & 1) == 0;
     tw += Ns * R;   // the next pass's table
     Ns *= R;
   }
   return a;
 }
 
-// All passes of the column DFTs of a tile; returns the tile holding the result (a or b).
-template <int DIR>
-__device__ float2* gen_dft_cols(float2* a, float2* b, int L, int nr, const int8_t* rad,
-                                const float2* tw, int NB, int lnb, int T) {
+// All passes of the column DFTs of a tile, ends as above.
+template <int DIR, int kFirst, int kLast>
+__device__ float2* gen_dft_cols(float2* a, float2* b, int L, int nr, const int8_t* rad, const float2* tw,
+                                int NB, int lnb, int T, const ColIO& io) {
   int Ns = 1;
+  if (nr == 0) {      // L = 1
+    const int c = threadIdx.x;
+    if (c < NB) {
+      if (kFirst == kGlobal) a[c] = c < io.width ? io.y[io.j2_0 + c] : make_float2(0.f, 0.f);
+      if (kLast == kGlobal && c < io.width) io.y[io.j2_0 + c] = a[c];   // w_M^0
+    }
+    __syncthreads();
+    return a;
+  }
   for (int p = 0; p < nr; ++p) {
     const int R = rad[p];
-    switch (R) {
-      case 2: gpass_cols<2, DIR>(a, b, L, Ns, NB, lnb, tw, T); break;
-      case 3: gpass_cols<3, DIR>(a, b, L, Ns, NB, lnb, tw, T); break;
-      case 4: gpass_cols<4, DIR>(a, b, L, Ns, NB, lnb, tw, T); break;
-      case 5: gpass_cols<5, DIR>(a, b, L, Ns, NB, lnb, tw, T); break;
-      default: gpass_cols<8, DIR>(a, b, L, Ns, NB, lnb, tw, T); break;
+    const bool g_in = kFirst == kGlobal && p == 0, g_out = kLast == kGlobal && p == nr - 1;
+    if (g_in) {
+      switch (R) {
+#define X(r) case r: gpass_cols<r, DIR, kGlobal, kSmem>(a, b, L, Ns, NB, lnb, tw, T, io); break;
+        GEN_RADICES(X)
+#undef X
+      }
+    } else if (g_out) {
+      switch (R) {
+#define X(r) case r: gpass_cols<r, DIR, kSmem, kGlobal>(a, b, L, Ns, NB, lnb, tw, T, io); break;
+        GEN_RADICES(X)
+#undef X
+      }
+    } else {
+      switch (R) {
+#define X(r) case r: gpass_cols<r, DIR, kSmem, kSmem>(a, b, L, Ns, NB, lnb, tw, T, io); break;
+        GEN_RADICES(X)
+#undef X
+      }
     }
     __syncthreads();
     float2* t = a; a = b; b = t;
@@ -210,10 +292,6 @@ __device__ float2* gen_dft_cols(float2* a, float2* b, int L, int nr, const int8_
     Ns *= R;
   }
   return a;
-}
-
-__device__ __forceinline__ float2 gen_tw_big(const GenChunk& g, int e) {
-  return cmul(__ldg(&g.tw_hi[e >> g.log_lo]), __ldg(&g.tw_lo[e & ((1 << g.log_lo) - 1)]));
 }
 
 // One pointing component's (P m)_s (Eq. 1); weights from the caller's natural-order arrays.
@@ -248,36 +326,51 @@ __device__ __forceinline__ float gen_pm(const GenParams& q, int64_t s) {
 
 // (P m) of a tile of one pointing component into tile a (element e = j1 NB + c holds samples
 // 2 (j1 M2 + j2_0 + c) + {0, 1}, or the one sample j1 M2 + j2_0 + c of an odd-length chunk).
-// U elements per thread are in flight at once: their pointing loads first, then the map
-// loads that depend on them (one element at a time leaves both round trips exposed).
+// U elements per thread are in flight at once: their pointing loads first (both samples of an
+// element by one load: the tile-order arrays start on multiples of 4), then the map loads that
+// depend on them.
 template <int NC>
-__device__ __forceinline__ void gen_gather_tile(const GenParams& q, const ChunkDesc& d, int j2_0,
+__device__ __forceinline__ void gen_gather_tile(const GenParams& q, const GenChunk& G, int j2_0,
                                                 int width, float2* a, int NB, int lnb, int T) {
   constexpr int U = 4;
-  const int n = d.M1 * NB;
-  const int nh = d.cplx ? 1 : 2;
-  const int64_t tb = d.off + (int64_t)d.M1 * j2_0 * nh;   // the tile's first sample
+  const bool cplx = G.d.cplx != 0;
+  const int n = G.d.M1 * NB;
+  const int64_t tb = G.toff + (int64_t)G.d.M1 * j2_0 * (cplx ? 1 : 2);   // the tile's first sample
+  ColParams cq{};
+  cq.map4 = q.map4;
   for (int e0 = threadIdx.x; e0 < n; e0 += U * T) {
-    int pi[U][2];
-    float cw[U][2], sw[U][2];
+    int2 pi[U];
+    float2 cw[U], sw[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int e = e0 + u * T;
       const int j1 = e >> lnb, c = e & (NB - 1);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        pi[u][h] = -1;
-        cw[u][h] = sw[u][h] = 0.f;
-        if (e < n && c < width && h < nh) {
-          const int64_t s = tb + ((int64_t)j1 * width + c) * nh + h;
-          pi[u][h] = __ldg(q.tpix + s);
+      pi[u] = make_int2(-1, -1);
+      cw[u] = sw[u] = make_float2(0.f, 0.f);
+      if (e < n && c < width) {
+        const int64_t el = (int64_t)j1 * width + c;
+        if (cplx) {
+          const int64_t s = tb + el;
+          pi[u].x = __ldg(q.tpix + s);
           if constexpr (NC == 3) {
             if (q.half_w) {
-              cw[u][h] = __half2float(static_cast<const __half*>(q.tcos)[s]);
-              sw[u][h] = __half2float(static_cast<const __half*>(q.tsin)[s]);
+              cw[u].x = __half2float(static_cast<const __half*>(q.tcos)[s]);
+              sw[u].x = __half2float(static_cast<const __half*>(q.tsin)[s]);
             } else {
-              cw[u][h] = __ldg(static_cast<const float*>(q.tcos) + s);
-              sw[u][h] = __ldg(static_cast<const float*>(q.tsin) + s);
+              cw[u].x = __ldg(static_cast<const float*>(q.tcos) + s);
+              sw[u].x = __ldg(static_cast<const float*>(q.tsin) + s);
+            }
+          }
+        } else {
+          const int64_t s = tb + 2 * el;
+          pi[u] = __ldcs(reinterpret_cast<const int2*>(q.tpix + s));
+          if constexpr (NC == 3) {
+            if (q.half_w) {
+              cw[u] = __half22float2(__ldcs(reinterpret_cast<const __half2*>(static_cast<const __half*>(q.tcos) + s)));
+              sw[u] = __half22float2(__ldcs(reinterpret_cast<const __half2*>(static_cast<const __half*>(q.tsin) + s)));
+            } else {
+              cw[u] = __ldcs(reinterpret_cast<const float2*>(static_cast<const float*>(q.tcos) + s));
+              sw[u] = __ldcs(reinterpret_cast<const float2*>(static_cast<const float*>(q.tsin) + s));
             }
           }
         }
@@ -286,28 +379,15 @@ __device__ __forceinline__ void gen_gather_tile(const GenParams& q, const ChunkD
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int e = e0 + u * T;
-      if (e >= n) continue;
-      float z[2];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int pp = pi[u][h];
-        if (pp < 0) {
-          z[h] = 0.f;
-        } else if constexpr (NC == 1) {
-          z[h] = __ldg(reinterpret_cast<const float*>(q.map4) + pp);
-        } else {
-          const float4 m = __ldg(reinterpret_cast<const float4*>(q.map4) + pp);
-          z[h] = fmaf(sw[u][h], m.z, fmaf(cw[u][h], m.y, m.x));
-        }
-      }
-      a[e] = make_float2(z[0], z[1]);   // odd-length chunk: z[1] = 0 (imaginary part)
+      // odd-length chunk: the imaginary part stays 0 (its pixel is -1)
+      if (e < n) a[e] = gather_two<NC>(cq, pi[u].x, pi[u].y, cw[u].x, cw[u].y, sw[u].x, sw[u].y);
     }
   }
 }
 
 // ------------------------------------------------------------ kernel A: columns forward
 template <int NC, int SRC>
-__global__ void __launch_bounds__(512) k_gen_col_forward(GenParams q) {
+__global__ void __launch_bounds__(512, 2) k_gen_col_forward(GenParams q) {
   extern __shared__ float2 gsm[];
   const int T = blockDim.x, NB = q.nb, lnb = NB == 16 ? 4 : 3;
   for (int64_t t = blockIdx.x; t < q.n_items; t += gridDim.x) {
@@ -320,7 +400,7 @@ __global__ void __launch_bounds__(512) k_gen_col_forward(GenParams q) {
     float2* a = gsm;
     float2* b = gsm + M1 * NB;
     if (SRC == kSrcGather && !q.composite) {
-      gen_gather_tile<NC>(q, d, j2_0, width, a, NB, lnb, T);
+      gen_gather_tile<NC>(q, G, j2_0, width, a, NB, lnb, T);
     } else for (int e = threadIdx.x; e < M1 * NB; e += T) {
       const int j1 = e >> lnb, c = e & (NB - 1);
       float2 z = make_float2(0.f, 0.f);
@@ -337,16 +417,11 @@ __global__ void __launch_bounds__(512) k_gen_col_forward(GenParams q) {
       a[e] = z;
     }
     __syncthreads();
-    const float2* r = gen_dft_cols<-1>(a, b, M1, G.nr1, G.rad1, G.tw_col, NB, lnb, T);
-    float2* y = q.ybuf + (G.yoff - q.base_y);
-    for (int e = threadIdx.x; e < M1 * NB; e += T) {
-      const int k1 = e >> lnb, c = e & (NB - 1);
-      if (c < width) {
-        const int j2 = j2_0 + c;
-        y[(int64_t)k1 * M2 + j2] = cmul(r[e], gen_tw_big(G, k1 * j2));
-      }
-    }
-    __syncthreads();
+    const ColIO io{q.ybuf + (G.yoff - q.base_y), &G, M2, j2_0, width};
+    if constexpr (SRC == kSrcTod)   // the data keep their own plan (see radix_plan)
+      gen_dft_cols<-1, kSmem, kGlobal>(a, b, M1, G.nr1d, G.rad1d, G.tw_col_d, NB, lnb, T, io);
+    else
+      gen_dft_cols<-1, kSmem, kGlobal>(a, b, M1, G.nr1, G.rad1, G.tw_col, NB, lnb, T, io);
   }
 }
 
@@ -355,14 +430,13 @@ __global__ void __launch_bounds__(512) k_gen_col_forward(GenParams q) {
 // sample order); runs of lanes on the same pixel are summed by a segmented suffix scan and
 // the first lane of each run issues one FP64 add per component.
 template <int NC>
-__device__ __forceinline__ void gen_scatter(const GenParams& q, const ChunkDesc& d, int j2_0,
+__device__ __forceinline__ void gen_scatter(const GenParams& q, const ChunkDesc& d, int64_t tb, int j2_0,
                                             int width, const float* smf, int NB, int lnb, int T,
                                             const int32_t* __restrict__ pix, const void* cosw,
                                             const void* sinw, float gain, bool tiled) {
   const int rw = d.cplx ? NB : 2 * NB;          // samples per tile row
   const int lrw = d.cplx ? lnb : lnb + 1;
   const int valid_u = d.cplx ? width : 2 * width;
-  const int64_t tb = d.off + (int64_t)d.M1 * j2_0 * (d.cplx ? 1 : 2);   // tile order
   const int total = d.M1 * rw;
   const int lane = threadIdx.x & 31;
   // two rounds of 32 samples per warp: both rounds' pointing loads are issued before the
@@ -422,8 +496,43 @@ __device__ __forceinline__ void gen_scatter(const GenParams& q, const ChunkDesc&
   }
 }
 
+// A full tile of an even-length chunk: four consecutive samples a lane with vector loads, rows of
+// ROWL lanes (bin4), half the shuffles of one sample a lane.
+template <int NC, int ROWL>
+__device__ __forceinline__ void gen_scatter_full(const GenParams& q, const GenChunk& G, int j2_0, const float* smf,
+                                                 int T) {
+  const int total = G.d.M1 * ROWL;                       // lanes of four samples
+  const int64_t tb = G.toff + 2 * (int64_t)G.d.M1 * j2_0;
+  const int lane = threadIdx.x & 31;
+  constexpr int U = 2;   // two rounds' pointing loads in flight
+  for (int l0 = threadIdx.x - lane; l0 < total; l0 += U * T) {
+    int4 p[U];
+    float4 c[U], w[U];
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const int l = l0 + k * T + lane;
+      p[k] = make_int4(-1, -1, -1, -1);
+      c[k] = w[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (l < total) {
+        p[k] = __ldcs(reinterpret_cast<const int4*>(q.tpix + tb) + l);
+        if constexpr (NC == 3) {
+          c[k] = load_w4(q.tcos, q.half_w, tb + 4 * l);
+          w[k] = load_w4(q.tsin, q.half_w, tb + 4 * l);
+        }
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      if (l0 + k * T >= total) break;   // warp-uniform
+      const int l = l0 + k * T + lane;
+      const float4 t = l < total ? reinterpret_cast<const float4*>(smf)[l] : make_float4(0.f, 0.f, 0.f, 0.f);
+      bin4<NC, ROWL>(q.acc, q.acc_stride, p[k], t, c[k], w[k], lane & (ROWL - 1));
+    }
+  }
+}
+
 template <int NC>
-__global__ void __launch_bounds__(512) k_gen_col_inverse(GenParams q) {
+__global__ void __launch_bounds__(512, 2) k_gen_col_inverse(GenParams q) {
   extern __shared__ float2 gsm[];
   const int T = blockDim.x, NB = q.nb, lnb = NB == 16 ? 4 : 3;
   for (int64_t t = blockIdx.x; t < q.n_items; t += gridDim.x) {
@@ -435,19 +544,20 @@ __global__ void __launch_bounds__(512) k_gen_col_inverse(GenParams q) {
     const int width = min(NB, M2 - j2_0);
     float2* a = gsm;
     float2* b = gsm + M1 * NB;
-    const float2* y = q.ybuf + (G.yoff - q.base_y);
-    for (int e = threadIdx.x; e < M1 * NB; e += T) {
-      const int k1 = e >> lnb, c = e & (NB - 1);
-      a[e] = c < width ? y[(int64_t)k1 * M2 + j2_0 + c] : make_float2(0.f, 0.f);
-    }
-    __syncthreads();
-    const float2* r = gen_dft_cols<+1>(a, b, M1, G.nr1, G.rad1, G.tw_col, NB, lnb, T);
+    const ColIO io{q.ybuf + (G.yoff - q.base_y), &G, M2, j2_0, width};
+    const float2* r = gen_dft_cols<+1, kGlobal, kSmem>(a, b, M1, G.nr1, G.rad1, G.tw_col, NB, lnb, T, io);
     const float* rf = reinterpret_cast<const float*>(r);
     if (!q.composite) {
-      gen_scatter<NC>(q, d, j2_0, width, rf, NB, lnb, T, q.tpix, q.tcos, q.tsin, 1.f, true);
+      if (width == NB && !d.cplx) {
+        if (NB == 16) gen_scatter_full<NC, 8>(q, G, j2_0, rf, T);
+        else gen_scatter_full<NC, 4>(q, G, j2_0, rf, T);
+      } else {
+        gen_scatter<NC>(q, d, G.toff + (int64_t)M1 * j2_0 * (d.cplx ? 1 : 2), j2_0, width, rf, NB, lnb, T,
+                        q.tpix, q.tcos, q.tsin, 1.f, true);
+      }
     } else {   // P^T t = g_a P_a^T t + g_b P_b^T t (App. B), natural-order pointing
-      gen_scatter<NC>(q, d, j2_0, width, rf, NB, lnb, T, q.pix, q.cosw, q.sinw, q.ga, false);
-      gen_scatter<NC>(q, d, j2_0, width, rf, NB, lnb, T, q.pix2, q.cos2, q.sin2, q.gb, false);
+      gen_scatter<NC>(q, d, 0, j2_0, width, rf, NB, lnb, T, q.pix, q.cosw, q.sinw, q.ga, false);
+      gen_scatter<NC>(q, d, 0, j2_0, width, rf, NB, lnb, T, q.pix2, q.cos2, q.sin2, q.gb, false);
     }
     __syncthreads();
   }
@@ -459,10 +569,18 @@ __global__ void __launch_bounds__(512) k_gen_col_inverse(GenParams q) {
 // sequence 2j holds row first + j and sequence 2j + 1 its partner.
 // MODE >= 0: the row mode folded in at compile time (the messenger step and its map-sized
 // form); -1: read from q.a.mode (set-up, PCG, chi^2, composite and the other modes).
-template <int MODE>
-__global__ void __launch_bounds__(1024) k_gen_row(GenParams q) {
+// MAXT: 256 (three CTAs an SM, 80 registers) or 1024 threads.
+template <int MODE, int MAXT>
+__global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1) k_gen_row(GenParams q) {
   extern __shared__ float2 gsm[];
-  __shared__ double red[32];
+  __shared__ float red[32];
+  // the current job and the next one: table entry, chunk record, tau, lambda tau, output scale.
+  // Warp 0 fetches the next ones piece by piece between its passes, so that no job starts with
+  // the chain of dependent loads (6 of 37 thousand cycles a job).
+  static_assert(sizeof(GenChunk) % 4 == 0 && sizeof(GenChunk) <= 4 * 32 * 4, "at most four words a lane");
+  __shared__ GenChunk s_rec[2];
+  __shared__ int4 s_job[2];
+  __shared__ float s_con[2][3];
   const int T = blockDim.x;
   const int mode = MODE >= 0 ? MODE : q.a.mode;
   const bool fwd = mode != kRowPcgRhs && mode != kRowMd;
@@ -481,70 +599,77 @@ __global__ void __launch_bounds__(1024) k_gen_row(GenParams q) {
   const bool want_x2 = chi2 != nullptr &&
                        (mode == kRowMessenger || mode == kRowMessengerF || mode == kRowChi2 ||
                         mode == kRowPcgRhs || mode == kRowResidual);
-  for (int64_t job = blockIdx.x; job < q.n_items; job += gridDim.x) {
-    const int4 it = __ldg(q.jobs + q.base + job);
-    const GenChunk& G = q.rec[it.x];
-    const ChunkDesc d = G.d;
+  const bool lam_inf = (__double2hiint(lambda) & 0x7fffffff) == 0x7ff00000;
+  const int lane = threadIdx.x & 31;
+  constexpr int kWords = sizeof(GenChunk) / 4;
+  // warp 0: the record and constants of job `nj` into slot s
+  auto put = [&](int s, int4 nj, const int* w) {
+    s_job[s] = nj;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (lane + 32 * k < kWords) reinterpret_cast<int*>(&s_rec[s])[lane + 32 * k] = w[k];
+    __syncwarp();
+    if (lane == 0) {
+      const float tau = (float)s_rec[s].d.tau, inv_n = 1.0f / (float)s_rec[s].d.n;
+      s_con[s][0] = tau;
+      s_con[s][1] = (mess || resid) && lam_inf ? 0.f : (float)(lambda * s_rec[s].d.tau);
+      s_con[s][2] = mess ? inv_n / tau : inv_n;
+    }
+  };
+  auto fetch = [&](int4 nj, int* w) {
+    const int* src = reinterpret_cast<const int*>(q.rec + nj.x);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) w[k] = lane + 32 * k < kWords ? __ldg(src + lane + 32 * k) : 0;
+  };
+  if (threadIdx.x < 32 && blockIdx.x < q.n_items) {
+    const int4 j0 = __ldg(q.jobs + q.base + blockIdx.x);
+    int w[4];
+    fetch(j0, w);
+    put(0, j0, w);
+  }
+  __shared__ int s_more;
+  if (threadIdx.x == 0) s_more = blockIdx.x < q.n_items;
+  __syncthreads();
+  // jobs come from a counter (their sizes differ: in shares of equal count the launch waited for
+  // the longest share)
+  for (int cur = 0; s_more; cur ^= 1) {
+    const int4 it = s_job[cur];
+    const GenChunk& G = s_rec[cur];
+    int nidx = 0;
+    int4 nj = make_int4(0, 0, 0, 0);
+    if (threadIdx.x < 32) {
+      if (lane == 0) nidx = (int)gridDim.x + (int)atomicAdd(q.queue, 1u);
+    }
+    const ChunkDesc& d = G.d;
     const int c = G.c;
     const int M1 = d.M1, M2 = d.M2, M = d.M;
     const bool self = it.z == 0;
     const int first = it.y, count = self ? 1 : it.z;
     const int nseq = self ? 1 : 2 * count;
     const FastDiv fm2(M2);
-    auto row_of = [&](int sq) { return self ? first : ((sq & 1) ? M1 - first - (sq >> 1) : first + (sq >> 1)); };
     float2* y = q.ybuf + (G.yoff - q.base_y);
     float2* a = gsm;
     float2* b = gsm + q.tile;
-    bool pz = false;
     float2* z = a;
-    if (threadIdx.x == 0 && job + gridDim.x < q.n_items) {
-      // the next job's rows (and its d~ / Nbar rows) into L2 while this one runs
-      const int4 nj = __ldg(q.jobs + q.base + job + gridDim.x);
-      const GenChunk& Gn = q.rec[nj.x];
-      const int nM1 = Gn.d.M1, nM2 = Gn.d.M2;
-      const int ncount = nj.z == 0 ? 1 : nj.z;
-      const float2* yn = q.ybuf + (Gn.yoff - q.base_y);
-      for (int s = 0; s < (nj.z == 0 ? 1 : 2 * ncount); ++s) {
-        const int r = nj.z == 0 ? nj.y : ((s & 1) ? nM1 - nj.y - (s >> 1) : nj.y + (s >> 1));
-        // rows of general chunks need not start on 16 bytes: prefetch their aligned interior
-        if (fwd) prefetch_l2_inner(yn + (int64_t)r * nM2, 8 * (size_t)nM2);
-        if (load_d) prefetch_l2_inner(q.dtab + Gn.d.spec + (int64_t)r * nM2, 8 * (size_t)nM2);
-        prefetch_l2_inner(q.nbar + Gn.d.spec + (int64_t)r * nM2, 4 * (size_t)nM2);
-      }
-    }
+    const RowIO io{y, &G, M1, M2, first, self};
     if (fwd) {
-      // four elements' loads in flight per thread before their stores
-      const int ne = nseq * M2;
-      for (int e0 = threadIdx.x; e0 < ne; e0 += 4 * T) {
-        float2 v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int e = e0 + u * T;
-          if (e < ne) {
-            const int sq = fm2.div(e), p = e - sq * M2;
-            v[u] = y[(int64_t)row_of(sq) * M2 + p];
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (e0 + u * T < ne) a[e0 + u * T] = v[u];
-      }
-      __syncthreads();
-      z = gen_dft_rows<-1>(a, b, pz, M2, G.nr2, G.rad2, G.tw_row, nseq, T);
+      if (mode == kRowSpectrum || mode == kRowNatural)   // the data keep their own plan (see radix_plan)
+        z = gen_dft_rows<-1, kGlobal, kSmem>(a, b, M2, G.nr2d, G.rad2d, G.tw_row_d, nseq, T, io);
+      else
+        z = gen_dft_rows<-1, kGlobal, kSmem>(a, b, M2, G.nr2, G.rad2, G.tw_row, nseq, T, io);
     }
     float2* other = z == a ? b : a;
-
-    const float tau = (float)d.tau;
-    const float inv_n = 1.0f / (float)d.n;
-    float lt = 0.f;
-    bool lam_inf = false;
-    if (mess || resid) {
-      lam_inf = isinf(lambda);
-      lt = lam_inf ? 0.f : (float)(lambda * d.tau);
+    int nw[4];
+    bool more = false;
+    if (threadIdx.x < 32) {
+      nidx = __shfl_sync(0xffffffffu, nidx, 0);
+      more = nidx < q.n_items;
+      if (more) nj = __ldg(q.jobs + q.base + nidx);
     }
+
+    const float tau = s_con[cur][0], lt = s_con[cur][1], sc = s_con[cur][2];
     const float lamf = lam_inf ? 1.f : (float)lambda;
-    const float cn = mode == kRowChi2 ? (float)(lambda * d.tau) : tau;
-    const float sc = mess ? inv_n / tau : inv_n;
+    const float cn = mode == kRowChi2 ? lt : tau;
     const float2* dt = q.dtab + d.spec;
     const float* nb = q.nbar + d.spec;
     auto filt = [&](float2 X, float2 D, float nbv) -> float2 {
@@ -564,10 +689,10 @@ __global__ void __launch_bounds__(1024) k_gen_row(GenParams q) {
       // every frequency on its own: k = r + M1 p for element p of row r
       for (int e = threadIdx.x; e < nseq * M2; e += T) {
         const int sq = fm2.div(e), p = e - sq * M2;
-        const int r = row_of(sq);
+        const int r = io.row(sq);
         const int slot = r * M2 + p;
         const int k = r + M1 * p;
-        const int ze = lay(e, pz);
+        const int ze = lay(e);
         const float2 X = fwd ? z[ze] : make_float2(0.f, 0.f);
         if (mode == kRowSpectrum) { q.dtab[d.spec + slot] = X; continue; }
         if (mode == kRowNatural) {
@@ -586,104 +711,142 @@ __global__ void __launch_bounds__(1024) k_gen_row(GenParams q) {
       // pairs (k, M - k): element p of a row with its partner qi in the partner row (or in
       // the same row for a self-paired row)
       const int npair = self ? M2 : count * M2;
-      for (int e = threadIdx.x; e < npair; e += T) {
-        int j = 0, p = e, qi, rA, rB, sA, sB;
-        if (self) {
-          rA = rB = first;
-          sA = sB = 0;
-          qi = rA == 0 ? (p == 0 ? 0 : M2 - p) : M2 - 1 - p;
-          if (p > qi) continue;
-        } else {
-          j = fm2.div(e);
-          p = e - j * M2;
-          rA = first + j;
-          rB = M1 - rA;
-          sA = 2 * j;
-          sB = 2 * j + 1;
-          qi = M2 - 1 - p;
+      constexpr int U = 2;   // pairs whose d~ and Nbar loads a thread has in flight
+      for (int e0 = threadIdx.x; e0 < npair; e0 += U * T) {
+        float2 Dk[U], Dp[U];
+        float nk[U], np[U];
+        int pv[U], jv[U], qv[U];
+        bool act[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int e = e0 + u * T;
+          int j = 0, p = e, qi;
+          bool on = e < npair;
+          if (self) {
+            qi = first == 0 ? (p == 0 ? 0 : M2 - p) : M2 - 1 - p;
+            on = on && p <= qi;
+          } else {
+            j = fm2.div(e);
+            p = e - j * M2;
+            qi = M2 - 1 - p;
+          }
+          act[u] = on; pv[u] = p; jv[u] = j; qv[u] = qi;
+          Dk[u] = Dp[u] = make_float2(0.f, 0.f);
+          nk[u] = np[u] = 0.f;
+          if (on && mode != kRowSpectrum && mode != kRowNatural) {
+            const int sk = (first + j) * M2 + p, sp = (self ? first : M1 - first - j) * M2 + qi;
+            if (load_d) { Dk[u] = __ldcs(dt + sk); Dp[u] = __ldcs(dt + sp); }
+            nk[u] = __ldcs(nb + sk);
+            np[u] = __ldcs(nb + sp);
+          }
         }
-        const int sk = rA * M2 + p, sp = rB * M2 + qi;                 // spectrum slots
-        const int ek = lay(sA * M2 + p, pz), ep = lay(sB * M2 + qi, pz);   // tile positions
-        const float2 Zk = fwd ? z[ek] : make_float2(0.f, 0.f);
-        const float2 Zp = fwd ? z[ep] : make_float2(0.f, 0.f);
-        if (rA == 0 && p == 0) {
-          const float X0 = Zk.x + Zk.y, XM = Zk.x - Zk.y;
-          if (mode == kRowSpectrum) { q.dtab[d.spec] = make_float2(X0, XM); continue; }
-          if (mode == kRowNatural) {
-            q.a.natural[d.nat] = make_float2(X0, 0.f);
-            q.a.natural[d.nat + M] = make_float2(XM, 0.f);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          if (!act[u]) continue;
+          const int p = pv[u], qi = qv[u], rA = first + jv[u];
+          const int rB = self ? rA : M1 - rA, sA = self ? 0 : 2 * jv[u], sB = self ? 0 : sA + 1;
+          const int sk = rA * M2 + p, sp = rB * M2 + qi;                     // spectrum slots
+          const int ek = lay(sA * M2 + p), ep = lay(sB * M2 + qi);           // tile positions
+          const float2 Zk = fwd ? z[ek] : make_float2(0.f, 0.f);
+          const float2 Zp = fwd ? z[ep] : make_float2(0.f, 0.f);
+          if (rA == 0 && p == 0) {
+            const float X0 = Zk.x + Zk.y, XM = Zk.x - Zk.y;
+            if (mode == kRowSpectrum) { q.dtab[d.spec] = make_float2(X0, XM); continue; }
+            if (mode == kRowNatural) {
+              q.a.natural[d.nat] = make_float2(X0, 0.f);
+              q.a.natural[d.nat + M] = make_float2(XM, 0.f);
+              continue;
+            }
+            const float2 D = Dk[u];
+            const float n0 = nk[u], nM = __ldg(q.nyq + c);
+            if (want_x2) {
+              const float f0 = D.x - X0, fM = D.y - XM;
+              x2 += __fdividef(f0 * f0, n0 + cn) + __fdividef(fM * fM, nM + cn);
+            }
+            if (!inv) continue;
+            const float Y0 = filt(make_float2(X0, 0.f), make_float2(D.x, 0.f), n0).x;
+            const float YM = filt(make_float2(XM, 0.f), make_float2(D.y, 0.f), nM).x;
+            z[ek] = make_float2(Y0 + YM, Y0 - YM);
             continue;
           }
-          const float2 D = load_d ? dt[0] : make_float2(0.f, 0.f);
-          const float n0 = nb[0], nM = __ldg(q.nyq + c);
+          const float2 w = cmul(__ldg(&G.pack_a[rA]), __ldg(&G.pack_b[p]));   // w_{2M}^k
+          const float2 E = cscale(cadd(Zk, cconj(Zp)), 0.5f);
+          const float2 O = cscale(mul_i<-1>(csub(Zk, cconj(Zp))), 0.5f);
+          const float2 wO = cmul(w, O);
+          const float2 Xk = cadd(E, wO);
+          const float2 Xp = cconj(csub(E, wO));
+          const bool same = self && qi == p;                 // k == M - k
+          if (mode == kRowSpectrum) {
+            q.dtab[d.spec + sk] = Xk;
+            if (!same) q.dtab[d.spec + sp] = Xp;
+            continue;
+          }
+          if (mode == kRowNatural) {
+            const int k = rA + M1 * p;
+            q.a.natural[d.nat + k] = Xk;
+            q.a.natural[d.nat + M - k] = Xp;
+            continue;
+          }
           if (want_x2) {
-            const float e0 = D.x - X0, eM = D.y - XM;
-            x2 += __fdividef(e0 * e0, n0 + cn) + __fdividef(eM * eM, nM + cn);
+            const float2 e1 = csub(Dk[u], Xk), e2 = csub(Dp[u], Xp);
+            float tt = __fdividef(e1.x * e1.x + e1.y * e1.y, nk[u] + cn);
+            if (!same) tt += __fdividef(e2.x * e2.x + e2.y * e2.y, np[u] + cn);
+            x2 += 2.f * tt;
           }
           if (!inv) continue;
-          const float Y0 = filt(make_float2(X0, 0.f), make_float2(D.x, 0.f), n0).x;
-          const float YM = filt(make_float2(XM, 0.f), make_float2(D.y, 0.f), nM).x;
-          z[ek] = make_float2(Y0 + YM, Y0 - YM);
-          continue;
+          const float2 Yk = filt(Xk, Dk[u], nk[u]);
+          const float2 Yp = filt(Xp, Dp[u], np[u]);
+          // Z'_k = (Y_k + conj Y_p) + i conj(w) (Y_k - conj Y_p)
+          // Z'_p = (Y_p + conj Y_k) - i w (Y_p - conj Y_k)
+          z[ek] = cadd(cadd(Yk, cconj(Yp)), mul_i<+1>(cmulc(csub(Yk, cconj(Yp)), w)));
+          if (!same) z[ep] = csub(cadd(Yp, cconj(Yk)), mul_i<+1>(cmul(w, csub(Yp, cconj(Yk)))));
         }
-        const float2 w = cmul(__ldg(&G.pack_a[rA]), __ldg(&G.pack_b[p]));   // w_{2M}^k
-        const float2 E = cscale(cadd(Zk, cconj(Zp)), 0.5f);
-        const float2 O = cscale(mul_i<-1>(csub(Zk, cconj(Zp))), 0.5f);
-        const float2 wO = cmul(w, O);
-        const float2 Xk = cadd(E, wO);
-        const float2 Xp = cconj(csub(E, wO));
-        const bool same = self && qi == p;                 // k == M - k
-        if (mode == kRowSpectrum) {
-          q.dtab[d.spec + sk] = Xk;
-          if (!same) q.dtab[d.spec + sp] = Xp;
-          continue;
-        }
-        if (mode == kRowNatural) {
-          const int k = rA + M1 * p;
-          q.a.natural[d.nat + k] = Xk;
-          q.a.natural[d.nat + M - k] = Xp;
-          continue;
-        }
-        const float2 Dk = load_d ? __ldcs(dt + sk) : make_float2(0.f, 0.f);
-        const float2 Dp = load_d ? __ldcs(dt + sp) : make_float2(0.f, 0.f);
-        const float nk = __ldcs(nb + sk), np = __ldcs(nb + sp);
-        if (want_x2) {
-          const float2 e1 = csub(Dk, Xk), e2 = csub(Dp, Xp);
-          float tt = __fdividef(e1.x * e1.x + e1.y * e1.y, nk + cn);
-          if (!same) tt += __fdividef(e2.x * e2.x + e2.y * e2.y, np + cn);
-          x2 += 2.f * tt;
-        }
-        if (!inv) continue;
-        const float2 Yk = filt(Xk, Dk, nk);
-        const float2 Yp = filt(Xp, Dp, np);
-        // Z'_k = (Y_k + conj Y_p) + i conj(w) (Y_k - conj Y_p)
-        // Z'_p = (Y_p + conj Y_k) - i w (Y_p - conj Y_k)
-        z[ek] = cadd(cadd(Yk, cconj(Yp)), mul_i<+1>(cmulc(csub(Yk, cconj(Yp)), w)));
-        if (!same) z[ep] = csub(cadd(Yp, cconj(Yk)), mul_i<+1>(cmul(w, csub(Yp, cconj(Yk)))));
       }
     }
+    if (threadIdx.x < 32 && more) fetch(nj, nw);
     if (want_x2) {
       // block reduction: FP32 within warps, FP64 across warps and CTAs
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) x2 += __shfl_down_sync(0xffffffffu, x2, o);
       if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x2;
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        double sum = 0.0;
-        for (int w = 0; w < T / 32; ++w) sum += red[w];
-        atomicAdd(chi2, sum / (double)d.n);
+    }
+    __syncthreads();
+    if (want_x2 && (int)threadIdx.x >= T - 32) {   // one warp; the others go on
+      double sum = lane < T / 32 ? f32_to_f64(red[lane]) : 0.0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+      if (lane == 0) atomicAdd(chi2, sum * G.inv_n);
+    }
+    if (threadIdx.x < 32) {
+      if (more) {
+        put(cur ^ 1, nj, nw);
+        // the next job's rows (and its d~ / Nbar rows) into L2 while this one ends, a row a lane
+        const GenChunk& Gn = s_rec[cur ^ 1];
+        const int nM1 = Gn.d.M1, nM2 = Gn.d.M2;
+        const int nrow = nj.z == 0 ? 1 : 2 * nj.z;
+        const float2* yn = q.ybuf + (Gn.yoff - q.base_y);
+        for (int s = lane; s < nrow; s += 32) {
+          const int r = nj.z == 0 ? nj.y : ((s & 1) ? nM1 - nj.y - (s >> 1) : nj.y + (s >> 1));
+          // rows of general chunks need not start on 16 bytes: prefetch their aligned interior
+          if (fwd) prefetch_l2_inner(yn + (int64_t)r * nM2, 8 * (size_t)nM2);
+          if (load_d) prefetch_l2_inner(q.dtab + Gn.d.spec + (int64_t)r * nM2, 8 * (size_t)nM2);
+          prefetch_l2_inner(q.nbar + Gn.d.spec + (int64_t)r * nM2, 4 * (size_t)nM2);
+        }
       }
     }
     if (inv) {
-      __syncthreads();
-      const float2* r = gen_dft_rows<+1>(z, other, pz, M2, G.nr2, G.rad2, G.tw_row, nseq, T);
-      for (int e = threadIdx.x; e < nseq * M2; e += T) {
-        const int sq = fm2.div(e), p = e - sq * M2;
-        const int row = row_of(sq);
-        y[(int64_t)row * M2 + p] = cmulc(r[lay(e, pz)], gen_tw_big(G, row * p));
-      }
+      gen_dft_rows<+1, kSmem, kGlobal>(z, other, M2, G.nr2, G.rad2, G.tw_row, nseq, T, io);
     }
+    if (threadIdx.x == 0) s_more = more;
     __syncthreads();
+  }
+  if (threadIdx.x == 0) {   // the last CTA out clears the counters for the next launch
+    __threadfence();
+    if (atomicAdd(q.queue + 1, 1u) == gridDim.x - 1) {
+      q.queue[0] = 0u;
+      q.queue[1] = 0u;
+      __threadfence();
+    }
   }
 }
 
@@ -693,7 +856,7 @@ __global__ void __launch_bounds__(1024) k_gen_row(GenParams q) {
 // M1 j2_0 nh + (j1 w + j2 - j2_0) nh + h, nh = 2 (even) or 1 (odd): a bijection of the
 // chunk's samples.
 __global__ void k_gen_tile_pointing(const int32_t* __restrict__ pix, const void* cosw,
-                                    const void* sinw, int wbytes, int64_t off, int n, int M1,
+                                    const void* sinw, int wbytes, int64_t off, int64_t toff, int n, int M1,
                                     int M2, int cplx, int nb, int32_t* __restrict__ tpix,
                                     void* tcos, void* tsin) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -704,7 +867,7 @@ __global__ void k_gen_tile_pointing(const int32_t* __restrict__ pix, const void*
   const int j1 = (int)(j / M2), j2 = (int)(j % M2);
   const int j2_0 = j2 - j2 % nb;
   const int w = min(nb, M2 - j2_0);
-  const int64_t o = off + ((int64_t)M1 * j2_0 + (int64_t)j1 * w + (j2 - j2_0)) * nh + h;
+  const int64_t o = toff + ((int64_t)M1 * j2_0 + (int64_t)j1 * w + (j2 - j2_0)) * nh + h;
   tpix[o] = pix[off + i];
   if (cosw) {
     if (wbytes == 2) {
@@ -723,7 +886,7 @@ cudaError_t launch_gen_tile_pointing(const mm_plan_s* p, cudaStream_t st) {
   for (int i = 0; i < p->n_gen; ++i) {
     const ChunkDesc& d = p->h_desc[p->h_gen_chunks[i]];
     k_gen_tile_pointing<<<(unsigned)((d.n + 255) / 256), 256, 0, st>>>(
-        p->pix, p->cosw, p->sinw, wb, d.off, d.n, d.M1, d.M2, d.cplx, p->gen_tune.col_nb,
+        p->pix, p->cosw, p->sinw, wb, d.off, p->h_gen_toff[i], d.n, d.M1, d.M2, d.cplx, p->gen_tune.col_nb,
         p->tpix, p->tcos, p->tsin);
   }
   return cudaGetLastError();
@@ -749,6 +912,7 @@ static GenParams gen_params(const mm_plan_s* p, const Batch& b, const int2* item
   q.ybuf = p->ybuf;
   q.acc = p->acc;
   q.acc_stride = acc_stride_of(p->n_pix, p->ncomp);
+  q.queue = p->row_queue;
   q.dtab = p->dtab;
   q.nbar = p->nbar;
   q.nyq = p->nyq;
@@ -823,9 +987,10 @@ cudaError_t launch_gen_row(const mm_plan_s* p, const Batch& b, const RowArgs& a,
   }
   q.tile = emax + (emax >> 4) + 1;
   const size_t smem = 2 * sizeof(float2) * (size_t)q.tile;
-  auto k = a.mode == kRowMessenger    ? k_gen_row<kRowMessenger>
-           : a.mode == kRowMessengerF ? k_gen_row<kRowMessengerF>
-                                      : k_gen_row<-1>;
+  const bool narrow = p->gen_tune.row_threads <= 256;
+  auto k = a.mode == kRowMessenger    ? (narrow ? k_gen_row<kRowMessenger, 256> : k_gen_row<kRowMessenger, 1024>)
+           : a.mode == kRowMessengerF ? (narrow ? k_gen_row<kRowMessengerF, 256> : k_gen_row<kRowMessengerF, 1024>)
+                                      : (narrow ? k_gen_row<-1, 256> : k_gen_row<-1, 1024>);
   return gen_launch(k, p->gen_tune.row_threads, smem, q.n_items, q, st);
 }
 

@@ -31,19 +31,19 @@ struct ChunkDesc {
 
 // Chunks of the same length share FFT shapes and twiddle tables and run in one launch.
 // Power-of-two lengths use the compile-time kernels; other 5-smooth lengths ("general")
-// use runtime mixed-radix Stockham passes with the radix sequences below.
+// use runtime mixed-radix Stockham passes.
 constexpr int kMaxRadices = 16;
 struct Group {
   int M, M1, M2, log_lo;   // w_M^e = tw_hi[e >> log_lo] * tw_lo[e & (2^log_lo - 1)]
   int n_chunks;
   int batch;               // chunks per batch
   int general, cplx;       // general path; odd length (complex transform)
-  int nr1, nr2;            // general: radix sequences of the M1 and M2 DFTs
-  int8_t rad1[kMaxRadices], rad2[kMaxRadices];
   int* chunks;             // device: chunk indices of this group
   float2* tw_col;          // per-pass twiddles of the length-M1 DFT (see tw_offset;
                            // general: [< 2 M1], pass tables of the tuned radix plan)
   float2* tw_row;          // per-pass twiddles of the length-M2 DFT (general: [< 2 M2])
+  float2* tw_col_d;        // general: the same of the data transform's plan
+  float2* tw_row_d;
   float2* tw_lo;           // [2^log_lo]          exp(-2 pi i m / M)
   float2* tw_hi;           // [M >> log_lo (+1)]   exp(-2 pi i m 2^log_lo / M)
   // four-step twiddles by tile and row (power-of-two lengths; see four_step_lo): column tile t:
@@ -107,8 +107,15 @@ struct GenChunk {
   int c;                   // chunk index in the plan
   int log_lo, nr1, nr2;
   int64_t yoff;            // intermediate offset in the general list
+  double inv_n;            // 1 / n
+  int64_t toff;            // first sample in the tile-order pointing (a multiple of 4)
   const float2* tw_col;    // per-pass tables of the M1 DFT for the radix plan rad1
   const float2* tw_row;    // per-pass tables of the M2 DFT for the radix plan rad2
+  // the data transform's plan (small radices, see radix_plan) and its tables
+  const float2* tw_col_d;
+  const float2* tw_row_d;
+  int nr1d, nr2d;
+  int8_t rad1d[kMaxRadices], rad2d[kMaxRadices];
   const float2* tw_lo;
   const float2* tw_hi;
   const float2* pack_a;
@@ -198,6 +205,7 @@ struct mm_plan_s {
   int64_t* h_gen_ctile;
   int64_t* h_gen_rjob;
   int64_t* h_gen_yoff;
+  int64_t* h_gen_toff;     // first sample in the tile-order pointing (multiples of 4)
   int* h_gen_chunks;
   mm::GenChunk* gen_rec;   // [n_gen] device records
   int2* gen_ctab;          // column tiles: (general index, first column), capacity gen_ccap
@@ -369,12 +377,81 @@ __device__ __forceinline__ void dft5(float2* v) {
 }
 
 template <int R, int DIR>
+__device__ __forceinline__ void dft_small(float2* v) {
+  if constexpr (R == 2) dft2<DIR>(v[0], v[1]);
+  else if constexpr (R == 3) dft3<DIR>(v);
+  else dft5<DIR>(v);
+}
+
+// DFT of N1 N2 points, N1 and N2 coprime, by the prime-factor map (no twiddles): input n =
+// (N2 n1 + N1 n2) mod N, output k = k1 mod N1 and k2 mod N2.
+template <int N1, int N2, int DIR>
+__device__ __forceinline__ void dft_coprime(float2* v) {
+  constexpr int N = N1 * N2;
+  float2 a[N2][N1];
+#pragma unroll
+  for (int n2 = 0; n2 < N2; ++n2) {
+#pragma unroll
+    for (int n1 = 0; n1 < N1; ++n1) a[n2][n1] = v[(N2 * n1 + N1 * n2) % N];
+    dft_small<N1, DIR>(a[n2]);
+  }
+#pragma unroll
+  for (int k1 = 0; k1 < N1; ++k1) {
+    float2 b[N2];
+#pragma unroll
+    for (int n2 = 0; n2 < N2; ++n2) b[n2] = a[n2][k1];
+    dft_small<N2, DIR>(b);
+#pragma unroll
+    for (int k2 = 0; k2 < N2; ++k2) {
+      int k = k1;                       // the k < N with k = k1 mod N1, k = k2 mod N2
+#pragma unroll
+      for (int i = 0; i < N2; ++i)
+        if (k % N2 != k2) k += N1;
+      v[k] = b[k2];
+    }
+  }
+}
+
+// DFT of 9 points as 3 x 3 with the twiddles w9^(n1 k2).
+template <int DIR>
+__device__ __forceinline__ void dft9(float2* v) {
+  constexpr float c[3] = {0.76604444311897803520f, 0.17364817766693034885f, -0.93969262078590838405f};   // cos(2 pi j / 9), j = 1, 2, 4
+  constexpr float w[3] = {0.64278760968653932632f, 0.98480775301220805937f, 0.34202014332566873304f};    // sin
+  float2 a[3][3];
+#pragma unroll
+  for (int n1 = 0; n1 < 3; ++n1) {
+#pragma unroll
+    for (int n2 = 0; n2 < 3; ++n2) a[n1][n2] = v[n1 + 3 * n2];
+    dft3<DIR>(a[n1]);
+  }
+  auto tw = [&](float2 z, int j) {
+    const float sn = DIR < 0 ? -w[j] : w[j];
+    return make_float2(z.x * c[j] - z.y * sn, z.x * sn + z.y * c[j]);
+  };
+  a[1][1] = tw(a[1][1], 0);
+  a[1][2] = tw(a[1][2], 1);
+  a[2][1] = tw(a[2][1], 1);
+  a[2][2] = tw(a[2][2], 2);
+#pragma unroll
+  for (int k2 = 0; k2 < 3; ++k2) {
+    float2 b[3] = {a[0][k2], a[1][k2], a[2][k2]};
+    dft3<DIR>(b);
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) v[k2 + 3 * k1] = b[k1];
+  }
+}
+
+template <int R, int DIR>
 __device__ __forceinline__ void dftR(float2* v) {
   if constexpr (R == 2) dft2<DIR>(v[0], v[1]);
   else if constexpr (R == 3) dft3<DIR>(v);
   else if constexpr (R == 4) dft4<DIR>(v[0], v[1], v[2], v[3]);
   else if constexpr (R == 5) dft5<DIR>(v);
+  else if constexpr (R == 6) dft_coprime<2, 3, DIR>(v);
   else if constexpr (R == 8) dft8<DIR>(v);
+  else if constexpr (R == 9) dft9<DIR>(v);
+  else if constexpr (R == 10) dft_coprime<2, 5, DIR>(v);
+  else if constexpr (R == 15) dft_coprime<3, 5, DIR>(v);
   else dft16<DIR>(v);
 }
 

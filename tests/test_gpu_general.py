@@ -315,3 +315,44 @@ def test_every_schedule_gives_the_same_iterate(uneven):
         assert rel(o, outs[0]) <= 1e-5
     with pytest.raises(binding.MMError):
         plan.set_tune(12, 256, 256, 0)
+
+
+@pytest.mark.parametrize("lens", [[2 * 9 * 16, 2 * 15 * 15], [2 * 6 * 10, 405, 2 * 25 * 25],
+                                  [2 * 729, 2 * 3 * 5, 2187, 2 * 4096 * 3], [2 * 500 * 3000, 2 * 480 * 4096]])
+@pytest.mark.parametrize("order", [0, 1, 2])
+def test_wide_radices_match_oracle(lens, order):
+    """Every radix of the iterations' plans (2 to 16, prime-factor and 3 x 3 butterflies) in column
+    and row DFTs, at the ends that read and write the intermediate, with odd and long chunks: a
+    step at lambda = inf, 3 and 1 within 1e-5 of the oracle, the rfft within 1e-6 rel-L2."""
+    import oracle.messenger as O
+    rng = np.random.default_rng(3)
+    n, npix = int(sum(lens)), 50
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    pix = np.repeat(rng.integers(-1, npix, size=n // 3 + 1), 3)[:n].astype(np.int32)
+    tod = rng.standard_normal(n).astype(np.float32)
+    params = np.array([[1.0, 0.5, 1.5, 50.0]] * len(lens))
+    prob = O.problem_from_synth(dict(pix=pix, cos=None, sin=None, tod=tod, offsets=off, npix=npix, ncomp=1,
+                                     params=params))
+    plan = binding.Plan(off, torch.from_numpy(pix).cuda(), None, None, npix, 1)
+    plan.set_tune(8, 512, 256 if order else 512, order)
+    d = torch.from_numpy(tod).cuda()
+    plan.set_noise(d, params=params)
+    m0 = rng.standard_normal((npix, 1))
+    for lam in (math.inf, 3.0, 1.0):
+        ref, chi_ref = O.messenger_step(prob, m0, lam)
+        m = torch.from_numpy(m0.copy()).cuda()
+        m2 = torch.zeros_like(m)
+        plan.stage(binding.MM_STAGE_LOAD, map_inout=m)     # the three general kernels, whatever the size
+        chi = torch.zeros(1, dtype=torch.float64, device="cuda")
+        for b in range(plan.n_batches()):
+            plan.stage(binding.MM_STAGE_GATHER_FFT, b)
+            plan.stage(binding.MM_STAGE_FILTER, b, lam, chi2_slot=chi)
+            plan.stage(binding.MM_STAGE_IFFT_BIN, b)
+        plan.stage(binding.MM_STAGE_MAP, map_inout=m2)
+        assert np.linalg.norm(m2.cpu().numpy() - ref) <= 1e-5 * np.linalg.norm(ref)
+        assert abs(chi.item() - chi_ref) <= 1e-5 * chi_ref
+    spec = torch.empty(sum(k // 2 + 1 for k in lens), 2, dtype=torch.float32, device="cuda")
+    plan.rfft(d, spec)
+    want = np.concatenate([np.fft.rfft(tod[off[c]:off[c + 1]].astype(np.float64)) for c in range(len(lens))])
+    got = spec.cpu().numpy().astype(np.float64)
+    assert np.linalg.norm(got[:, 0] + 1j * got[:, 1] - want) <= 1e-6 * np.linalg.norm(want)
