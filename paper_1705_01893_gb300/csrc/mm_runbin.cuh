@@ -4,13 +4,15 @@
 //
 // What bounds it: a reduction per sample and sum saturates the L2's atomic units (12 per
 // sample for the weight blocks: 1.90 ms for 8 x 2^22 samples), and FP64 arithmetic runs on a
-// pipe of about two lanes per SM and clock.  So the runs of a tile of 1024 samples are listed
-// by warp ballots, a thread sums one run (5 to 8 FP64 instructions a sample, products and sums
-// contracted), and the finished sums are handed out again one (run, sum) per lane, so that a
-// warp's reductions cover the consecutive words of two to ten pixels instead of 32 scattered
-// ones.  Measured on 512^2 IQU rasters at 4 samples per pixel: weight blocks of 8 x 2^22
-// samples 1900 -> 652 us (9.96 M FP64 warp instructions, 0.5 ms of that pipe), P^T 425 -> 289 us,
-// binned map of 2 x 2^22 samples 349 -> 181 us.
+// pipe of about two lanes per SM and clock.  So a lane takes four consecutive samples and adds
+// them up while they stay on one pixel (5 to 8 FP64 instructions a sample, products and sums
+// contracted, no lane idle); where a run of the lane ends, its sums go through shared memory and
+// are handed out again one (run, sum) per lane, so that a warp's reductions cover the
+// consecutive words of two to ten pixels instead of 32 scattered ones.  Lists of whole runs, a
+// run a thread, leave the FP64 pipe half idle where the runs differ in length (P^T of 2 M samples
+// on a diagonal raster 31 us, 24.7 so).  Measured on 512^2 IQU rasters at 4 samples per pixel:
+// weight blocks of 8 x 2^22 samples 1900 -> 566 us, P^T 425 -> 239 us, binned map of 2 x 2^22
+// samples 349 -> 150 us.
 #pragma once
 
 #include "mm_internal.cuh"
@@ -28,7 +30,8 @@ __device__ __forceinline__ float load_w(const void* w, int half_w, int64_t s) {
   return half_w ? __half2float(static_cast<const __half*>(w)[s]) : static_cast<const float*>(w)[s];
 }
 
-constexpr int kBinTile = 1024, kBinThreads = 256;
+constexpr int kBinWarps = 8, kBinSegs = 4, kBinThreads = 32 * kBinWarps;
+constexpr int kBinTile = kBinThreads * 4 * kBinSegs;
 
 // Op: NF float streams per sample (load), NV sums per run (add), NO outputs per run (emit).
 // Samples [n0, n1); samples with a pixel outside [0, n_pix) are skipped.  Op::tile(first,
@@ -37,87 +40,67 @@ constexpr int kBinTile = 1024, kBinThreads = 256;
 template <class Op>
 __global__ void __launch_bounds__(kBinThreads) k_run_bin(Op op, const int32_t* __restrict__ pix,
                                                          int64_t n0, int64_t n1, int64_t n_pix) {
-  constexpr int NF = Op::NF, NV = Op::NV, NO = Op::NO, W = kBinThreads / 32;
+  constexpr int NF = Op::NF, NV = Op::NV, NO = Op::NO;
   constexpr int SV = NV | 1;   // odd stride: the sums of neighbouring runs on different banks
-  __shared__ int s_pix[kBinTile];
-  __shared__ float s_f[NF > 0 ? NF : 1][kBinTile];
-  __shared__ uint16_t s_run[kBinTile];     // first position | (length - 1) << 11, valid runs only
-  static_assert(kBinTile <= 2048, "11 bits of position");
-  __shared__ double s_val[kBinThreads * SV];
-  __shared__ int s_cnt[W];
+  __shared__ double s_val_[kBinWarps][32 * SV];
+  __shared__ int2 s_at_[kBinWarps][32];      // pixel, tile position
   __shared__ double s_op[2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t base = n0 + (int64_t)blockIdx.x * kBinTile;
-  const int cnt = n1 - base < kBinTile ? (int)(n1 - base) : kBinTile;
-  op.tile(base, base + cnt - 1, s_op);
+  double* s_val = s_val_[warp];
+  int2* s_at = s_at_[warp];
+  const int64_t tile = n0 + (int64_t)blockIdx.x * kBinTile;
+  op.tile(tile, (n1 - tile < kBinTile ? n1 : tile + kBinTile) - 1, s_op);
+  __syncthreads();
+  for (int g = 0; g < kBinSegs; ++g) {
+    const int at = ((g * kBinWarps + warp) * 32 + lane) * 4;   // the lane's first sample in the tile
+    if (tile + at - 4 * lane >= n1) break;   // warp-uniform
+    int p[5];
+    float f[4][NF > 0 ? NF : 1];
 #pragma unroll
-  for (int k = 0; k < kBinTile / kBinThreads; ++k) {
-    const int i = threadIdx.x + k * kBinThreads;
-    if (i < cnt) {
-      s_pix[i] = pix[base + i];
+    for (int k = 0; k < 4; ++k) {
+      const int64_t s = tile + at + k;
+      const bool in = s < n1;
+      p[k] = in ? pix[s] : -1;
+      if (p[k] >= n_pix) p[k] = -1;
 #pragma unroll
-      for (int f = 0; f < NF; ++f) s_f[f][i] = op.load(f, base + i);
+      for (int j = 0; j < NF; ++j) f[k][j] = in ? op.load(j, s) : 0.f;
     }
-  }
-  __syncthreads();
-  // run starts: warp w lists positions [256 w, 256 w + 256) in rounds of 32; position 0 of a
-  // round always starts a run, so a run lies within its round (and has at most 32 samples)
-  constexpr int R = kBinTile / kBinThreads;
-  unsigned head[R], keep[R];
-  int mine = 0;
+    p[4] = -2;
+    double v[NV];
 #pragma unroll
-  for (int k = 0; k < R; ++k) {
-    const int i = warp * (32 * R) + 32 * k + lane;
-    const int p = i < cnt ? s_pix[i] : -1;
-    const bool h = lane == 0 || i >= cnt || p != s_pix[i - 1] || op.cut(i);
-    head[k] = __ballot_sync(0xffffffffu, h);
-    keep[k] = __ballot_sync(0xffffffffu, h && i < cnt && p >= 0 && p < n_pix);
-    mine += __popc(keep[k]);
-  }
-  if (lane == 0) s_cnt[warp] = mine;
-  __syncthreads();
-  int at = 0, nrun = 0;
+    for (int j = 0; j < NV; ++j) v[j] = 0.0;
+    int len = 0;
 #pragma unroll
-  for (int w = 0; w < W; ++w) {
-    const int c = s_cnt[w];
-    at += w < warp ? c : 0;
-    nrun += c;
-  }
-#pragma unroll
-  for (int k = 0; k < R; ++k) {
-    if ((keep[k] >> lane) & 1u) {
-      const unsigned later = lane == 31 ? 0u : head[k] >> (lane + 1);
-      const int len = later ? __ffs(later) : 32 - lane;
-      s_run[at + __popc(keep[k] & ((1u << lane) - 1u))] =
-          (uint16_t)((warp * (32 * R) + 32 * k + lane) | (len - 1) << 11);
-    }
-    at += __popc(keep[k]);
-  }
-  __syncthreads();
-  for (int r0 = 0; r0 < nrun; r0 += kBinThreads) {
-    const int nb = nrun - r0 < kBinThreads ? nrun - r0 : kBinThreads;
-    if ((int)threadIdx.x < nb) {
-      const int e = s_run[r0 + threadIdx.x], a = e & 2047, b = a + (e >> 11) + 1;
-      double v[NV];
-#pragma unroll
-      for (int j = 0; j < NV; ++j) v[j] = 0.0;
-      for (int i = a; i < b; ++i) {
-        float f[NF > 0 ? NF : 1];
-#pragma unroll
-        for (int j = 0; j < NF; ++j) f[j] = s_f[j][i];
-        op.add(v, f);
+    for (int k = 0; k < 4; ++k) {
+      const bool on = p[k] >= 0;
+      if (on) {
+        op.add(v, f[k]);
+        ++len;
       }
-      op.close(v, b - a);
+      // runs that end at this sample
+      const bool end = on && (p[k + 1] != p[k] || (k < 3 && op.cut(at + k + 1)));
+      const unsigned m = __ballot_sync(0xffffffffu, end);
+      if (m == 0) continue;
+      if (end) {
+        const int r = __popc(m & ((1u << lane) - 1u));
+        op.close(v, len);
+        s_at[r] = make_int2(p[k], at + k);
 #pragma unroll
-      for (int j = 0; j < NV; ++j) s_val[threadIdx.x * SV + j] = v[j];
+        for (int j = 0; j < NV; ++j) {
+          s_val[r * SV + j] = v[j];
+          v[j] = 0.0;
+        }
+        len = 0;
+      }
+      __syncwarp();
+      const int nr = __popc(m);
+      for (int t = lane; t < nr * NO; t += 32) {
+        const int r = t / NO, o = t - r * NO;
+        const int2 e = s_at[r];
+        op.emit(e.x, o, s_val + r * SV, tile + e.y, s_op);
+      }
+      __syncwarp();
     }
-    __syncthreads();
-    for (int t = threadIdx.x; t < nb * NO; t += kBinThreads) {
-      const int r = t / NO, o = t - r * NO;
-      const int a = s_run[r0 + r] & 2047;
-      op.emit(s_pix[a], o, s_val + r * SV, base + a, s_op);
-    }
-    __syncthreads();
   }
 }
 
