@@ -369,7 +369,7 @@ static cudaError_t col_adjoint_m1(const mm_plan_s* p, const Batch& b, const AdjC
                                   cudaStream_t st) {
   constexpr int T = col_threads(M1);
   const Group& g = p->groups[b.group];
-  ColParams q;
+  ColParams q{};
   q.desc = p->d_desc;
   q.chunks = g.chunks + b.first;
   q.count = b.count;

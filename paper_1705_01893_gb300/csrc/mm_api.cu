@@ -168,7 +168,9 @@ static int radix_plan(int L, int8_t* rad, int order = 0) {
 // 4, 5, 6, 8, 9, 10, 15 and 16 (three for nearly every length up to 4096, where radices up to 8
 // take four to six), the smallest sum of radices among those.  A pass costs a trip of the tile
 // through shared memory, its barrier and index arithmetic.  order 0: large radices first; 1:
-// small ones first; 2: the odd ones first.  @WIDE@
+// small ones first; 2: the odd ones first.  64 uneven chunks on 1024^2, with the first and last
+// passes on the intermediate itself: inverse columns 264 -> 226 us, rows 328 -> 330 (those were
+// bound by what their jobs began and ended with, see k_gen_row: 234 since).
 static int radix_plan_wide(int L, int8_t* rad, int order) {
   static const int set[] = {16, 15, 10, 9, 8, 6, 5, 4, 3, 2};
   struct Best { int n, sum, first; };
@@ -226,7 +228,7 @@ constexpr int kNoiseTable = 1024 + 32;
 // -------------------------------------------------------------------- workspace layout
 struct Layout {
   size_t desc, chunks, params, ntab, tw, hits, valid, W, Minv, acc, acc12, map4, bvec, dtab, nbar, nyq, c0,
-      ybuf, scal, tpix, tcos, tsin, lam, iter, map64, groups, gen, gen_rec, gen_ctab, gen_rtab,
+      ybuf, scal, tpix, tcos, tsin, tpix2, tcos2, tsin2, lam, iter, map64, groups, gen, gen_rec, gen_ctab, gen_rtab,
       adapt, queue, fitems, fctr, fault, small, total, ybytes;
   int64_t gen_ccap, gen_rcap;
   int lam_cap;
@@ -253,7 +255,7 @@ static size_t ybuf_budget() {
 }
 
 static mm_status make_layout(int n_chunks, const int64_t* off, int64_t n_pix, int ncomp,
-                             int wdtype, Layout* L, bool force_general = false) {
+                             int wdtype, Layout* L, bool composite = false) {
   MM_ARG(n_chunks >= 1, "n_chunks must be >= 1 (got %d)", n_chunks);
   MM_ARG(off != nullptr, "offsets is NULL");
   MM_ARG(n_pix >= 1 && n_pix < (int64_t(1) << 31), "n_pix out of range (%lld)", (long long)n_pix);
@@ -270,7 +272,7 @@ static mm_status make_layout(int n_chunks, const int64_t* off, int64_t n_pix, in
   // launches of a few small waves (about 25 us per iteration for one chunk of 2^17 samples
   // beside 24.6 M general samples: 0.851 -> 0.827 ms), more than the general kernels' lower
   // rate costs on that many samples.
-  bool any_general = force_general;
+  bool any_general = false;
   std::vector<std::pair<int64_t, int64_t>> pow2_total;   // (length, samples of that length)
   for (int c = 0; c < n_chunks; ++c) {
     const int64_t n = off[c + 1] - off[c];
@@ -293,7 +295,13 @@ static mm_status make_layout(int n_chunks, const int64_t* off, int64_t n_pix, in
     MM_ARG(n >= 1, "chunk %d is empty or offsets decrease", c);
     int M, M1, M2, cplx = 0;
     bool general = false;
-    if (force_general || joins_general(n) || !(fft_shape(n, &M, &M1, &M2) && off[c] % 4 == 0)) {
+    if (composite && !gen_shape(n, &M, &M1, &M2, &cplx)) {   // the lengths composite plans take
+      mm_set_error("chunk %d: length %lld unsupported in a composite plan (prime factors 2, 3, 5 "
+                   "only, n/2 up to 2^21)", c, (long long)n);
+      return MM_ERR_UNSUPPORTED;
+    }
+    cplx = 0;
+    if (joins_general(n) || !(fft_shape(n, &M, &M1, &M2) && off[c] % 4 == 0)) {
       if (!gen_shape(n, &M, &M1, &M2, &cplx)) {
         mm_set_error("chunk %d: length %lld unsupported (need prime factors 2, 3, 5 only and "
                      "n <= 2^24; n/2 up to 2^21 for lengths that are not powers of two)",
@@ -386,6 +394,10 @@ static mm_status make_layout(int n_chunks, const int64_t* off, int64_t n_pix, in
   L->tpix = take(sizeof(int32_t) * (size_t)tile_n);
   L->tcos = take(wb * (size_t)tile_n);
   L->tsin = take(wb * (size_t)tile_n);
+  const size_t n2 = composite && ngen < (size_t)n_chunks ? (size_t)L->n_total : 0;
+  L->tpix2 = take(sizeof(int32_t) * n2);
+  L->tcos2 = take(wb * n2);
+  L->tsin2 = take(wb * n2);
   // graph mode: schedule table, iteration counter + chi^2 pointer slot, FP64 map
   L->lam_cap = 65536;
   L->lam = take(sizeof(double) * L->lam_cap);
@@ -867,7 +879,7 @@ __global__ void k_map_to4(int64_t n_pix, const double* __restrict__ map,
 
 // ----------------------------------------------------------------- operator kernels
 // Four samples of P m a thread with 16-byte accesses (8-byte for FP16 weights), for arrays on
-// such boundaries; 8 x 2^22 samples of the 512^2 map: 159 -> 98 us (one sample a thread is
+// such boundaries; 8 x 2^22 samples of the 512^2 map: 159 -> 78 us (one sample a thread is
 // short of loads in flight).
 template <int NC>
 __global__ void k_gather_vec(int64_t n4, const int32_t* __restrict__ pix, const void* cosw,
@@ -1325,6 +1337,9 @@ static mm_status plan_create(mm_plan* out, int n_chunks, const int64_t* offsets,
   p->tpix = reinterpret_cast<int32_t*>(ws + L.tpix);
   p->tcos = ncomp == 3 ? static_cast<void*>(ws + L.tcos) : nullptr;
   p->tsin = ncomp == 3 ? static_cast<void*>(ws + L.tsin) : nullptr;
+  p->tpix2 = reinterpret_cast<int32_t*>(ws + L.tpix2);
+  p->tcos2 = ncomp == 3 ? static_cast<void*>(ws + L.tcos2) : nullptr;
+  p->tsin2 = ncomp == 3 ? static_cast<void*>(ws + L.tsin2) : nullptr;
   p->d_groups = reinterpret_cast<Group*>(ws + L.groups);
   p->n_gen = (int)L.gen_list.size();
   {

@@ -28,15 +28,15 @@ __global__ void __launch_bounds__(T, pass_ctas(T, 8)) k_col_forward(ColParams q)
                                              DstYData{q.ybuf + (int64_t)ci * d.M, &q.g, j2_0, M2});
     } else {
       load_col_twiddles<M1, CB, T>(s4, q.g, cb);
-      smem_fft<M1, CB, ColLayout<CB>, T, -1>(
-          sm, q.g.tw_col, SrcGather<NC, CB>{&q, d.off + (int64_t)cb * (2 * CB * M1)},
-          DstY<M1, CB, true>{q.ybuf + (int64_t)ci * d.M, s4, j2_0, M2});
+      using Src = typename std::conditional<SRC == kSrcGather2, SrcGather2<NC, CB>, SrcGather<NC, CB>>::type;
+      smem_fft<M1, CB, ColLayout<CB>, T, -1>(sm, q.g.tw_col, Src{&q, d.off + (int64_t)cb * (2 * CB * M1)},
+                                             DstY<M1, CB, true>{q.ybuf + (int64_t)ci * d.M, s4, j2_0, M2});
     }
     __syncthreads();
   }
 }
 
-template <int M1, int CB, int T, int NC>
+template <int M1, int CB, int T, int NC, bool COMP>
 __global__ void __launch_bounds__(T, pass_ctas(T, 8)) k_col_inverse(ColParams q) {
   extern __shared__ float2 sm[];
   const int M2 = q.g.M2;
@@ -64,7 +64,9 @@ __global__ void __launch_bounds__(T, pass_ctas(T, 8)) k_col_inverse(ColParams q)
       // lie in one row i
       const int i = e / RUN;
       const int so = e + (Lay::kPad ? 2 * (i >> 4) * Lay::kPad : 0);
-      scatter4<NC, ROWL>(q, tbase + e, *reinterpret_cast<const float4*>(smf + so), e4 & (ROWL - 1));
+      const float4 t4 = *reinterpret_cast<const float4*>(smf + so);
+      if constexpr (COMP) scatter4_pair<NC, ROWL>(q, tbase + e, t4, e4 & (ROWL - 1));
+      else scatter4<NC, ROWL>(q, tbase + e, t4, e4 & (ROWL - 1));
     }
     __syncthreads();
   }
@@ -116,12 +118,19 @@ cudaError_t launch_tile_pointing(const mm_plan_s* p, cudaStream_t st) {
   const uintptr_t wm = wb == 2 ? 7 : 15;
   const int aligned = (((uintptr_t)p->pix & 15) == 0 ? 1 : 0) |
                       ((((uintptr_t)p->cosw | (uintptr_t)p->sinw) & wm) == 0 ? 2 : 0);
+  const int aligned_b = (((uintptr_t)p->pix_b & 15) == 0 ? 1 : 0) |
+                        ((((uintptr_t)p->cos_b | (uintptr_t)p->sin_b) & wm) == 0 ? 2 : 0);
   for (int c = 0; c < p->n_chunks; ++c) {
     const ChunkDesc& d = p->h_desc[c];
     if (p->groups[d.grp].general) continue;   // the general path has its own tile copy
-    k_tile_pointing<<<(unsigned)((d.n / 4 + 255) / 256), 256, 0, st>>>(
+    const unsigned grid = (unsigned)((d.n / 4 + 255) / 256);
+    k_tile_pointing<<<grid, 256, 0, st>>>(
         p->pix, p->cosw, p->sinw, wb, d.off, ilog2(d.M1), ilog2(d.M2), ilog2(2 * col_cb(d.M1)), aligned,
         p->tpix, p->tcos, p->tsin);
+    if (p->composite)
+      k_tile_pointing<<<grid, 256, 0, st>>>(
+          p->pix_b, p->cos_b, p->sin_b, wb, d.off, ilog2(d.M1), ilog2(d.M2), ilog2(2 * col_cb(d.M1)), aligned_b,
+          p->tpix2, p->tcos2, p->tsin2);
   }
   return cudaGetLastError();
 }
@@ -142,6 +151,11 @@ static ColParams make_params(const mm_plan_s* p, const Batch& b, const float* to
   q.tod = tod;
   q.ybuf = ybuf ? ybuf : p->ybuf;
   q.acc = p->acc;
+  q.pix2 = p->tpix2;
+  q.cosw2 = p->tcos2;
+  q.sinw2 = p->tsin2;
+  q.ga = p->gain_a;
+  q.gb = p->gain_b;
   q.acc_stride = acc_stride_of(p->n_pix, p->ncomp);
   return q;
 }
@@ -160,19 +174,12 @@ static cudaError_t col_forward_m1(const mm_plan_s* p, const Batch& b, int src, c
   const size_t smem = sizeof(float2) * ColLayout<CB>::size(M1);
   cudaError_t e;
   int grid = 0;
-  if (src == kSrcTod) {
-    auto k = k_col_forward<M1, CB, kColT, 1, kSrcTod>;
-    if ((e = persistent_grid(k, kColT, smem, ntiles, &grid)) != cudaSuccess) return e;
-    k<<<grid, kColT, smem, st>>>(q);
-  } else if (p->ncomp == 3) {
-    auto k = k_col_forward<M1, CB, kColT, 3, kSrcGather>;
-    if ((e = persistent_grid(k, kColT, smem, ntiles, &grid)) != cudaSuccess) return e;
-    k<<<grid, kColT, smem, st>>>(q);
-  } else {
-    auto k = k_col_forward<M1, CB, kColT, 1, kSrcGather>;
-    if ((e = persistent_grid(k, kColT, smem, ntiles, &grid)) != cudaSuccess) return e;
-    k<<<grid, kColT, smem, st>>>(q);
-  }
+  const bool iqu = p->ncomp == 3;
+  auto k = src == kSrcTod ? k_col_forward<M1, CB, kColT, 1, kSrcTod>
+           : p->composite ? (iqu ? k_col_forward<M1, CB, kColT, 3, kSrcGather2> : k_col_forward<M1, CB, kColT, 1, kSrcGather2>)
+                          : (iqu ? k_col_forward<M1, CB, kColT, 3, kSrcGather> : k_col_forward<M1, CB, kColT, 1, kSrcGather>);
+  if ((e = persistent_grid(k, kColT, smem, ntiles, &grid)) != cudaSuccess) return e;
+  k<<<grid, kColT, smem, st>>>(q);
   return cudaGetLastError();
 }
 
@@ -185,15 +192,11 @@ static cudaError_t col_inverse_m1(const mm_plan_s* p, const Batch& b, cudaStream
   const size_t smem = sizeof(float2) * ColLayout<CB>::size(M1);
   cudaError_t e;
   int grid = 0;
-  if (p->ncomp == 3) {
-    auto k = k_col_inverse<M1, CB, kColT, 3>;
-    if ((e = persistent_grid(k, kColT, smem, ntiles, &grid)) != cudaSuccess) return e;
-    k<<<grid, kColT, smem, st>>>(q);
-  } else {
-    auto k = k_col_inverse<M1, CB, kColT, 1>;
-    if ((e = persistent_grid(k, kColT, smem, ntiles, &grid)) != cudaSuccess) return e;
-    k<<<grid, kColT, smem, st>>>(q);
-  }
+  const bool iqu = p->ncomp == 3;
+  auto k = p->composite ? (iqu ? k_col_inverse<M1, CB, kColT, 3, true> : k_col_inverse<M1, CB, kColT, 1, true>)
+                        : (iqu ? k_col_inverse<M1, CB, kColT, 3, false> : k_col_inverse<M1, CB, kColT, 1, false>);
+  if ((e = persistent_grid(k, kColT, smem, ntiles, &grid)) != cudaSuccess) return e;
+  k<<<grid, kColT, smem, st>>>(q);
   return cudaGetLastError();
 }
 

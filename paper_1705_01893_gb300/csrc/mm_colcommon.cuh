@@ -23,6 +23,11 @@ struct ColParams {
   int count;           // chunks in the batch
   double* acc;         // planar FP64 accumulators: component k of pixel p at k * acc_stride + p
   int64_t acc_stride;  // n_pix
+  // composite pointing (App. B): P = ga P_1 + gb P_2, the second component in tile order too
+  const int32_t* __restrict__ pix2;
+  const void* cosw2;
+  const void* sinw2;
+  float ga, gb;
 };
 
 // The column kernels' parameters for batch b (plan-owned tile-order pointing, map, buffers).
@@ -179,6 +184,22 @@ __device__ __forceinline__ void bin4(double* acc, int64_t acc_stride, int4 p4, f
   if (b2 && l > 2) emit_run<NC>(acc, acc_stride, p[2], v[0][2], v[1][2], v[2][2], pol);
 }
 
+// g_a P_a^T t + g_b P_b^T t for the same samples (App. B).
+template <int NC, int ROWL>
+__device__ __forceinline__ void scatter4_pair(const ColParams& q, int64_t s, float4 t4, int qpos) {
+#pragma unroll 1
+  for (int k = 0; k < 2; ++k) {
+    const float g = k ? q.gb : q.ga;
+    const int4 p4 = __ldcs(reinterpret_cast<const int4*>((k ? q.pix2 : q.pix) + s));
+    float4 c = make_float4(0.f, 0.f, 0.f, 0.f), w = c;
+    if constexpr (NC == 3) {
+      c = load_w4(k ? q.cosw2 : q.cosw, q.half_w, s);
+      w = load_w4(k ? q.sinw2 : q.sinw, q.half_w, s);
+    }
+    bin4<NC, ROWL>(q.acc, q.acc_stride, p4, make_float4(g * t4.x, g * t4.y, g * t4.z, g * t4.w), c, w, qpos);
+  }
+}
+
 template <int NC, int ROWL = 8>
 __device__ __forceinline__ void scatter4(const ColParams& q, int64_t s, float4 t4, int qpos) {
   const int4 p4 = __ldcs(reinterpret_cast<const int4*>(q.pix + s));
@@ -212,6 +233,22 @@ struct SrcGather {   // z = ((P m)_s, (P m)_s+1), Eq. 1; tile-ordered pointing f
       }
     }
     return gather_two<NC>(*q, p.x, p.y, cw0, cw1, sw0, sw1);
+  }
+};
+
+template <int NC, int CB>
+struct SrcGather2 {   // z of g_a P_a m + g_b P_b m (App. B)
+  const ColParams* q;
+  int64_t tbase;
+  __device__ __forceinline__ float2 operator()(int b, int i) const {
+    ColParams second{};
+    second.pix = q->pix2;
+    second.cosw = q->cosw2;
+    second.sinw = q->sinw2;
+    second.half_w = q->half_w;
+    second.map4 = q->map4;
+    const float2 u = SrcGather<NC, CB>{q, tbase}(b, i), v = SrcGather<NC, CB>{&second, tbase}(b, i);
+    return make_float2(fmaf(q->gb, v.x, q->ga * u.x), fmaf(q->gb, v.y, q->ga * u.y));
   }
 };
 

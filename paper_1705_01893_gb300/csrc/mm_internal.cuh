@@ -219,6 +219,9 @@ struct mm_plan_s {
   int32_t* tpix;    // pointing copied into column-tile order (see k_tile_pointing)
   void* tcos;
   void* tsin;
+  int32_t* tpix2;   // the same of a composite plan's second component (compile-time chunks)
+  void* tcos2;
+  void* tsin2;
 };
 
 namespace mm {
@@ -687,7 +690,7 @@ enum RowMode {
   kRowMessengerF = 6, // forward, Y = Nbar X / (lambda tau + Nbar) (the F part, no d~), chi^2
                       // partial sum_k w_k |X_k|^2 / N_k / n, inverse
   kRowMd = 7,         // no forward: Y = lambda tau d~ / (lambda tau + Nbar) (the m_d part), inverse
-  // composite pointing (App. B), general path only:
+  // composite pointing (App. B; run-time instance of the compile-time lengths):
   kRowResidual = 8,   // forward, Y = (d~ - X) / (n (Nbar / lambda + tau)), chi^2, inverse
   // the messenger step that also keeps its forward spectrum X = (P m)~ in row layout at
   // RowArgs::natural + spec (the adjoint's recomputation; run-time instance only)
@@ -711,7 +714,7 @@ struct RowArgs {
 };
 
 // Source of the forward column pass.
-enum ColSrc { kSrcGather = 0, kSrcTod = 1 };
+enum ColSrc { kSrcGather = 0, kSrcTod = 1, kSrcGather2 = 2 /* composite pointing */ };
 
 cudaError_t launch_col_forward(const mm_plan_s* p, const Batch& b, int src, const float* tod,
                                cudaStream_t st);

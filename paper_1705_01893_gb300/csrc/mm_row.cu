@@ -15,7 +15,7 @@ __global__ void __launch_bounds__(T, pass_ctas(T, 12)) k_row(RowParams q) {
   const int njobs = q.count * jobs_pc;
   const int mode = MODE >= 0 ? MODE : q.a.mode;
   const bool reads_d = mode == kRowMessenger || mode == kRowPcgRhs || mode == kRowChi2 ||
-                       mode == kRowPcgApply || mode == kRowMd;
+                       mode == kRowPcgApply || mode == kRowMd || mode == kRowResidual;
   // per-pass twiddles of the row DFT, staged once per CTA after the 2 rows of data
   float2* tws = sm + 2 * M2;
   for (int i = threadIdx.x; i < tw_size(M2); i += T) tws[i] = q.g.tw_row[i];

@@ -89,12 +89,13 @@ __device__ __forceinline__ void kernel_body_job(const RowParams& q, float2* sm, 
   const bool fwd = mode != kRowPcgRhs && mode != kRowMd;
   const bool mess = mode == kRowMessenger || mode == kRowMessengerF || mode == kRowMd ||
                     mode == kRowMessengerKeep;
-  const bool inv = mess || mode == kRowPcgApply || mode == kRowPcgRhs;
+  const bool resid = mode == kRowResidual;
+  const bool inv = mess || resid || mode == kRowPcgApply || mode == kRowPcgRhs;
 
   // The job's constants come from thread 0: FP64 products and conversions in every warp, and a
   // chain of them in thread 0 that all others wait for, held up each job by 2 to 3 of 46
   // thousand cycles.  They are ready by the first barrier of the forward row DFTs.
-  __shared__ float s_con[2];    // tau, lambda tau
+  __shared__ float s_con[3];    // tau, lambda tau, lambda
   double* chi2 = q.a.chi2;
   bool lam_inf = false;
   {
@@ -108,6 +109,7 @@ __device__ __forceinline__ void kernel_body_job(const RowParams& q, float2* sm, 
     if (threadIdx.x == 0) {
       s_con[0] = (float)d.tau;
       s_con[1] = mess && lam_inf ? 0.f : (float)(lambda * d.tau);
+      if (resid) s_con[2] = (float)lambda;
     }
     if (inv) load_row_twiddles<M2, T>(s4, q.g, rA, rB);
     if (!fwd) __syncthreads();
@@ -121,11 +123,12 @@ __device__ __forceinline__ void kernel_body_job(const RowParams& q, float2* sm, 
   // per-mode constants
   const float tau = s_con[0], lt = s_con[1];
   const float inv_n = 1.0f / (float)d.n;
-  if (!mess) lam_inf = false;
+  if (!mess && !resid) lam_inf = false;
   // N' = Nbar + cn for chi^2: tau (Eq. 3) or lambda tau (chi^2(m, lambda))
   const float cn = (mode == kRowChi2 || mode == kRowChi2Modes) ? lt : tau;
   // output scale: irfft normalisation 1/n, and T^-1 = 1/tau for the messenger map step
   const float sc = mess ? inv_n / tau : inv_n;
+  const float lamf = resid && !lam_inf ? s_con[2] : 1.f;
   const float2* dt = q.dtab + d.spec;
   const float* nb = q.nbar + d.spec;
   const float2 wa = __ldg(&q.g.tw_pack_a[rA]);
@@ -137,12 +140,14 @@ __device__ __forceinline__ void kernel_body_job(const RowParams& q, float2* sm, 
       const float r = __fdividef(sc, lt + nbv);
       return make_float2((lt * D.x + nbv * X.x) * r, (lt * D.y + nbv * X.y) * r);
     }
+    if (resid)   // (d~ - X) / (n (Nbar / lambda + tau)); lambda = inf: / (n tau)
+      return cscale(csub(D, X), lam_inf ? __fdividef(sc, tau) : __fdividef(sc, __fdividef(nbv, lamf) + tau));
     if (mode == kRowPcgApply) return cscale(X, __fdividef(sc, nbv + tau));
     return cscale(D, __fdividef(sc, nbv + tau));  // kRowPcgRhs
   };
   const bool want_x2 = chi2 != nullptr &&
                        (mode == kRowMessenger || mode == kRowMessengerF || mode == kRowChi2 ||
-                        mode == kRowChi2Modes ||
+                        mode == kRowChi2Modes || resid ||
                         mode == kRowPcgRhs);
   const bool spec_out = mode == kRowSpectrum || mode == kRowNatural;
   const bool load_d = !spec_out && mode != kRowPcgApply && mode != kRowMessengerF;
