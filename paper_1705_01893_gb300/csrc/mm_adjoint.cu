@@ -78,9 +78,9 @@ __global__ void __launch_bounds__(T, pass_ctas(T, 8)) k_row_adjoint(AdjRowParams
     const float lt = lam_inf ? 0.f : (float)(q.lambda * d.tau);
     const float lam = lam_inf ? 0.f : (float)q.lambda;
     const float sc = 1.0f / ((float)d.n * tau);        // irfft 1/n and T^-1
-    float fk = 1.f, fs = 1.f;
     const bool has_par = THETA && q.params != nullptr;
-    if (has_par) { fk = (float)q.params[4 * c + 1]; fs = (float)q.params[4 * c + 3]; }
+    // f_knee / f = fkn / k
+    const float fkn = has_par ? (float)q.params[4 * c + 1] * (float)d.n / (float)q.params[4 * c + 3] : 1.f;
     const float2* dt = q.dtab + d.spec;
     const float2* rs = THETA ? q.rspec + d.spec : nullptr;
     const float* nb = q.nbar + d.spec;
@@ -99,17 +99,14 @@ __global__ void __launch_bounds__(T, pass_ctas(T, 8)) k_row_adjoint(AdjRowParams
         Tm = D;
         Y = make_float2(0.f, 0.f);
       } else {
-        const float den = lt + nbv;
-        const float a = lt / den, b = nbv / den;
+        const float inv = 1.0f / (lt + nbv);
+        const float a = lt * inv, b = nbv * inv;
         Tm = make_float2(a * D.x + b * R.x, a * D.y + b * R.y);
         const float c1 = V.x * (R.x - D.x) + V.y * (R.y - D.y);   // Re(conj V (R - D))
-        const float g1 = lt * nbv / (den * den);
+        const float g1 = a * b;
         s0 += wt * c1 * g1;
-        if (has_par) {
-          const float f = (kk == 0 ? 1.f : (float)kk) * fs / (float)d.n;
-          sal += wt * c1 * g1 * logf(fk / f);
-        }
-        stau -= wt * c1 * lam * nbv / (den * den);
+        if (has_par) sal += wt * c1 * g1 * logf(fkn / (kk == 0 ? 1.f : (float)kk));   // ln(f_knee / f)
+        stau -= wt * c1 * lam * (b * inv);
         Y = make_float2(b * V.x * sc, b * V.y * sc);
       }
       sT += wt * (V.x * Tm.x + V.y * Tm.y);
@@ -257,39 +254,49 @@ __global__ void __launch_bounds__(T, pass_ctas(T, 8)) k_col_inverse_adjoint(ColP
   }
 }
 
-// u = W gbar (FP32 copy for the gathers), and FP32 copies of m and m'.
+// u = W gbar (FP32 copy for the gathers) and, for the theta terms, an FP32 copy of m' (mp).  gbar
+// comes from the caller (g) or, from the second transposed step on, from the accumulators: the
+// binned adjoint on kept pixels, cleared for the next pass.
 template <int NC>
 __global__ void k_adj_prep(int64_t n_pix, const double* __restrict__ W, const double* __restrict__ g,
-                           const double* __restrict__ m, const double* __restrict__ mp,
-                           const uint8_t* __restrict__ valid, void* u4, void* m4, void* mp4) {
+                           double* __restrict__ acc, const double* __restrict__ mp,
+                           const uint8_t* __restrict__ valid, void* u4, void* mp4) {
   const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (p >= n_pix) return;
-  constexpr int B = NC == 3 ? 6 : 1;
   const bool ok = valid[p] != 0;
   double a[NC], u[NC];
+  if (g) {
 #pragma unroll
-  for (int i = 0; i < NC; ++i) a[i] = g[NC * p + i];
-  const double* w = W + B * p;
-  if constexpr (NC == 1) {
-    u[0] = w[0] * a[0];
-    reinterpret_cast<float*>(u4)[p] = (float)u[0];
-    reinterpret_cast<float*>(m4)[p] = ok ? (float)m[p] : 0.f;
-    reinterpret_cast<float*>(mp4)[p] = ok ? (float)mp[p] : 0.f;
+    for (int i = 0; i < NC; ++i) a[i] = g[NC * p + i];
   } else {
+    take_acc<NC>(acc, n_pix, p, a);
+#pragma unroll
+    for (int i = 0; i < NC; ++i) a[i] = ok ? a[i] : 0.0;
+  }
+  if constexpr (NC == 1) {
+    u[0] = W[p] * a[0];
+    reinterpret_cast<float*>(u4)[p] = (float)u[0];
+    if (mp) reinterpret_cast<float*>(mp4)[p] = ok ? (float)mp[p] : 0.f;
+  } else {
+    double w[6];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const double2 v = reinterpret_cast<const double2*>(W + 6 * p)[i];
+      w[2 * i] = v.x;
+      w[2 * i + 1] = v.y;
+    }
     u[0] = w[0] * a[0] + w[1] * a[1] + w[2] * a[2];
     u[1] = w[1] * a[0] + w[3] * a[1] + w[4] * a[2];
     u[2] = w[2] * a[0] + w[4] * a[1] + w[5] * a[2];
     reinterpret_cast<float4*>(u4)[p] = make_float4((float)u[0], (float)u[1], (float)u[2], 0.f);
-    reinterpret_cast<float4*>(m4)[p] =
-        ok ? make_float4((float)m[3 * p], (float)m[3 * p + 1], (float)m[3 * p + 2], 0.f)
-           : make_float4(0.f, 0.f, 0.f, 0.f);
-    reinterpret_cast<float4*>(mp4)[p] =
-        ok ? make_float4((float)mp[3 * p], (float)mp[3 * p + 1], (float)mp[3 * p + 2], 0.f)
-           : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (mp)
+      reinterpret_cast<float4*>(mp4)[p] =
+          ok ? make_float4((float)mp[3 * p], (float)mp[3 * p + 1], (float)mp[3 * p + 2], 0.f)
+             : make_float4(0.f, 0.f, 0.f, 0.f);
   }
 }
 
-// gbar for the previous step: the binned adjoint, on kept pixels; clears the accumulators.
+// gbar for the next segment's first transposed step, out of the way of the recomputation's sums.
 template <int NC>
 __global__ void k_adj_take_g(int64_t n_pix, double* __restrict__ acc, const uint8_t* __restrict__ valid,
                              double* __restrict__ g) {
@@ -426,7 +433,7 @@ using namespace mm;
 static size_t up256(size_t x) { return (x + 255) & ~size_t(255); }
 
 struct AdjLayout {
-  size_t ckpt, seg, g, u4, m4, mp4, keep, acc, total;
+  size_t ckpt, seg, g, u4, mp4, keep, acc, total;
   int nseg;
 };
 
@@ -441,7 +448,6 @@ static AdjLayout adj_layout(const mm_plan_s* p, int n_iter, int every) {
   L.seg = take(map * (size_t)(every + 1));
   L.g = take(map);
   L.u4 = take(m4);
-  L.m4 = take(m4);
   L.mp4 = take(m4);
   // forward spectra (P m_i)~ of one segment's iterations, row layout, for the theta sums
   L.keep = take(sizeof(float2) * (size_t)p->spec_total * (size_t)every);
@@ -522,9 +528,8 @@ static mm_status adjoint_backward(mm_plan p, const double* lambdas, int n_iter,
                                   const AdjLayout& L, char* w, cudaStream_t s) {
   const size_t mapb = sizeof(double) * p->ncomp * (size_t)p->n_pix;
   double* seg = reinterpret_cast<double*>(w + L.seg);
-  double* g = reinterpret_cast<double*>(w + L.g);
+  double* gbuf = reinterpret_cast<double*>(w + L.g);
   void* u4 = w + L.u4;
-  void* m4 = w + L.m4;
   void* mp4 = w + L.mp4;
   float2* keep = reinterpret_cast<float2*>(w + L.keep);
   const size_t kstride = (size_t)p->spec_total;
@@ -533,17 +538,16 @@ static mm_status adjoint_backward(mm_plan p, const double* lambdas, int n_iter,
   const size_t mstride = (size_t)len;
   const bool theta = grad_theta != nullptr;
 
-  ADJ_CUDA(cudaMemcpyAsync(g, grad_map_out, mapb, cudaMemcpyDeviceToDevice, s));
   ADJ_CUDA(cudaMemsetAsync(grad_tod, 0, sizeof(float) * (size_t)p->n_total, s));
   ADJ_CUDA(cudaMemsetAsync(acc, 0, sizeof(double) * kAdjN * p->n_chunks, s));
   const unsigned nbp = (unsigned)((p->n_pix + 255) / 256);
-  // transposed step i (mi = m_i, mo = m_{i+1}, rs = (P m_i)~: read only for the theta terms)
-  auto step = [&](int i, const double* mi, const double* mo, const float2* rs) -> mm_status {
-    if (p->ncomp == 3)
-      k_adj_prep<3><<<nbp, 256, 0, s>>>(p->n_pix, p->W, g, mi, mo, p->valid, u4, m4, mp4);
-    else
-      k_adj_prep<1><<<nbp, 256, 0, s>>>(p->n_pix, p->W, g, mi, mo, p->valid, u4, m4, mp4);
+  // transposed step i (mo = m_{i+1}, rs = (P m_i)~: read only for the theta terms)
+  const double* g = grad_map_out;   // NULL: the previous step's sums in the accumulators
+  auto step = [&](int i, const double* mo, const float2* rs) -> mm_status {
+    if (p->ncomp == 3) k_adj_prep<3><<<nbp, 256, 0, s>>>(p->n_pix, p->W, g, p->acc, mo, p->valid, u4, mp4);
+    else k_adj_prep<1><<<nbp, 256, 0, s>>>(p->n_pix, p->W, g, p->acc, mo, p->valid, u4, mp4);
     ADJ_CUDA(cudaGetLastError());
+    g = nullptr;
     const AdjColExtra x{u4, mp4, grad_tod, acc};
     for (int b = 0; b < p->n_batches; ++b) {
       const Batch& B = p->h_batches[b];
@@ -551,35 +555,42 @@ static mm_status adjoint_backward(mm_plan p, const double* lambdas, int n_iter,
       ADJ_CUDA(launch_row_adjoint(p, B, p->ybuf, theta ? rs : nullptr, lambdas[i], acc, s));
       ADJ_CUDA(launch_col_adjoint(p, B, x, theta, s));
     }
-    if (p->ncomp == 3) k_adj_take_g<3><<<nbp, 256, 0, s>>>(p->n_pix, p->acc, p->valid, g);
-    else k_adj_take_g<1><<<nbp, 256, 0, s>>>(p->n_pix, p->acc, p->valid, g);
-    ADJ_CUDA(cudaGetLastError());
+    return MM_OK;
+  };
+  // the last transposed step's sums (the gradient for the first map) are not asked for
+  auto finish = [&]() -> mm_status {
+    ADJ_CUDA(cudaMemsetAsync(p->acc, 0, sizeof(double) * p->ncomp * acc_stride_of(p->n_pix, p->ncomp), s));
     return MM_OK;
   };
   if (!theta) {
     // with lambda held constant the step is affine in (m, d): its transpose does not depend
     // on the iterates, so no checkpoint is read and nothing is recomputed
     for (int i = n_iter - 1; i >= 0; --i) {
-      mm_status st = step(i, g, g, nullptr);
+      mm_status st = step(i, nullptr, nullptr);
       if (st != MM_OK) return st;
     }
-    return MM_OK;
+    return finish();
   }
   for (int sg = L.nseg - 1; sg >= 0; --sg) {
     const int i0 = sg * ckpt_every;
     const int i1 = i0 + ckpt_every < n_iter ? i0 + ckpt_every : n_iter;
     ADJ_CUDA(cudaMemcpyAsync(seg, ckpt + sg * mstride, mapb, cudaMemcpyDeviceToDevice, s));
     for (int i = i0; i < i1; ++i) {
-      // recompute m_{i+1} from m_i, keeping the forward spectrum (P m_i)~
-      double* nxt = seg + (i - i0 + 1) * mstride;
-      ADJ_CUDA(cudaMemcpyAsync(nxt, seg + (i - i0) * mstride, mapb, cudaMemcpyDeviceToDevice, s));
-      mm_status st = messenger_step_keep(p, lambdas[i], nxt, keep + (i - i0) * kstride, s);
+      // recompute m_{i+1} from m_i, keeping the forward spectrum (P m_i)~; m_i is in map4 already
+      // after the first step of a segment
+      mm_status st = messenger_step_keep(p, lambdas[i], i == i0 ? seg : nullptr, seg + (i - i0 + 1) * mstride,
+                                         keep + (i - i0) * kstride, s);
       if (st != MM_OK) return st;
     }
     for (int i = i1 - 1; i >= i0; --i) {
-      mm_status st = step(i, seg + (i - i0) * mstride, seg + (i - i0 + 1) * mstride,
-                          keep + (i - i0) * kstride);
+      mm_status st = step(i, seg + (i - i0 + 1) * mstride, keep + (i - i0) * kstride);
       if (st != MM_OK) return st;
+    }
+    if (sg > 0) {
+      if (p->ncomp == 3) k_adj_take_g<3><<<nbp, 256, 0, s>>>(p->n_pix, p->acc, p->valid, gbuf);
+      else k_adj_take_g<1><<<nbp, 256, 0, s>>>(p->n_pix, p->acc, p->valid, gbuf);
+      ADJ_CUDA(cudaGetLastError());
+      g = gbuf;
     }
   }
   if (theta) {
@@ -587,7 +598,7 @@ static mm_status adjoint_backward(mm_plan p, const double* lambdas, int n_iter,
                                                         grad_theta);
     ADJ_CUDA(cudaGetLastError());
   }
-  return MM_OK;
+  return finish();
 }
 
 static mm_status adjoint_outputs_check(mm_plan p, const double* grad_map_out,

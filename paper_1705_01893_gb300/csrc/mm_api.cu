@@ -814,6 +814,22 @@ __device__ __forceinline__ void sym_apply(const double* W, const double* a, doub
   }
 }
 
+// A pixel's symmetric block, 48 bytes as three 16-byte loads (IQU).
+template <int NC>
+__device__ __forceinline__ void load_block(const double* __restrict__ W, int64_t p, double* w) {
+  if constexpr (NC == 1) {
+    w[0] = W[p];
+  } else {
+    const double2* q = reinterpret_cast<const double2*>(W + 6 * p);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const double2 v = q[i];
+      w[2 * i] = v.x;
+      w[2 * i + 1] = v.y;
+    }
+  }
+}
+
 template <int NC>
 __device__ __forceinline__ void store_map4(void* map4, int64_t p, const double* m) {
   if constexpr (NC == 1) reinterpret_cast<float*>(map4)[p] = (float)m[0];
@@ -830,8 +846,7 @@ __global__ void k_bin_apply(int64_t n_pix, double* __restrict__ acc, const doubl
   constexpr int B = NC == 3 ? 6 : 1;
   double a[NC], w[B], m[NC];
   take_acc<NC>(acc, n_pix, p, a);
-#pragma unroll
-  for (int i = 0; i < B; ++i) w[i] = W[B * p + i];
+  load_block<NC>(W, p, w);
   sym_apply<NC>(w, a, m);
   store_map4<NC>(map4, p, m);
   if (map_out)
@@ -850,8 +865,7 @@ __global__ void k_bin_resid(int64_t n_pix, double* __restrict__ acc, const doubl
   constexpr int B = NC == 3 ? 6 : 1;
   double a[NC], w[B], u[NC], m[NC];
   take_acc<NC>(acc, n_pix, p, a);
-#pragma unroll
-  for (int i = 0; i < B; ++i) w[i] = W[B * p + i];
+  load_block<NC>(W, p, w);
   sym_apply<NC>(w, a, u);
 #pragma unroll
   for (int i = 0; i < NC; ++i) { m[i] = m64[NC * p + i] + u[i]; m64[NC * p + i] = m[i]; }
@@ -970,8 +984,7 @@ __device__ __forceinline__ void block_apply(const double* Minv, int64_t pixel, c
                                             double* z) {
   constexpr int B = NC == 3 ? 6 : 1;
   double w[B];
-#pragma unroll
-  for (int i = 0; i < B; ++i) w[i] = Minv[B * pixel + i];
+  load_block<NC>(Minv, pixel, w);
   sym_apply<NC>(w, r, z);
 }
 
@@ -1082,12 +1095,12 @@ __global__ void k_pcg_update(int64_t n_pix, double* __restrict__ x, double* __re
   }
 }
 
-// beta = rz_next / rz_cur; p = z + beta p; map4 = p; pq cleared by the next k_pcg_q's
-// predecessor (this kernel's last block is not known, so pq is reset by the driver).
+// beta = rz_next / rz_cur; p = z + beta p; map4 = p; p.q cleared for the next iteration.
 template <int NC>
 __global__ void k_pcg_dir(int64_t n_pix, const double* __restrict__ z, double* __restrict__ pv,
-                          void* map4, const double* sc, int rz_cur, int rz_next) {
+                          void* map4, double* sc, int rz_cur, int rz_next) {
   const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (p == 0) sc[kPcgPq] = 0.0;   // read by the update kernel before, added to by the next q kernel
   if (p >= n_pix) return;
   const double beta = sc[rz_next] / sc[rz_cur];
   double m[NC];
@@ -1763,15 +1776,17 @@ extern "C" mm_status mm_messenger_iterate(mm_plan p, const double* lambdas, int 
   return check_waits(p, s, "mm_messenger_iterate");
 }
 
-mm_status mm::messenger_step_keep(mm_plan_s* p, double lambda, double* map_inout, float2* keep,
-                                  cudaStream_t s) {
-  mm_status st = load_map(p, map_inout, s);
-  if (st != MM_OK) return st;
+mm_status mm::messenger_step_keep(mm_plan_s* p, double lambda, const double* map_in, double* map_out,
+                                  float2* keep, cudaStream_t s) {
+  if (map_in) {
+    mm_status st = load_map(p, map_in, s);
+    if (st != MM_OK) return st;
+  }
   RowArgs a{kRowMessengerKeep, lambda, nullptr, keep};
   FOR_BATCHES(L_(launch_col_forward(p, B, kSrcGather, nullptr, s)); L_(launch_row(p, B, a, s));
               L_(launch_col_inverse(p, B, s)));
-  if (p->ncomp == 3) k_bin_apply<3><<<blocks_for(p->n_pix, 256), 256, 0, s>>>(p->n_pix, p->acc, p->W, p->map4, map_inout);
-  else k_bin_apply<1><<<blocks_for(p->n_pix, 256), 256, 0, s>>>(p->n_pix, p->acc, p->W, p->map4, map_inout);
+  if (p->ncomp == 3) k_bin_apply<3><<<blocks_for(p->n_pix, 256), 256, 0, s>>>(p->n_pix, p->acc, p->W, p->map4, map_out);
+  else k_bin_apply<1><<<blocks_for(p->n_pix, 256), 256, 0, s>>>(p->n_pix, p->acc, p->W, p->map4, map_out);
   LAUNCHED("k_bin_apply");
   return MM_OK;
 }
@@ -1800,8 +1815,7 @@ __global__ void k_bin_md(int64_t n_pix, double* __restrict__ acc, const double* 
     constexpr int B = NC == 3 ? 6 : 1;
     double a[NC], w[B], m[NC];
     take_acc<NC>(acc, n_pix, p, a);
-#pragma unroll
-    for (int i = 0; i < B; ++i) w[i] = W[B * p + i];
+    load_block<NC>(W, p, w);
     sym_apply<NC>(w, a, m);
     if (md)
 #pragma unroll
@@ -2038,7 +2052,7 @@ extern "C" mm_status mm_messenger_stage(mm_plan p, int stage, int batch, double 
 // graph whose cooling parameter and chi^2 slot come from device memory.
 // The kernels of one graph-mode iteration (lambda and the chi^2 slot from device memory,
 // the iteration counter advanced by the map step) launched on s.
-static cudaError_t launch_iteration(mm_plan p, cudaStream_t s) {
+static cudaError_t launch_iteration(mm_plan p, double* map_out, cudaStream_t s) {
   RowArgs a{kRowMessenger, 1.0, nullptr, nullptr};
   a.lam_table = p->lam_table;
   a.iter = p->iter;
@@ -2056,9 +2070,9 @@ static cudaError_t launch_iteration(mm_plan p, cudaStream_t s) {
   }
   if (e != cudaSuccess) return e;
   if (p->ncomp == 3)
-    k_bin_apply<3><<<blocks_for(p->n_pix, 256), 256, 0, s>>>(p->n_pix, p->acc, p->W, p->map4, p->map64, p->iter);
+    k_bin_apply<3><<<blocks_for(p->n_pix, 256), 256, 0, s>>>(p->n_pix, p->acc, p->W, p->map4, map_out, p->iter);
   else
-    k_bin_apply<1><<<blocks_for(p->n_pix, 256), 256, 0, s>>>(p->n_pix, p->acc, p->W, p->map4, p->map64, p->iter);
+    k_bin_apply<1><<<blocks_for(p->n_pix, 256), 256, 0, s>>>(p->n_pix, p->acc, p->W, p->map4, map_out, p->iter);
   return cudaGetLastError();
 }
 
@@ -2069,7 +2083,7 @@ static mm_status capture_iteration_graph(mm_plan p) {
   cudaStream_t s = p->graph_stream;
   // relaxed: the launchers may query occupancy / set kernel attributes on first use
   MM_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeRelaxed));
-  cudaError_t e = launch_iteration(p, s);
+  cudaError_t e = launch_iteration(p, nullptr, s);
   cudaGraph_t graph = nullptr;
   const cudaError_t ec = cudaStreamEndCapture(s, &graph);
   if (e != cudaSuccess || ec != cudaSuccess) {
@@ -2151,7 +2165,7 @@ static mm_status build_adaptive_graph(mm_plan p) {
     cudaGraph_t body = np.conditional.phGraph_out[0];
     e = cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
     if (e == cudaSuccess) {
-      cudaError_t el = launch_iteration(p, s);
+      cudaError_t el = launch_iteration(p, p->map64, s);
       if (el == cudaSuccess) {
         k_adapt<<<1, 32, 0, s>>>(static_cast<AdaptState*>(p->adapt_st), p->lam_table, p->iter, h);
         el = cudaGetLastError();
@@ -2254,9 +2268,10 @@ extern "C" mm_status mm_messenger_graph(mm_plan p, const double* lambdas, int n_
   if (chi2_out) MM_CUDA(cudaMemsetAsync(chi2_out, 0, sizeof(double) * n_iter, s));
   st = load_map(p, map_inout, s);
   if (st != MM_OK) return st;
-  for (int it = 0; it < n_iter; ++it) MM_CUDA(cudaGraphLaunch(p->graph_exec, s));
-  MM_CUDA(cudaMemcpyAsync(map_inout, p->map64, sizeof(double) * p->ncomp * p->n_pix,
-                          cudaMemcpyDeviceToDevice, s));
+  // the last iteration is launched by itself: only it writes the FP64 map (24 of the 136 bytes
+  // per pixel that the map step moves), straight into the caller's
+  for (int it = 0; it + 1 < n_iter; ++it) MM_CUDA(cudaGraphLaunch(p->graph_exec, s));
+  MM_CUDA(launch_iteration(p, map_inout, s));
   return check_waits(p, s, "mm_messenger_graph");
 }
 
@@ -2309,13 +2324,13 @@ extern "C" mm_status mm_pcg_iterate(mm_plan p, int n_iter, double* map_inout, vo
     else k_map_to4<1><<<nb, 256, 0, s>>>(p->n_pix, pv, p->valid, p->map4);
     LAUNCHED("k_map_to4");
   }
+  // the two r.z slots change places every iteration; a call begins and ends with the current one
+  // in slot 0 (one copy after an odd number, instead of a copy and a clear each iteration)
+  MM_CUDA(cudaMemsetAsync(sc + kPcgPq, 0, sizeof(double), s));
   for (int it = 0; it < n_iter; ++it) {
-    // the parity of rz slots is kept in scalar slot 7 across calls
-    MM_CUDA(cudaMemsetAsync(sc + kPcgPq, 0, sizeof(double), s));
     mm_status st = apply_A(p, s);
     if (st != MM_OK) return st;
-    int cur = kPcgRz0, nxt = kPcgRz1;
-    // parity bookkeeping on the host: each call restarts parity at slot 0 after copying
+    const int cur = it & 1 ? kPcgRz1 : kPcgRz0, nxt = it & 1 ? kPcgRz0 : kPcgRz1;
     double* slot = chi2_out ? chi2_out + it : nullptr;
     if (tri) k_pcg_q<3><<<nb, 256, 0, s>>>(p->n_pix, p->acc, p->valid, pv, q, sc, nxt, p->scal + kScalCdd, slot);
     else k_pcg_q<1><<<nb, 256, 0, s>>>(p->n_pix, p->acc, p->valid, pv, q, sc, nxt, p->scal + kScalCdd, slot);
@@ -2326,9 +2341,9 @@ extern "C" mm_status mm_pcg_iterate(mm_plan p, int n_iter, double* map_inout, vo
     if (tri) k_pcg_dir<3><<<nb, 256, 0, s>>>(p->n_pix, z, pv, p->map4, sc, cur, nxt);
     else k_pcg_dir<1><<<nb, 256, 0, s>>>(p->n_pix, z, pv, p->map4, sc, cur, nxt);
     LAUNCHED("k_pcg_dir");
-    // rz_cur <- rz_next for the next iteration
-    MM_CUDA(cudaMemcpyAsync(sc + kPcgRz0, sc + kPcgRz1, sizeof(double), cudaMemcpyDeviceToDevice, s));
   }
+  if (n_iter & 1)
+    MM_CUDA(cudaMemcpyAsync(sc + kPcgRz0, sc + kPcgRz1, sizeof(double), cudaMemcpyDeviceToDevice, s));
   return check_waits(p, s, "mm_pcg_iterate");
 }
 

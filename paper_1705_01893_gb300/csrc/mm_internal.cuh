@@ -719,10 +719,11 @@ enum ColSrc { kSrcGather = 0, kSrcTod = 1, kSrcGather2 = 2 /* composite pointing
 cudaError_t launch_col_forward(const mm_plan_s* p, const Batch& b, int src, const float* tod,
                                cudaStream_t st);
 cudaError_t launch_row(const mm_plan_s* p, const Batch& b, const RowArgs& a, cudaStream_t st);
-// One messenger iteration on map_inout (as mm_messenger_iterate) that also keeps each
-// chunk's forward spectrum (P m)~ in row layout at keep + ChunkDesc::spec (mm_api.cu).
-mm_status messenger_step_keep(mm_plan_s* p, double lambda, double* map_inout, float2* keep,
-                              cudaStream_t s);
+// One messenger iteration from map_in (NULL: from the map that the previous one left in map4) to
+// map_out that also keeps each chunk's forward spectrum (P m)~ in row layout at keep +
+// ChunkDesc::spec (mm_api.cu).
+mm_status messenger_step_keep(mm_plan_s* p, double lambda, const double* map_in, double* map_out,
+                              float2* keep, cudaStream_t s);
 // Fused A + B + C launch of one batch's messenger iteration (mm_fused.cu).
 bool fused_eligible(const mm_plan_s* p, const Batch& b);
 int fused_items_per_chunk(int M1, int M2, bool general);
