@@ -385,15 +385,51 @@ __device__ __forceinline__ void gen_gather_tile(const GenParams& q, const GenChu
   }
 }
 
+// The column kernels' current and next tile: table entry and chunk record in shared memory,
+// fetched piece by piece by warp 0 while the current tile is worked on, so that no tile starts
+// with the chain of dependent loads (64 uneven chunks: forward columns 195 -> 178 us).
+struct TileFeed {
+  int2 item[2];
+  GenChunk rec[2];
+};
+__device__ __forceinline__ void feed_words(const GenChunk* src, int lane, int* w) {
+  constexpr int kWords = sizeof(GenChunk) / 4;
+  static_assert(sizeof(GenChunk) % 4 == 0 && kWords <= 4 * 32, "at most four words a lane");
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    w[k] = lane + 32 * k < kWords ? __ldg(reinterpret_cast<const int*>(src) + lane + 32 * k) : 0;
+}
+__device__ __forceinline__ void feed_put(GenChunk* dst, int lane, const int* w) {
+  constexpr int kWords = sizeof(GenChunk) / 4;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    if (lane + 32 * k < kWords) reinterpret_cast<int*>(dst)[lane + 32 * k] = w[k];
+}
+
 // ------------------------------------------------------------ kernel A: columns forward
 template <int NC, int SRC>
 __global__ void __launch_bounds__(512, 2) k_gen_col_forward(GenParams q) {
   extern __shared__ float2 gsm[];
   const int T = blockDim.x, NB = q.nb, lnb = NB == 16 ? 4 : 3;
-  for (int64_t t = blockIdx.x; t < q.n_items; t += gridDim.x) {
-    const int2 it = __ldg(q.items + q.base + t);
-    const GenChunk& G = q.rec[it.x];
-    const ChunkDesc d = G.d;
+  __shared__ TileFeed feed;
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x < 32 && blockIdx.x < q.n_items) {
+    const int2 it0 = __ldg(q.items + q.base + blockIdx.x);
+    int w[4];
+    feed_words(q.rec + it0.x, lane, w);
+    feed_put(&feed.rec[0], lane, w);
+    feed.item[0] = it0;
+  }
+  __syncthreads();
+  int cur = 0;
+  for (int64_t t = blockIdx.x; t < q.n_items; t += gridDim.x, cur ^= 1) {
+    const int2 it = feed.item[cur];
+    const GenChunk& G = feed.rec[cur];
+    const ChunkDesc& d = G.d;
+    const bool more = threadIdx.x < 32 && t + gridDim.x < q.n_items;
+    int2 nit = make_int2(0, 0);
+    int nw[4];
+    if (more) nit = __ldg(q.items + q.base + t + gridDim.x);
     const int M1 = d.M1, M2 = d.M2;
     const int j2_0 = it.y;
     const int width = min(NB, M2 - j2_0);
@@ -416,7 +452,12 @@ __global__ void __launch_bounds__(512, 2) k_gen_col_forward(GenParams q) {
       }
       a[e] = z;
     }
+    if (more) feed_words(q.rec + nit.x, lane, nw);
     __syncthreads();
+    if (more) {
+      feed_put(&feed.rec[cur ^ 1], lane, nw);
+      feed.item[cur ^ 1] = nit;
+    }
     const ColIO io{q.ybuf + (G.yoff - q.base_y), &G, M2, j2_0, width};
     if constexpr (SRC == kSrcTod)   // the data keep their own plan (see radix_plan)
       gen_dft_cols<-1, kSmem, kGlobal>(a, b, M1, G.nr1d, G.rad1d, G.tw_col_d, NB, lnb, T, io);
@@ -535,10 +576,25 @@ template <int NC>
 __global__ void __launch_bounds__(512, 2) k_gen_col_inverse(GenParams q) {
   extern __shared__ float2 gsm[];
   const int T = blockDim.x, NB = q.nb, lnb = NB == 16 ? 4 : 3;
-  for (int64_t t = blockIdx.x; t < q.n_items; t += gridDim.x) {
-    const int2 it = __ldg(q.items + q.base + t);
-    const GenChunk& G = q.rec[it.x];
-    const ChunkDesc d = G.d;
+  __shared__ TileFeed feed;
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x < 32 && blockIdx.x < q.n_items) {
+    const int2 it0 = __ldg(q.items + q.base + blockIdx.x);
+    int w[4];
+    feed_words(q.rec + it0.x, lane, w);
+    feed_put(&feed.rec[0], lane, w);
+    feed.item[0] = it0;
+  }
+  __syncthreads();
+  int cur = 0;
+  for (int64_t t = blockIdx.x; t < q.n_items; t += gridDim.x, cur ^= 1) {
+    const int2 it = feed.item[cur];
+    const GenChunk& G = feed.rec[cur];
+    const ChunkDesc& d = G.d;
+    const bool more = threadIdx.x < 32 && t + gridDim.x < q.n_items;
+    int2 nit = make_int2(0, 0);
+    int nw[4];
+    if (more) nit = __ldg(q.items + q.base + t + gridDim.x);
     const int M1 = d.M1, M2 = d.M2;
     const int j2_0 = it.y;
     const int width = min(NB, M2 - j2_0);
@@ -546,6 +602,7 @@ __global__ void __launch_bounds__(512, 2) k_gen_col_inverse(GenParams q) {
     float2* b = gsm + M1 * NB;
     const ColIO io{q.ybuf + (G.yoff - q.base_y), &G, M2, j2_0, width};
     const float2* r = gen_dft_cols<+1, kGlobal, kSmem>(a, b, M1, G.nr1, G.rad1, G.tw_col, NB, lnb, T, io);
+    if (more) feed_words(q.rec + nit.x, lane, nw);
     const float* rf = reinterpret_cast<const float*>(r);
     if (!q.composite) {
       if (width == NB && !d.cplx) {
@@ -558,6 +615,10 @@ __global__ void __launch_bounds__(512, 2) k_gen_col_inverse(GenParams q) {
     } else {   // P^T t = g_a P_a^T t + g_b P_b^T t (App. B), natural-order pointing
       gen_scatter<NC>(q, d, 0, j2_0, width, rf, NB, lnb, T, q.pix, q.cosw, q.sinw, q.ga, false);
       gen_scatter<NC>(q, d, 0, j2_0, width, rf, NB, lnb, T, q.pix2, q.cos2, q.sin2, q.gb, false);
+    }
+    if (more) {
+      feed_put(&feed.rec[cur ^ 1], lane, nw);
+      feed.item[cur ^ 1] = nit;
     }
     __syncthreads();
   }
@@ -577,7 +638,6 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1) k_gen_row(GenParams
   // the current job and the next one: table entry, chunk record, tau, lambda tau, output scale.
   // Warp 0 fetches the next ones piece by piece between its passes, so that no job starts with
   // the chain of dependent loads (6 of 37 thousand cycles a job).
-  static_assert(sizeof(GenChunk) % 4 == 0 && sizeof(GenChunk) <= 4 * 32 * 4, "at most four words a lane");
   __shared__ GenChunk s_rec[2];
   __shared__ int4 s_job[2];
   __shared__ float s_con[2][3];
@@ -601,13 +661,10 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1) k_gen_row(GenParams
                         mode == kRowPcgRhs || mode == kRowResidual);
   const bool lam_inf = (__double2hiint(lambda) & 0x7fffffff) == 0x7ff00000;
   const int lane = threadIdx.x & 31;
-  constexpr int kWords = sizeof(GenChunk) / 4;
   // warp 0: the record and constants of job `nj` into slot s
   auto put = [&](int s, int4 nj, const int* w) {
     s_job[s] = nj;
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (lane + 32 * k < kWords) reinterpret_cast<int*>(&s_rec[s])[lane + 32 * k] = w[k];
+    feed_put(&s_rec[s], lane, w);
     __syncwarp();
     if (lane == 0) {
       const float tau = (float)s_rec[s].d.tau, inv_n = 1.0f / (float)s_rec[s].d.n;
@@ -616,11 +673,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1) k_gen_row(GenParams
       s_con[s][2] = mess ? inv_n / tau : inv_n;
     }
   };
-  auto fetch = [&](int4 nj, int* w) {
-    const int* src = reinterpret_cast<const int*>(q.rec + nj.x);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) w[k] = lane + 32 * k < kWords ? __ldg(src + lane + 32 * k) : 0;
-  };
+  auto fetch = [&](int4 nj, int* w) { feed_words(q.rec + nj.x, lane, w); };
   if (threadIdx.x < 32 && blockIdx.x < q.n_items) {
     const int4 j0 = __ldg(q.jobs + q.base + blockIdx.x);
     int w[4];
