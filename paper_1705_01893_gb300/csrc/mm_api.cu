@@ -836,22 +836,39 @@ __device__ __forceinline__ void store_map4(void* map4, int64_t p, const double* 
   else reinterpret_cast<float4*>(map4)[p] = make_float4((float)m[0], (float)m[1], (float)m[2], 0.f);
 }
 
-// m = (P^T T^-1 P)^-1 acc (the map step of Sec. 2.1); acc is cleared for the next pass.
-template <int NC>
-__global__ void k_bin_apply(int64_t n_pix, double* __restrict__ acc, const double* __restrict__ W,
-                            void* map4, double* __restrict__ map_out, int* iter = nullptr) {
-  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (iter && p == 0) *iter += 1;   // graph mode: next iteration of the schedule
-  if (p >= n_pix) return;
+// m = (P^T T^-1 P)^-1 acc (the map step of Sec. 2.1); acc is cleared for the next pass.  U pixels a
+// thread, every load before the first store: with the loads of a pixel's three sums between the
+// stores that clear them, 4 M pixels took 245 us (302 with the FP64 map written); all loads first
+// 170 (210), two pixels a thread 95 (97), near the 80 us of their FP64 instructions.
+template <int NC, int U>
+__global__ void __launch_bounds__(256) k_bin_apply(int64_t n_pix, double* __restrict__ acc,
+                                                   const double* __restrict__ W, void* map4,
+                                                   double* __restrict__ map_out, int* iter) {
   constexpr int B = NC == 3 ? 6 : 1;
-  double a[NC], w[B], m[NC];
-  take_acc<NC>(acc, n_pix, p, a);
-  load_block<NC>(W, p, w);
-  sym_apply<NC>(w, a, m);
-  store_map4<NC>(map4, p, m);
-  if (map_out)
+  const int64_t p0 = blockIdx.x * (int64_t)(256 * U) + threadIdx.x;
+  if (iter && p0 == 0) *iter += 1;   // graph mode: next iteration of the schedule
+  double a[U][NC], w[U][B];
 #pragma unroll
-    for (int i = 0; i < NC; ++i) map_out[NC * p + i] = m[i];
+  for (int u = 0; u < U; ++u) {
+    const int64_t p = p0 + 256 * u;
+    if (p >= n_pix) continue;
+#pragma unroll
+    for (int i = 0; i < NC; ++i) a[u][i] = __ldcs(acc + i * acc_stride_of(n_pix, NC) + p);
+    load_block<NC>(W, p, w[u]);
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int64_t p = p0 + 256 * u;
+    if (p >= n_pix) continue;
+#pragma unroll
+    for (int i = 0; i < NC; ++i) acc[i * acc_stride_of(n_pix, NC) + p] = 0.0;
+    double m[NC];
+    sym_apply<NC>(w[u], a[u], m);
+    store_map4<NC>(map4, p, m);
+    if (map_out)
+#pragma unroll
+      for (int i = 0; i < NC; ++i) map_out[NC * p + i] = m[i];
+  }
 }
 
 // Composite map step (App. B, compact form): m += D^-1 acc with D^-1 in W; acc cleared; the
@@ -1111,6 +1128,16 @@ __global__ void k_pcg_dir(int64_t n_pix, const double* __restrict__ z, double* _
     pv[j] = m[i];
   }
   store_map4<NC>(map4, p, m);
+}
+
+// The map step; two pixels a thread where that still fills the GPU.
+static cudaError_t launch_bin_apply(const mm_plan_s* p, double* map_out, int* iter, cudaStream_t s) {
+  const bool wide = p->n_pix >= (1 << 19);
+  auto k = p->ncomp == 3 ? (wide ? k_bin_apply<3, 2> : k_bin_apply<3, 1>)
+                         : (wide ? k_bin_apply<1, 2> : k_bin_apply<1, 1>);
+  const int per = wide ? 512 : 256;
+  k<<<(unsigned)((p->n_pix + per - 1) / per), 256, 0, s>>>(p->n_pix, p->acc, p->W, p->map4, map_out, iter);
+  return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------------- plan API
@@ -1769,9 +1796,7 @@ extern "C" mm_status mm_messenger_iterate(mm_plan p, const double* lambdas, int 
                   L_(launch_col_forward(p, B, kSrcGather, nullptr, s)); L_(launch_row(p, B, a, s));
                   L_(launch_col_inverse(p, B, s)); });
     double* mo = it == n_iter - 1 ? map_inout : nullptr;
-    if (p->ncomp == 3) k_bin_apply<3><<<blocks_for(p->n_pix, 256), 256, 0, s>>>(p->n_pix, p->acc, p->W, p->map4, mo);
-    else k_bin_apply<1><<<blocks_for(p->n_pix, 256), 256, 0, s>>>(p->n_pix, p->acc, p->W, p->map4, mo);
-    LAUNCHED("k_bin_apply");
+    MM_CUDA(launch_bin_apply(p, mo, nullptr, s));
   }
   return check_waits(p, s, "mm_messenger_iterate");
 }
@@ -1785,9 +1810,7 @@ mm_status mm::messenger_step_keep(mm_plan_s* p, double lambda, const double* map
   RowArgs a{kRowMessengerKeep, lambda, nullptr, keep};
   FOR_BATCHES(L_(launch_col_forward(p, B, kSrcGather, nullptr, s)); L_(launch_row(p, B, a, s));
               L_(launch_col_inverse(p, B, s)));
-  if (p->ncomp == 3) k_bin_apply<3><<<blocks_for(p->n_pix, 256), 256, 0, s>>>(p->n_pix, p->acc, p->W, p->map4, map_out);
-  else k_bin_apply<1><<<blocks_for(p->n_pix, 256), 256, 0, s>>>(p->n_pix, p->acc, p->W, p->map4, map_out);
-  LAUNCHED("k_bin_apply");
+  MM_CUDA(launch_bin_apply(p, map_out, nullptr, s));
   return MM_OK;
 }
 
@@ -2033,9 +2056,7 @@ extern "C" mm_status mm_messenger_stage(mm_plan p, int stage, int batch, double 
       break;
     }
     case MM_STAGE_MAP:
-      if (p->ncomp == 3) k_bin_apply<3><<<blocks_for(p->n_pix, 256), 256, 0, s>>>(p->n_pix, p->acc, p->W, p->map4, map_inout);
-      else k_bin_apply<1><<<blocks_for(p->n_pix, 256), 256, 0, s>>>(p->n_pix, p->acc, p->W, p->map4, map_inout);
-      LAUNCHED("k_bin_apply");
+      MM_CUDA(launch_bin_apply(p, map_inout, nullptr, s));
       return MM_OK;
     default:
       mm_set_error("unknown stage %d", stage);
@@ -2069,11 +2090,7 @@ static cudaError_t launch_iteration(mm_plan p, double* map_out, cudaStream_t s) 
     e = launch_col_inverse(p, B, s);
   }
   if (e != cudaSuccess) return e;
-  if (p->ncomp == 3)
-    k_bin_apply<3><<<blocks_for(p->n_pix, 256), 256, 0, s>>>(p->n_pix, p->acc, p->W, p->map4, map_out, p->iter);
-  else
-    k_bin_apply<1><<<blocks_for(p->n_pix, 256), 256, 0, s>>>(p->n_pix, p->acc, p->W, p->map4, map_out, p->iter);
-  return cudaGetLastError();
+  return launch_bin_apply(p, map_out, p->iter, s);
 }
 
 static mm_status capture_iteration_graph(mm_plan p) {

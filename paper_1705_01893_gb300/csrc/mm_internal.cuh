@@ -265,15 +265,14 @@ __host__ __device__ __forceinline__ int64_t acc_stride_of(int64_t n_pix, int nco
   return ncomp == 1 ? n_pix : ((n_pix + 31) / 32) * 32 + 32;
 }
 
-// Read pixel p's sums from the planar accumulators and clear them for the next pass.
+// Read pixel p's sums from the planar accumulators and clear them for the next pass: all loads
+// first (the compiler keeps a load behind a store to the same array).
 template <int NC>
 __device__ __forceinline__ void take_acc(double* acc, int64_t n_pix, int64_t p, double* a) {
 #pragma unroll
-  for (int i = 0; i < NC; ++i) {
-    double* q = acc + i * acc_stride_of(n_pix, NC) + p;
-    a[i] = *q;
-    *q = 0.0;
-  }
+  for (int i = 0; i < NC; ++i) a[i] = __ldcs(acc + i * acc_stride_of(n_pix, NC) + p);
+#pragma unroll
+  for (int i = 0; i < NC; ++i) acc[i * acc_stride_of(n_pix, NC) + p] = 0.0;
 }
 
 // ------------------------------------------------------------------------- butterflies
