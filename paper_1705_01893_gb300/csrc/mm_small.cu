@@ -8,8 +8,8 @@
 // nothing of the chunk leaves the chip between gather and binning.  The map step is shared out
 // over all CTAs between two grid barriers (one cluster: the cluster's own barrier), and one
 // launch runs the whole schedule.  What bounds an iteration is then the chain of barriers,
-// exchanges and L2 round trips.Measured: one chunk of 2^15 samples, T-only, 101 iterations
-// 2.10 -> 1.35 ms; 12 ragged IQU chunks of 1500 to 12000 samples, 21 iterations 844 -> 318 us.
+// exchanges and L2 round trips.  Measured: one chunk of 2^15 samples, T-only, 101 iterations
+// 2.10 -> 1.16 ms; 12 ragged IQU chunks of 1500 to 12000 samples, 21 iterations 844 -> 328 us.
 //
 // Lengths are general (radices 2, 3, 4, 5, 8, 16 at run time), with the layouts and scales of
 // the other paths: row layout of d~ and Nbar, sums scaled by 1 / (n tau).
@@ -579,6 +579,8 @@ static cudaError_t small_clusters(K k, int S, size_t smem, int* n) {
   const int most = optin - (int)fa.sharedSizeBytes;
   if (smem > (size_t)most) return cudaSuccess;
   if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess) return e;
+  if (S > 8 && (e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
+    return e;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute at[2];
   small_config(&cfg, at, S, S, smem, nullptr);
@@ -591,9 +593,10 @@ static cudaError_t small_clusters(K k, int S, size_t smem, int* n) {
 // Words of a work buffer times a cluster's turns up to which a plan takes this path.  Measured
 // per iteration against the three-kernel path (chunks x samples): power-of-two lengths, T-only,
 // 4 x 2^15 (2450 words) 16.3 against 24.4 us, 8 x 2^16 (4900) 23.2 / 28.1, 4 x 2^17 (9700)
-// 44.7 / 28.5; IQU 18.7 / 28.3, 32.0 / 32.2, 52.2 / 34.6.  General lengths, whose three kernels
-// are slower, IQU: 12 chunks of 1500 to 12000 samples 15.8 / 40.9, 4 of 20000 to 90000 (5600
-// words) 46.3 / 53.1.
+// 44.7 / 28.5; IQU 18.7 / 28.3, 32.0 / 32.2, 52.2 / 34.6 (clusters of 8).  Clusters of 16, where
+// they fit (about four at once): IQU 4 x 2^15 16.3, 4 x 2^16 18.9 us, T-only 4 x 2^17 22.9.  General
+// lengths, whose three kernels are slower, IQU: 12 chunks of 1500 to 12000 samples 15.8 / 40.9, 4 of 20000 to 90000 (5600
+// words) 46.3 / 53.1, with clusters of 16 25.6.
 static int small_limit(bool general, int ncomp) {
   return general ? 6144 : ncomp == 1 ? 5120 : 4096;
 }
@@ -602,16 +605,23 @@ template <int NC>
 static cudaError_t small_plan_nc(const mm_plan_s* p, SmallShape* out) {
   *out = SmallShape{};
   const int limit = small_limit(p->n_gen > 0, NC);
-  for (int c = 0; c < p->n_chunks; ++c)
-    if (p->h_desc[c].M > 8 * limit) return cudaSuccess;
+  int tables = 0;
+  for (int c = 0; c < p->n_chunks; ++c) {
+    const ChunkDesc& d = p->h_desc[c];
+    if (d.M > 16 * limit) return cudaSuccess;
+    tables = std::max(tables, small_table_words(d, p->groups[d.grp].log_lo));
+  }
+  auto largest = [&](int S) {
+    int tile = 0;
+    for (int c = 0; c < p->n_chunks; ++c) tile = std::max(tile, small_tile_words(p->h_desc[c], S));
+    return tile;
+  };
   SmallShape best;
-  for (int S = 8; S >= 1; S /= 2) {
-    int tile = 0, tables = 0, n = 0;
-    for (int c = 0; c < p->n_chunks; ++c) {
-      const ChunkDesc& d = p->h_desc[c];
-      tile = std::max(tile, small_tile_words(d, S));
-      tables = std::max(tables, small_table_words(d, p->groups[d.grp].log_lo));
-    }
+  // clusters of 16 for chunks whose share of 8 CTAs is not tiny (below, the larger cluster's
+  // barriers cost more than the halved tiles save: 4 x 2^12 10.4 us against 11.4)
+  for (int S = largest(8) >= 512 ? 16 : 8; S >= 1; S /= 2) {
+    const int tile = largest(S);
+    int n = 0;
     if (tile > limit) break;   // smaller clusters hold larger tiles
     // the largest cluster size whose clusters keep a chunk each; else the one with the most clusters
     cudaError_t e = small_clusters(k_small<NC, true>, S, small_smem(tile, tables, NC, true), &n);
