@@ -50,8 +50,8 @@ struct Src2Rows {             // rows rA (b = 0) and rB (b = 1) of yV
 
 // The filtered adjoint spectrum b v~ of rows rA, rB of yV; THETA: also the theta sums, with
 // the forward spectrum read from rspec.
-template <int M2, int T, bool THETA>
-__global__ void __launch_bounds__(T, pass_ctas(T, 8)) k_row_adjoint(AdjRowParams q) {
+template <int M2, int T, bool THETA, bool ROOMY>
+__global__ void __launch_bounds__(T, pass_ctas(T, 8, ROOMY)) k_row_adjoint(AdjRowParams q) {
   extern __shared__ float2 sm[];
   using Lay = RowLayout<M2>;
   __shared__ double red[kAdjN - 1][32];
@@ -198,9 +198,9 @@ __device__ __forceinline__ float4 gather4_map(const ColParams& q, const void* ma
 
 // Inverse column DFTs of the adjoint spectrum -> t = irfft(b v~)/tau; bin P^T t (the next
 // gbar), accumulate dL/dd += v/tau - t and (THETA) <v, P m'> per chunk.
-template <int M1, int CB, int T, int NC, bool THETA>
-__global__ void __launch_bounds__(T, pass_ctas(T, 8)) k_col_inverse_adjoint(ColParams q,
-                                                                          AdjColExtra x) {
+template <int M1, int CB, int T, int NC, bool THETA, bool ROOMY>
+__global__ void __launch_bounds__(T, pass_ctas(T, 8, ROOMY)) k_col_inverse_adjoint(ColParams q,
+                                                                                 AdjColExtra x) {
   extern __shared__ float2 sm[];
   __shared__ double red[32];
   const int M2 = q.g.M2;
@@ -346,9 +346,11 @@ static cudaError_t row_adjoint_m2(const mm_plan_s* p, const Batch& b, float2* yV
   q.acc = acc;
   const bool theta = rspec != nullptr;
   const size_t smem = sizeof(float2) * (2 * M2 + tw_size(M2));
-  auto k = theta ? k_row_adjoint<M2, T, true> : k_row_adjoint<M2, T, false>;
+  constexpr bool R = T != 512;
+  auto roomy = theta ? k_row_adjoint<M2, T, true, R> : k_row_adjoint<M2, T, false, R>;
+  auto k = theta ? k_row_adjoint<M2, T, true, false> : k_row_adjoint<M2, T, false, false>;
   int grid = 0;
-  cudaError_t e = persistent_grid(k, T, smem, (g.M1 / 2 + 1) * b.count, &grid);
+  cudaError_t e = pass_grid(roomy, k, T, smem, (g.M1 / 2 + 1) * b.count, &k, &grid);
   if (e != cudaSuccess) return e;
   k<<<grid, T, smem, st>>>(q);
   return cudaGetLastError();
@@ -395,15 +397,11 @@ static cudaError_t col_adjoint_m1(const mm_plan_s* p, const Batch& b, const AdjC
   const size_t smem = sizeof(float2) * M1 * kColCB;
   int grid = 0;
   cudaError_t e;
-  if (p->ncomp == 3) {
-    auto k = k_col_inverse_adjoint<M1, kColCB, T, 3, THETA>;
-    if ((e = persistent_grid(k, T, smem, ntiles, &grid)) != cudaSuccess) return e;
-    k<<<grid, T, smem, st>>>(q, x);
-  } else {
-    auto k = k_col_inverse_adjoint<M1, kColCB, T, 1, THETA>;
-    if ((e = persistent_grid(k, T, smem, ntiles, &grid)) != cudaSuccess) return e;
-    k<<<grid, T, smem, st>>>(q, x);
-  }
+  constexpr bool R = T != 512;
+  auto roomy = p->ncomp == 3 ? k_col_inverse_adjoint<M1, kColCB, T, 3, THETA, R> : k_col_inverse_adjoint<M1, kColCB, T, 1, THETA, R>;
+  auto k = p->ncomp == 3 ? k_col_inverse_adjoint<M1, kColCB, T, 3, THETA, false> : k_col_inverse_adjoint<M1, kColCB, T, 1, THETA, false>;
+  if ((e = pass_grid(roomy, k, T, smem, ntiles, &k, &grid)) != cudaSuccess) return e;
+  k<<<grid, T, smem, st>>>(q, x);
   return cudaGetLastError();
 }
 

@@ -11,8 +11,8 @@
 namespace mm {
 
 // Persistent over the batch's tiles (chunk ci, column block cb).
-template <int M1, int CB, int T, int NC, int SRC>
-__global__ void __launch_bounds__(T, pass_ctas(T, 8)) k_col_forward(ColParams q) {
+template <int M1, int CB, int T, int NC, int SRC, bool ROOMY>
+__global__ void __launch_bounds__(T, pass_ctas(T, 8, ROOMY)) k_col_forward(ColParams q) {
   extern __shared__ float2 sm[];
   __shared__ float2 s4[SRC == kSrcTod ? 1 : four_step_n(M1, kColLo) * CB];
   const int M2 = q.g.M2;
@@ -36,8 +36,8 @@ __global__ void __launch_bounds__(T, pass_ctas(T, 8)) k_col_forward(ColParams q)
   }
 }
 
-template <int M1, int CB, int T, int NC, bool COMP>
-__global__ void __launch_bounds__(T, pass_ctas(T, 8)) k_col_inverse(ColParams q) {
+template <int M1, int CB, int T, int NC, bool COMP, bool ROOMY>
+__global__ void __launch_bounds__(T, pass_ctas(T, 8, ROOMY)) k_col_inverse(ColParams q) {
   extern __shared__ float2 sm[];
   const int M2 = q.g.M2;
   const int tpc = M2 / CB;
@@ -175,10 +175,14 @@ static cudaError_t col_forward_m1(const mm_plan_s* p, const Batch& b, int src, c
   cudaError_t e;
   int grid = 0;
   const bool iqu = p->ncomp == 3;
-  auto k = src == kSrcTod ? k_col_forward<M1, CB, kColT, 1, kSrcTod>
-           : p->composite ? (iqu ? k_col_forward<M1, CB, kColT, 3, kSrcGather2> : k_col_forward<M1, CB, kColT, 1, kSrcGather2>)
-                          : (iqu ? k_col_forward<M1, CB, kColT, 3, kSrcGather> : k_col_forward<M1, CB, kColT, 1, kSrcGather>);
-  if ((e = persistent_grid(k, kColT, smem, ntiles, &grid)) != cudaSuccess) return e;
+  auto pick = [&](auto roomy_) {
+    constexpr bool R = decltype(roomy_)::value && kColT != 512;
+    return src == kSrcTod ? k_col_forward<M1, CB, kColT, 1, kSrcTod, R>
+           : p->composite ? (iqu ? k_col_forward<M1, CB, kColT, 3, kSrcGather2, R> : k_col_forward<M1, CB, kColT, 1, kSrcGather2, R>)
+                          : (iqu ? k_col_forward<M1, CB, kColT, 3, kSrcGather, R> : k_col_forward<M1, CB, kColT, 1, kSrcGather, R>);
+  };
+  auto k = pick(std::false_type{});
+  if ((e = pass_grid(pick(std::true_type{}), k, kColT, smem, ntiles, &k, &grid)) != cudaSuccess) return e;
   k<<<grid, kColT, smem, st>>>(q);
   return cudaGetLastError();
 }
@@ -193,9 +197,13 @@ static cudaError_t col_inverse_m1(const mm_plan_s* p, const Batch& b, cudaStream
   cudaError_t e;
   int grid = 0;
   const bool iqu = p->ncomp == 3;
-  auto k = p->composite ? (iqu ? k_col_inverse<M1, CB, kColT, 3, true> : k_col_inverse<M1, CB, kColT, 1, true>)
-                        : (iqu ? k_col_inverse<M1, CB, kColT, 3, false> : k_col_inverse<M1, CB, kColT, 1, false>);
-  if ((e = persistent_grid(k, kColT, smem, ntiles, &grid)) != cudaSuccess) return e;
+  auto pick = [&](auto roomy_) {
+    constexpr bool R = decltype(roomy_)::value && kColT != 512;
+    return p->composite ? (iqu ? k_col_inverse<M1, CB, kColT, 3, true, R> : k_col_inverse<M1, CB, kColT, 1, true, R>)
+                        : (iqu ? k_col_inverse<M1, CB, kColT, 3, false, R> : k_col_inverse<M1, CB, kColT, 1, false, R>);
+  };
+  auto k = pick(std::false_type{});
+  if ((e = pass_grid(pick(std::true_type{}), k, kColT, smem, ntiles, &k, &grid)) != cudaSuccess) return e;
   k<<<grid, kColT, smem, st>>>(q);
   return cudaGetLastError();
 }

@@ -752,14 +752,25 @@ cudaError_t launch_col_forward_ex(const mm_plan_s* p, const Batch& b, int src, c
 // threads: two CTAs per SM overlap one's loads with the other's DFT passes.
 constexpr int kColCB = 16;
 __host__ __device__ constexpr int col_cb(int M1) { return M1 <= 512 ? kColCB : 8192 / M1; }
-// Resident CTAs per SM that the pass kernels are compiled for: 64 registers a thread (1024
-// threads on an SM) from 128 threads a CTA on, 80 to 128 registers below that.  Left to
-// itself the compiler gives the 128- and 256-thread shapes 120 to 170 registers, which leaves
-// 12 to 16 warps on an SM to hide the loads; capped, they spill at most 50 bytes.  Measured on
-// the 4 x 2^20-sample, 256^2 iteration (rows of 1024 points, 128 threads): 83 -> 73 us; the
-// 20-step gradient on the same data 7.21 -> 6.39 ms; the 512-thread shapes keep their 2.
-__host__ __device__ constexpr int pass_ctas(int threads, int below128) {
-  return threads > 512 ? 1 : threads >= 128 ? 1024 / threads : below128;
+// Resident CTAs per SM that the pass kernels are compiled for, two instances each.  ROOMY: two (one
+// above 512 threads), which leaves the 128- and 256-thread shapes the 120 to 170 registers that
+// the compiler takes by itself, but only 12 to 16 warps on an SM to hide the loads.  Otherwise 64
+// registers a thread (1024 threads on an SM) from 128 threads a CTA on, 80 to 128 below that, for
+// at most 50 bytes of spills.  The roomy one runs launches that it holds in one wave anyway (2
+// chunks of 2^18 samples, 3 iterations: 145 us, capped 150); beyond, the full SM pays (256^2,
+// 4 x 2^20 iteration, rows of 1024 points: 83 -> 73 us; the 20-step gradient on the same data 7.21
+// -> 6.39 ms).  The 512-thread shapes have one instance.
+__host__ __device__ constexpr int pass_ctas(int threads, int below128, bool roomy) {
+  return threads > 512 ? 1 : threads == 512 || roomy ? 2 : threads >= 128 ? 1024 / threads : below128;
+}
+// The instance for `work` items and its grid.
+template <typename K>
+static cudaError_t pass_grid(K roomy, K full, int threads, size_t smem, int work, K* k, int* grid) {
+  int most = 0;
+  const cudaError_t e = resident_ctas(reinterpret_cast<const void*>(roomy), threads, smem, &most);
+  if (e != cudaSuccess) return e;
+  *k = work <= most ? roomy : full;
+  return persistent_grid(*k, threads, smem, work, grid);
 }
 // Threads of the column kernels for column length M1 (16 complex values per thread per pass).
 __host__ __device__ constexpr int col_threads(int M1) {

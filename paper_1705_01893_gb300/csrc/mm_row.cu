@@ -5,8 +5,8 @@
 
 namespace mm {
 
-template <int M2, int T, int MODE>
-__global__ void __launch_bounds__(T, pass_ctas(T, 12)) k_row(RowParams q) {
+template <int M2, int T, int MODE, bool ROOMY>
+__global__ void __launch_bounds__(T, pass_ctas(T, 12, ROOMY)) k_row(RowParams q) {
   extern __shared__ float2 sm[];
   using Lay = RowLayout<M2>;
   __shared__ float red[32];
@@ -97,11 +97,16 @@ static cudaError_t row_m2(const mm_plan_s* p, const Batch& b, const RowArgs& a,
   const size_t smem = sizeof(float2) * (2 * M2 + tw_size(M2));
   // the per-iteration modes (messenger step, its map-sized form) get their own instances
   // with the mode folded in; the set-up, PCG and chi^2 modes share one
-  auto k = a.mode == kRowMessenger    ? k_row<M2, T, kRowMessenger>
-           : a.mode == kRowMessengerF ? k_row<M2, T, kRowMessengerF>
-                                      : k_row<M2, T, -1>;
+  constexpr bool R = T != 512;   // one instance only at 512 threads
+  auto roomy = a.mode == kRowMessenger    ? k_row<M2, T, kRowMessenger, R>
+               : a.mode == kRowMessengerF ? k_row<M2, T, kRowMessengerF, R>
+                                          : k_row<M2, T, -1, R>;
+  auto full = a.mode == kRowMessenger    ? k_row<M2, T, kRowMessenger, false>
+              : a.mode == kRowMessengerF ? k_row<M2, T, kRowMessengerF, false>
+                                         : k_row<M2, T, -1, false>;
+  auto k = full;
   int grid = 0;
-  cudaError_t e = persistent_grid(k, T, smem, (g.M1 / 2 + 1) * b.count, &grid);
+  cudaError_t e = pass_grid(roomy, full, T, smem, (g.M1 / 2 + 1) * b.count, &k, &grid);
   if (e != cudaSuccess) return e;
   k<<<grid, T, smem, st>>>(q);
   return cudaGetLastError();
