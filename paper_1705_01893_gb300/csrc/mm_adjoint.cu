@@ -153,9 +153,9 @@ __global__ void __launch_bounds__(T, pass_ctas(T, 8, ROOMY)) k_row_adjoint(AdjRo
       const float2 Dq = THETA && !same ? dt[sp] : make_float2(0.f, 0.f);
       const float2 Yk = mode(Vk, Rk, Dk, nb[sk], k, 2.f);
       const float2 Yp = same ? Yk : mode(Vp, Rp, Dq, nb[sp], M - k, 2.f);
-      sm[Lay::at(0, p)] = cadd(cadd(Yk, cconj(Yp)), mul_i<+1>(cmulc(csub(Yk, cconj(Yp)), w)));
-      if (!same)
-        sm[Lay::at(qs, qi)] = csub(cadd(Yp, cconj(Yk)), mul_i<+1>(cmul(w, csub(Yp, cconj(Yk)))));
+      const float2 S = cadd(Yk, cconj(Yp)), Tw = mul_i<+1>(cmulc(csub(Yk, cconj(Yp)), w));
+      sm[Lay::at(0, p)] = cadd(S, Tw);
+      if (!same) sm[Lay::at(qs, qi)] = cconj(csub(S, Tw));
     }
     if constexpr (THETA) {
       // block sums (FP32 within a warp, FP64 across warps), one FP64 add per chunk and term

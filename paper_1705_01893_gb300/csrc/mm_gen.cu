@@ -849,10 +849,10 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1) k_gen_row(GenParams
           if (!inv) continue;
           const float2 Yk = filt(Xk, Dk[u], nk[u]);
           const float2 Yp = filt(Xp, Dp[u], np[u]);
-          // Z'_k = (Y_k + conj Y_p) + i conj(w) (Y_k - conj Y_p)
-          // Z'_p = (Y_p + conj Y_k) - i w (Y_p - conj Y_k)
-          z[ek] = cadd(cadd(Yk, cconj(Yp)), mul_i<+1>(cmulc(csub(Yk, cconj(Yp)), w)));
-          if (!same) z[ep] = csub(cadd(Yp, cconj(Yk)), mul_i<+1>(cmul(w, csub(Yp, cconj(Yk)))));
+          // Z'_k = S + T, Z'_p = conj(S - T) with S = Y_k + conj Y_p, T = i conj(w) (Y_k - conj Y_p)
+          const float2 S = cadd(Yk, cconj(Yp)), Tw = mul_i<+1>(cmulc(csub(Yk, cconj(Yp)), w));
+          z[ek] = cadd(S, Tw);
+          if (!same) z[ep] = cconj(csub(S, Tw));
         }
       }
     }

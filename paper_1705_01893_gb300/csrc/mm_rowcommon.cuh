@@ -9,7 +9,7 @@
 //   t~ = (lambda tau d~ + Nbar (Pm)~) / (lambda tau + Nbar)),
 // accumulates chi^2 = (1/n) sum_k w_k |d~ - (Pm)~|^2 / N (Eq. 3 evaluated per Fourier mode,
 // Sec. 3.1), merges the filtered Hermitian spectrum back into the packed form
-//   Z'_k = (Y_k + conj Y_{M-k}) + i conj(w_{2M}^k) (Y_k - conj Y_{M-k})
+//   Z'_k = S + T, Z'_{M-k} = conj(S - T),  S = Y_k + conj Y_{M-k}, T = i conj(w_{2M}^k) (Y_k - conj Y_{M-k})
 // and runs the inverse row DFTs, so the spectrum never leaves the chip between the forward
 // and inverse transforms.
 #pragma once
@@ -264,14 +264,10 @@ __device__ __forceinline__ void kernel_body_job(const RowParams& q, float2* sm, 
       if (!inv) continue;
       const float2 Yk = filt(Xk, Dk[u], nk[u]);
       const float2 Yp = filt(Xp, Dp[u], np[u]);
-      // Z'_k = (Y_k + conj Y_p) + i conj(w) (Y_k - conj Y_p);
-      // Z'_p = (Y_p + conj Y_k) - i w (Y_p - conj Y_k)
-      const float2 zk = cadd(cadd(Yk, cconj(Yp)), mul_i<+1>(cmulc(csub(Yk, cconj(Yp)), w)));
-      sm[Lay::at(0, p)] = zk;
-      if (!same) {
-        const float2 zp = csub(cadd(Yp, cconj(Yk)), mul_i<+1>(cmul(w, csub(Yp, cconj(Yk)))));
-        sm[Lay::at(qs, qi)] = zp;
-      }
+      // Z'_k = S + T, Z'_p = conj(S - T) with S = Y_k + conj Y_p, T = i conj(w) (Y_k - conj Y_p)
+      const float2 S = cadd(Yk, cconj(Yp)), Tw = mul_i<+1>(cmulc(csub(Yk, cconj(Yp)), w));
+      sm[Lay::at(0, p)] = cadd(S, Tw);
+      if (!same) sm[Lay::at(qs, qi)] = cconj(csub(S, Tw));
     }
   }
 

@@ -387,8 +387,9 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(SmallParams q) {
             if (!same) t += __fdividef(e2.x * e2.x + e2.y * e2.y, np + tau);
             x2 += 2.f * t;
             const float2 Yk = filt(Xk, Dk, nk), Yp = filt(Xp, Dp, np);
-            z[ek] = cadd(cadd(Yk, cconj(Yp)), mul_i<+1>(cmulc(csub(Yk, cconj(Yp)), w)));
-            if (!same) z[ep] = csub(cadd(Yp, cconj(Yk)), mul_i<+1>(cmul(w, csub(Yp, cconj(Yk)))));
+            const float2 Sm = cadd(Yk, cconj(Yp)), Tw = mul_i<+1>(cmulc(csub(Yk, cconj(Yp)), w));
+            z[ek] = cadd(Sm, Tw);
+            if (!same) z[ep] = cconj(csub(Sm, Tw));
           }
         }
         if (q.chi2) {   // FP32 within a warp, FP64 across warps and CTAs
