@@ -285,8 +285,8 @@ mm_status mm_chi2(mm_plan p, const double* map, double lambda, double* chi2_dev,
  *   m' = m + D^-1 P^T (Nbar / lambda + T)^-1 (d - P m)      (lambda = inf: T^-1)
  * (the map is not reset at lambda = inf: F(inf) != 0 for two components).  Arguments as
  * for mm_plan_pointing, plus the second component and the two gains (finite, not both 0);
- * every chunk runs on the general-length kernels (lengths with prime factors 2, 3, 5 up to
- * 2^21).  Available on a composite plan: mm_set_noise_psd, mm_lambda_max,
+ * chunk lengths have prime factors 2, 3, 5 and n / 2 <= 2^21; those of power-of-two length on
+ * multiples of 4 samples run on the compile-time kernels, the others on the general ones.  Available on a composite plan: mm_set_noise_psd, mm_lambda_max,
  * mm_messenger_iterate, mm_chi2, mm_chi2_modes, mm_rfft, mm_plan_maps (weight = D^-1),
  * mm_autotune / mm_set_tune / mm_get_tune; the other iteration forms and the operators
  * return MM_ERR_UNSUPPORTED.  The workspace size comes from

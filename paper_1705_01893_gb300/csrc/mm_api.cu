@@ -1053,14 +1053,16 @@ __global__ void k_pcg_q(int64_t n_pix, double* __restrict__ acc, const uint8_t* 
   const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   double s = 0.0;
   if (p < n_pix) {
-    double a[NC];
-    take_acc<NC>(acc, n_pix, p, a);
+    double a[NC], pp[NC];
     const bool ok = valid[p] != 0;
+#pragma unroll
+    for (int i = 0; i < NC; ++i) pp[i] = pv[NC * p + i];
+    take_acc<NC>(acc, n_pix, p, a);
 #pragma unroll
     for (int i = 0; i < NC; ++i) {
       const double qq = ok ? a[i] : 0.0;
       q[NC * p + i] = qq;
-      s += pv[NC * p + i] * qq;
+      s += pp[i] * qq;
     }
   }
   s = block_sum(s, red);
@@ -1081,21 +1083,31 @@ __global__ void k_pcg_update(int64_t n_pix, double* __restrict__ x, double* __re
                              const double* __restrict__ Minv, double* sc, int rz_cur, int rz_next) {
   __shared__ double red[32];
   const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const double alpha = sc[rz_cur] / sc[kPcgPq];
+  __shared__ double s_alpha;   // one FP64 division a CTA, not one a thread
+  if (threadIdx.x == 0) s_alpha = sc[rz_cur] / sc[kPcgPq];
+  __syncthreads();
+  const double alpha = s_alpha;
   double rz = 0, xb = 0, xr = 0;
   if (p < n_pix) {
-    double rr[NC], zz[NC];
+    // all loads before the first store (see k_bin_apply)
+    double rr[NC], zz[NC], xv[NC], pp[NC], qq[NC], bb[NC], w[NC == 3 ? 6 : 1];
 #pragma unroll
     for (int i = 0; i < NC; ++i) {
       const int64_t j = NC * p + i;
-      const double xv = x[j] + alpha * pv[j];
-      x[j] = xv;
-      rr[i] = r[j] - alpha * q[j];
-      r[j] = rr[i];
-      xb += xv * bvec[j];
-      xr += xv * rr[i];
+      xv[i] = x[j]; pp[i] = pv[j]; rr[i] = r[j]; qq[i] = q[j]; bb[i] = bvec[j];
     }
-    block_apply<NC>(Minv, p, rr, zz);
+    load_block<NC>(Minv, p, w);
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+      const int64_t j = NC * p + i;
+      xv[i] += alpha * pp[i];
+      x[j] = xv[i];
+      rr[i] -= alpha * qq[i];
+      r[j] = rr[i];
+      xb += xv[i] * bb[i];
+      xr += xv[i] * rr[i];
+    }
+    sym_apply<NC>(w, rr, zz);
 #pragma unroll
     for (int i = 0; i < NC; ++i) {
       z[NC * p + i] = zz[i];
@@ -1118,14 +1130,21 @@ __global__ void k_pcg_dir(int64_t n_pix, const double* __restrict__ z, double* _
                           void* map4, double* sc, int rz_cur, int rz_next) {
   const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (p == 0) sc[kPcgPq] = 0.0;   // read by the update kernel before, added to by the next q kernel
+  __shared__ double s_beta;
+  if (threadIdx.x == 0) s_beta = sc[rz_next] / sc[rz_cur];
+  __syncthreads();
   if (p >= n_pix) return;
-  const double beta = sc[rz_next] / sc[rz_cur];
-  double m[NC];
+  const double beta = s_beta;
+  double m[NC], pp[NC];
 #pragma unroll
   for (int i = 0; i < NC; ++i) {
-    const int64_t j = NC * p + i;
-    m[i] = z[j] + beta * pv[j];
-    pv[j] = m[i];
+    m[i] = z[NC * p + i];
+    pp[i] = pv[NC * p + i];
+  }
+#pragma unroll
+  for (int i = 0; i < NC; ++i) {
+    m[i] += beta * pp[i];
+    pv[NC * p + i] = m[i];
   }
   store_map4<NC>(map4, p, m);
 }

@@ -116,3 +116,36 @@ def test_composite_refuses_single_component_forms():
         with pytest.raises(binding.MMError) as e:
             call()
         assert e.value.code == binding.MM_ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("lens", [[1024, 2048], [1 << 12, 3000, 1 << 12, 1125]])
+@pytest.mark.parametrize("half", [False, True])
+def test_composite_kernels_match_oracle(lens, half):
+    """IQU composite plans with unequal gains whose power-of-two chunks run on the compile-time
+    kernels, alone and beside general lengths, FP32 and FP16 weights: two steps and chi^2 within
+    1e-5 of the oracle."""
+    rng = np.random.default_rng(8)
+    n, npix = int(sum(lens)), 30
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    wt = np.float16 if half else np.float32
+    comps = []
+    for k in range(2):
+        pix = np.repeat(rng.integers(-1, npix, size=n // 3 + 1), 3)[:n].astype(np.int32)
+        psi = rng.uniform(0, np.pi, n)
+        comps.append((pix, np.cos(2 * psi).astype(wt), np.sin(2 * psi).astype(wt)))
+    tod = rng.standard_normal(n).astype(np.float32)
+    params = np.array([[1.0, 0.5, 1.5, 50.0]] * len(lens))
+    ga, gb = 1.0, -0.6
+    psd = [O.psd_from_params(k, 50.0, 1.0, 0.5, 1.5) for k in lens]
+    prob = C.CompositeProblem((*comps[0], ga), (*comps[1], float(np.float32(gb))), tod, off, npix, 3, psd,
+                              np.ones(len(lens)))
+    lam = [4.0, 1.0]
+    ref, chi_ref = C.run(prob, lam)
+    up = lambda a: torch.from_numpy(a).cuda()
+    plan = binding.Plan(off, *[up(a) for a in comps[0]], npix, 3, second=(*[up(a) for a in comps[1]], ga, gb))
+    plan.set_noise(up(tod), params=params)
+    m = torch.zeros(npix, 3, dtype=torch.float64, device="cuda")
+    chi = torch.zeros(2, dtype=torch.float64, device="cuda")
+    plan.messenger(m, lam, chi)
+    assert np.linalg.norm(m.cpu().numpy() - ref) <= 1e-5 * np.linalg.norm(ref)
+    assert np.max(np.abs(chi.cpu().numpy() - chi_ref) / chi_ref) <= 1e-5
