@@ -347,8 +347,9 @@ mm_status mm_chi2_modes(mm_plan p, const double* map, double lambda, double* chi
  * mixed-radix kernels; no counterpart in the paper, which gives no implementation).
  * mm_autotune measures, on this plan's own chunks and on `stream`, the column-tile width
  * (8 or 16 columns), threads per CTA of the column (256, 512) and row (256, 512, 1024)
- * kernels and the radix order (0: radix 8 first, then 4/2, 5, 3; 1: radix 4 in place of 8;
- * 2: radices 3 and 5 first) and keeps the fastest.  It launches the column passes and the
+ * kernels and the order of the radices (iterations: 0 large first, 1 small first, 2 odd first;
+ * transform of the data, radices up to 8: 0 radix 8 first, then 4/2, 5, 3, 1 radix 4 in place of
+ * 8, 2 radices 3 and 5 first) and keeps the fastest.  It launches the column passes and the
  * row pass in PCG-operator mode only, which leave no state behind (the accumulators are
  * cleared), needs mm_set_noise_psd first, synchronises `stream`, and drops a captured
  * iteration graph (recaptured on the next mm_messenger_graph).  mm_set_tune sets a schedule

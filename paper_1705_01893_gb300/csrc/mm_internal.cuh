@@ -97,7 +97,8 @@ struct GenTune {
   int col_nb;         // columns per column tile: 8 or 16
   int col_threads;    // 256 or 512
   int row_threads;    // 256, 512 or 1024
-  int radix_order;    // 0: radix 8 first, then 4/2, 5, 3; 1: radix 4 instead of 8; 2: 3s and 5s first
+  int radix_order;    // 0, 1 or 2: order of the iterations' and the data's radices (radix_plan_wide,
+                      // radix_plan)
 };
 
 // Everything a general-path kernel needs about one chunk, in one record (one dependent load
