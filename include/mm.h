@@ -170,7 +170,9 @@ mm_status mm_plan_batches(mm_plan p, int* n_batches);
  * then per iteration: for each batch b, FUSED(b) where the batch is fused
  * (mm_plan_fused_batches), else GATHER_FFT(b), FILTER(b), IFFT_BIN(b); then MAP.  The same
  * sequence through this entry point gives identical results, and the three separate stages
- * on a fused batch the same up to the order of the FP64 pixel additions.
+ * on a fused batch the same up to the order of the FP64 pixel additions.  Small plans (a few
+ * short chunks) run mm_messenger_iterate and mm_messenger_graph as one launch for the whole
+ * schedule instead; these stages then give its results up to FP32 rounding.
  *   MM_STAGE_LOAD:       map_inout (device float64 [n_pix][ncomp]) -> internal FP32 map;
  *   MM_STAGE_GATHER_FFT: P m gathered from the internal map, packed, column DFTs (Eq. 1);
  *   MM_STAGE_FILTER:     row DFTs, per-mode messenger filter at `lambda` (>= 1 or INFINITY),

@@ -2002,7 +2002,7 @@ static mm_status check_waits(mm_plan p, cudaStream_t s, const char* who) {
   if (f) {
     MM_CUDA(cudaMemsetAsync(p->fault, 0, sizeof(int), s));
     MM_CUDA(clear_after_fault(p, s));
-    mm_set_error("%s: a bounded wait of the fused launch ran out (its results are wrong)", who);
+    mm_set_error("%s: a bounded wait of the call's kernels ran out (its results are wrong)", who);
     return MM_ERR_TIMEOUT;
   }
   return MM_OK;
