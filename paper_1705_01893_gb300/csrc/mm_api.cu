@@ -174,7 +174,7 @@ static int radix_plan(int L, int8_t* rad, int order = 0) {
 static int radix_plan_wide(int L, int8_t* rad, int order) {
   static const int set[] = {16, 15, 10, 9, 8, 6, 5, 4, 3, 2};
   struct Best { int n, sum, first; };
-  std::map<int, Best> best;
+  static thread_local std::map<int, Best> best;   // by length, at most the 5-smooth ones up to 4096
   std::function<Best(int)> solve = [&](int x) -> Best {
     if (x == 1) return Best{0, 0, 0};
     auto it = best.find(x);
@@ -1165,8 +1165,9 @@ static unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t
 // Tables of the general path for the current schedule (p->gen_tune): prefix sums over the
 // general chunk list, one record per general chunk (descriptor, twiddle tables, radix
 // sequences of the chosen order) and the work-item tables (chunk, tile / row) of the column
-// and row kernels; uploaded and synchronised.
-static cudaError_t gen_upload(mm_plan_s* p, cudaStream_t s) {
+// and row kernels; uploaded and synchronised.  tables: also the DFT tables and the tile-order
+// pointing, which depend on the schedule but not on the noise model.
+static cudaError_t gen_upload(mm_plan_s* p, cudaStream_t s, bool tables = true) {
   const int ng = p->n_gen, nb = p->gen_tune.col_nb;
   std::vector<GenChunk> rec(ng);
   std::vector<int2> ct;
@@ -1213,7 +1214,7 @@ static cudaError_t gen_upload(mm_plan_s* p, cudaStream_t s) {
   p->h_gen_yoff[ng] = yo;
   if (ct_n > p->gen_ccap) return cudaErrorInvalidValue;
   // per-pass DFT tables of every general group, for the radix order in use
-  for (int g = 0; g < p->n_groups; ++g) {
+  for (int g = 0; tables && g < p->n_groups; ++g) {
     const Group& G = p->groups[g];
     if (!G.general) continue;
     for (int t = 0; t < 4; ++t) {
@@ -1242,7 +1243,7 @@ static cudaError_t gen_upload(mm_plan_s* p, cudaStream_t s) {
   if ((e = cudaMemcpyAsync(p->gen_ctab, ct.data(), sizeof(int2) * ct.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) return e;
   if ((e = cudaMemcpyAsync(p->gen_rtab, rt.data(), sizeof(int4) * rt.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) return e;
   // the column kernels read the pointing in tile order for this schedule's tile width
-  if ((e = launch_gen_tile_pointing(p, s)) != cudaSuccess) return e;
+  if (tables && (e = launch_gen_tile_pointing(p, s)) != cudaSuccess) return e;
   return cudaStreamSynchronize(s);
 }
 
@@ -1665,7 +1666,7 @@ extern "C" mm_status mm_set_noise_psd(mm_plan p, const double* psd_dev, const do
     p->h_desc[c].tau = taus[c];
   }
   MM_CUDA(cudaMemcpyAsync(p->d_desc, p->h_desc, sizeof(ChunkDesc) * C, cudaMemcpyHostToDevice, s));
-  if (p->n_gen > 0) MM_CUDA(gen_upload(p, s));     // the general records carry tau too
+  if (p->n_gen > 0) MM_CUDA(gen_upload(p, s, false));   // the general records carry tau too
   const double* d_params = nullptr;
   if (params) {
     MM_CUDA(cudaMemcpyAsync(p->params, params, sizeof(double) * 4 * C, cudaMemcpyHostToDevice, s));
