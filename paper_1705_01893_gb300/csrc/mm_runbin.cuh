@@ -30,8 +30,7 @@ __device__ __forceinline__ float load_w(const void* w, int half_w, int64_t s) {
   return half_w ? __half2float(static_cast<const __half*>(w)[s]) : static_cast<const float*>(w)[s];
 }
 
-constexpr int kBinWarps = 8, kBinSegs = 4, kBinThreads = 32 * kBinWarps;
-constexpr int kBinTile = kBinThreads * 4 * kBinSegs;
+constexpr int kBinWarps = 8, kBinThreads = 32 * kBinWarps;
 
 // Op: NF float streams per sample (load), NV sums per run (add), NO outputs per run (emit).
 // Samples [n0, n1); samples with a pixel outside [0, n_pix) are skipped.  Op::tile(first,
@@ -39,8 +38,9 @@ constexpr int kBinTile = kBinThreads * 4 * kBinSegs;
 // position that starts a run whatever its pixel.
 template <class Op>
 __global__ void __launch_bounds__(kBinThreads) k_run_bin(Op op, const int32_t* __restrict__ pix,
-                                                         int64_t n0, int64_t n1, int64_t n_pix) {
+                                                         int64_t n0, int64_t n1, int64_t n_pix, int segs) {
   constexpr int NF = Op::NF, NV = Op::NV, NO = Op::NO;
+  const int tile_n = kBinThreads * 4 * segs;   // samples of a CTA, `segs` rounds of 1024
   constexpr int SV = NV | 1;   // odd stride: the sums of neighbouring runs on different banks
   __shared__ double s_val_[kBinWarps][32 * SV];
   __shared__ int2 s_at_[kBinWarps][32];      // pixel, tile position
@@ -48,10 +48,10 @@ __global__ void __launch_bounds__(kBinThreads) k_run_bin(Op op, const int32_t* _
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double* s_val = s_val_[warp];
   int2* s_at = s_at_[warp];
-  const int64_t tile = n0 + (int64_t)blockIdx.x * kBinTile;
-  op.tile(tile, (n1 - tile < kBinTile ? n1 : tile + kBinTile) - 1, s_op);
+  const int64_t tile = n0 + (int64_t)blockIdx.x * tile_n;
+  op.tile(tile, (n1 - tile < tile_n ? n1 : tile + tile_n) - 1, s_op);
   __syncthreads();
-  for (int g = 0; g < kBinSegs; ++g) {
+  for (int g = 0; g < segs; ++g) {
     const int at = ((g * kBinWarps + warp) * 32 + lane) * 4;   // the lane's first sample in the tile
     if (tile + at - 4 * lane >= n1) break;   // warp-uniform
     int p[5];
@@ -108,7 +108,9 @@ template <class Op>
 static cudaError_t launch_run_bin(const Op& op, const int32_t* pix, int64_t n0, int64_t n1,
                                   int64_t n_pix, cudaStream_t st) {
   if (n1 <= n0) return cudaSuccess;
-  k_run_bin<Op><<<(unsigned)((n1 - n0 + kBinTile - 1) / kBinTile), kBinThreads, 0, st>>>(op, pix, n0, n1, n_pix);
+  // four rounds a CTA where that still gives every SM several CTAs
+  const int segs = n1 - n0 < (1 << 22) ? 1 : 4, tile = kBinThreads * 4 * segs;
+  k_run_bin<Op><<<(unsigned)((n1 - n0 + tile - 1) / tile), kBinThreads, 0, st>>>(op, pix, n0, n1, n_pix, segs);
   return cudaGetLastError();
 }
 
