@@ -199,6 +199,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(SmallParams q) {
     return q.half_w ? __half2float(static_cast<const __half*>(w)[s]) : __ldg(static_cast<const float*>(w) + s);
   };
   if (threadIdx.x == 0) st.dead = 0;
+  // A peer's shared memory may be written only between two cluster barriers: one that shows that
+  // the peer runs (this one, before the first exchange) and the one at the end, before which none
+  // leaves.  A cluster's CTAs are scheduled together, but need not have started together.
+  cl.sync();
 
   for (int it = 0; it < q.n_iter; ++it) {
     const bool lam_inf = isinf(q.lambda[it]);
@@ -518,8 +522,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(SmallParams q) {
     }
     if (it + 1 < q.n_iter) sync_all();
   }
-  // no CTA leaves while a peer may still write into its shared memory
-  cl.sync();
+  cl.sync();   // no CTA leaves while a peer may still write into its shared memory
 }
 
 // ------------------------------------------------------------------------ host side
