@@ -63,7 +63,9 @@ __device__ __forceinline__ float2 gather_two(const ColParams& q, int p0, int p1,
     if (p0 >= 0) a = __ldg(map + p0);
     float4 b = a;
     if (p1 != p0) b = p1 < 0 ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(map + p1);
-    return make_float2(fmaf(s0, a.z, fmaf(c0, a.y, a.x)), fmaf(s1, b.z, fmaf(c1, b.y, b.x)));
+    // the pixel decides, not the zero map value: an excluded sample may have any weights (NaN, inf)
+    return make_float2(p0 < 0 ? 0.f : fmaf(s0, a.z, fmaf(c0, a.y, a.x)),
+                       p1 < 0 ? 0.f : fmaf(s1, b.z, fmaf(c1, b.y, b.x)));
   }
 }
 
