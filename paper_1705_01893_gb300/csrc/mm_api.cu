@@ -923,7 +923,7 @@ __global__ void k_gather_vec(int64_t n4, const int32_t* __restrict__ pix, const 
   q.sinw = sinw;
   q.half_w = half_w;
   q.map4 = map4;
-  __stcs(reinterpret_cast<float4*>(out) + i, gather4<NC>(q, 4 * i));
+  __stcs(reinterpret_cast<float4*>(out) + i, gather4<NC, true>(q, 4 * i));
 }
 
 template <int NC>

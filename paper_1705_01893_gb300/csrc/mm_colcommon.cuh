@@ -44,8 +44,9 @@ __device__ __forceinline__ float4 load_w4(const void* w, int half_w, int64_t s) 
   return __ldcs(reinterpret_cast<const float4*>(static_cast<const float*>(w) + s));
 }
 
-// (P m) of two consecutive samples.  They share a pixel more often than not, and then one map
-// load serves both: the gathers are short of L1 requests (a vertical sweep touches a line per
+// (P m) of two consecutive samples; the weights of an excluded one (pixel -1) must be finite, as
+// those of the tile-order copies are (included_w).  They share a pixel more often than not, and
+// then one map load serves both: the gathers are short of L1 requests (a vertical sweep touches a line per
 // pixel), not of bytes.  256^2, 4 x 2^20: 1523 -> 1461 us per
 // 21 iterations; the 20-step gradient 6424 -> 6009 us; 512^2, 8 x 2^22: 435 -> 432 us an iteration.
 template <int NC>
@@ -63,20 +64,25 @@ __device__ __forceinline__ float2 gather_two(const ColParams& q, int p0, int p1,
     if (p0 >= 0) a = __ldg(map + p0);
     float4 b = a;
     if (p1 != p0) b = p1 < 0 ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(map + p1);
-    // the pixel decides, not the zero map value: an excluded sample may have any weights (NaN, inf)
-    return make_float2(p0 < 0 ? 0.f : fmaf(s0, a.z, fmaf(c0, a.y, a.x)),
-                       p1 < 0 ? 0.f : fmaf(s1, b.z, fmaf(c1, b.y, b.x)));
+    return make_float2(fmaf(s0, a.z, fmaf(c0, a.y, a.x)), fmaf(s1, b.z, fmaf(c1, b.y, b.x)));
   }
 }
 
-// (P m) for samples s..s+3.
-template <int NC>
+// (P m) of four consecutive samples of tile-order pointing; kAnyWeights: of a caller's arrays, whose
+// excluded samples may have any weights.
+template <int NC, bool kAnyWeights = false>
 __device__ __forceinline__ float4 gather4(const ColParams& q, int64_t s) {
   const int4 p = __ldcs(reinterpret_cast<const int4*>(q.pix + s));
   float4 c = make_float4(0.f, 0.f, 0.f, 0.f), w = c;
   if constexpr (NC == 3) {
     c = load_w4(q.cosw, q.half_w, s);
     w = load_w4(q.sinw, q.half_w, s);
+    if (kAnyWeights && (p.x | p.y | p.z | p.w) < 0) {   // rarely taken: selects on every sample cost 6%
+      if (p.x < 0) c.x = w.x = 0.f;
+      if (p.y < 0) c.y = w.y = 0.f;
+      if (p.z < 0) c.z = w.z = 0.f;
+      if (p.w < 0) c.w = w.w = 0.f;
+    }
   }
   const float2 lo = gather_two<NC>(q, p.x, p.y, c.x, c.y, w.x, w.y);
   const float2 hi = gather_two<NC>(q, p.z, p.w, c.z, c.w, w.z, w.w);

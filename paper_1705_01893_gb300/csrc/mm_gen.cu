@@ -907,7 +907,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1) k_gen_row(GenParams
 // (j1, j2, h) (even n: s = 2 (j1 M2 + j2) + h; odd n: s = j1 M2 + j2, h = 0) goes to
 // tile t = j2 / nb (first column j2_0 = t nb, width w = min(nb, M2 - j2_0)) at
 // M1 j2_0 nh + (j1 w + j2 - j2_0) nh + h, nh = 2 (even) or 1 (odd): a bijection of the
-// chunk's samples.
+// chunk's samples.  Excluded samples get weight 0 (as in k_tile_pointing).
 __global__ void k_gen_tile_pointing(const int32_t* __restrict__ pix, const void* cosw,
                                     const void* sinw, int wbytes, int64_t off, int64_t toff, int n, int M1,
                                     int M2, int cplx, int nb, int32_t* __restrict__ tpix,
@@ -921,14 +921,15 @@ __global__ void k_gen_tile_pointing(const int32_t* __restrict__ pix, const void*
   const int j2_0 = j2 - j2 % nb;
   const int w = min(nb, M2 - j2_0);
   const int64_t o = toff + ((int64_t)M1 * j2_0 + (int64_t)j1 * w + (j2 - j2_0)) * nh + h;
-  tpix[o] = pix[off + i];
+  const int p = pix[off + i];
+  tpix[o] = p;
   if (cosw) {
     if (wbytes == 2) {
-      static_cast<__half*>(tcos)[o] = static_cast<const __half*>(cosw)[off + i];
-      static_cast<__half*>(tsin)[o] = static_cast<const __half*>(sinw)[off + i];
+      static_cast<uint16_t*>(tcos)[o] = p < 0 ? 0 : static_cast<const uint16_t*>(cosw)[off + i];
+      static_cast<uint16_t*>(tsin)[o] = p < 0 ? 0 : static_cast<const uint16_t*>(sinw)[off + i];
     } else {
-      static_cast<float*>(tcos)[o] = static_cast<const float*>(cosw)[off + i];
-      static_cast<float*>(tsin)[o] = static_cast<const float*>(sinw)[off + i];
+      static_cast<float*>(tcos)[o] = p < 0 ? 0.f : static_cast<const float*>(cosw)[off + i];
+      static_cast<float*>(tsin)[o] = p < 0 ? 0.f : static_cast<const float*>(sinw)[off + i];
     }
   }
 }
