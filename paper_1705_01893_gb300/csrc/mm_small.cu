@@ -497,19 +497,18 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(SmallParams q) {
       double* out = it == q.n_iter - 1 ? q.map_out : nullptr;
       for (int64_t p = 32 * ((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) + (threadIdx.x & 31); p < q.n_pix;
            p += (int64_t)gridDim.x * kSmallThreads) {
-        double a[NC], m[NC];
+        double a[NC], m[NC], w[NC == 3 ? 6 : 1];
 #pragma unroll
-        for (int k = 0; k < NC; ++k) {
-          a[k] = __ldcg(q.acc + k * stride + p);
-          q.acc[k * stride + p] = 0.0;
-        }
+        for (int k = 0; k < NC; ++k) a[k] = __ldcg(q.acc + k * stride + p);
+#pragma unroll
+        for (int k = 0; k < (NC == 3 ? 6 : 1); ++k) w[k] = __ldg(q.W + (NC == 3 ? 6 : 1) * p + k);
+        // every load before the first store
+#pragma unroll
+        for (int k = 0; k < NC; ++k) q.acc[k * stride + p] = 0.0;
         if constexpr (NC == 1) {
-          m[0] = __ldg(q.W + p) * a[0];
+          m[0] = w[0] * a[0];
           reinterpret_cast<float*>(q.map4)[p] = (float)m[0];
         } else {
-          double w[6];
-#pragma unroll
-          for (int k = 0; k < 6; ++k) w[k] = __ldg(q.W + 6 * p + k);
           m[0] = w[0] * a[0] + w[1] * a[1] + w[2] * a[2];
           m[1] = w[1] * a[0] + w[3] * a[1] + w[4] * a[2];
           m[2] = w[2] * a[0] + w[4] * a[1] + w[5] * a[2];
@@ -605,6 +604,19 @@ static int small_limit(bool general, int ncomp) {
   return general ? 6144 : ncomp == 1 ? 5120 : 4096;
 }
 
+// Pixels up to which a plan takes this path: its map step runs on its own CTAs, at about 3.2 ns a
+// pixel and CTA (IQU; T-only 0.55), against the whole GPU in a launch of its own; and beyond the
+// second limits the sums, weights and map no longer stay in L2.  Per iteration against the
+// three-kernel path, IQU, 2^12 samples (8 CTAs): 2^15 pixels 21.9 / 23.0 us, 2^16 35.1 / 24.0, 2^20
+// 437 / 51.7; 2^15 samples (16 CTAs): 2^16 pixels 26.1 / 28.5, 2^17 39.4 / 31.2; 4 x 2^15 samples (64 CTAs):
+// 2^18 pixels 28.0 / 35.0, 2^19 41.5 / 40.3, 2^20 148 / 57.2; 12 ragged chunks: 2^19 pixels 31.0 / 49.7,
+// 2^20 99.5 / 71.1.  T-only: 2^12 samples: 2^17 pixels 17.4 / 23.0, 2^18 26.4 / 23.0; 4 x 2^15 samples: 2^20
+// pixels 23.4 / 32.7, 2^21 32.5 / 35.5, 2^22 186 / 48.3; 40 x 2^13: 2^21 pixels 30.8 / 39.6, 2^22 100 / 51.1.
+static int64_t small_pixels(int ctas, int ncomp) {
+  const int64_t per_cta = (int64_t)ctas * (ncomp == 1 ? 20480 : 4096), l2 = ncomp == 1 ? 1 << 21 : 1 << 19;
+  return per_cta < l2 ? per_cta : l2;
+}
+
 template <int NC>
 static cudaError_t small_plan_nc(const mm_plan_s* p, SmallShape* out) {
   *out = SmallShape{};
@@ -639,7 +651,8 @@ static cudaError_t small_plan_nc(const mm_plan_s* p, SmallShape* out) {
     if (cl > best.clusters) best = SmallShape{S, cl, tile, tables, 0};
   }
   if (best.clusters > 0 &&
-      (int64_t)best.tile * ((p->n_chunks + best.clusters - 1) / best.clusters) <= limit)
+      (int64_t)best.tile * ((p->n_chunks + best.clusters - 1) / best.clusters) <= limit &&
+      p->n_pix <= small_pixels(best.S * best.clusters, NC))
     *out = best;
   return cudaSuccess;
 }
