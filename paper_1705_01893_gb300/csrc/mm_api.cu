@@ -767,38 +767,42 @@ __global__ void k_pixel_solve(int64_t n_pix, int ncomp, double rcond_min,
                               uint8_t* __restrict__ valid, double* __restrict__ W,
                               double* __restrict__ Minv, unsigned long long* n_valid) {
   const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (p >= n_pix) return;
-  bool ok = hits[p] >= 1;
-  if (ncomp == 1) {
-    const double a = acc12[2 * p], b = acc12[2 * p + 1];
-    ok = ok && a > 0.0 && b > 0.0;
-    W[p] = ok ? 1.0 / a : 0.0;
-    Minv[p] = ok ? 1.0 / b : 0.0;
-  } else {
-    double A[12];
+  bool ok = false;
+  if (p < n_pix) {
+    ok = hits[p] >= 1;
+    if (ncomp == 1) {
+      const double a = acc12[2 * p], b = acc12[2 * p + 1];
+      ok = ok && a > 0.0 && b > 0.0;
+      W[p] = ok ? 1.0 / a : 0.0;
+      Minv[p] = ok ? 1.0 / b : 0.0;
+    } else {
+      double A[12];
 #pragma unroll
-    for (int i = 0; i < 6; ++i) {   // 96 bytes per pixel, 16 at a time
-      const double2 v = reinterpret_cast<const double2*>(acc12 + 12 * p)[i];
-      A[2 * i] = v.x;
-      A[2 * i + 1] = v.y;
-    }
-    double wi[6] = {0, 0, 0, 0, 0, 0}, mi[6] = {0, 0, 0, 0, 0, 0};
-    if (ok && !sym3_surely_kept(A, rcond_min)) {
-      double emin, emax;
-      sym3_eig(A, &emin, &emax);
-      ok = emax > 0.0 && emin / emax >= rcond_min;
-    }
-    if (ok) ok = sym3_inv(A, wi) && sym3_inv(A + 6, mi);
-    if (!ok)
-      for (int i = 0; i < 6; ++i) wi[i] = mi[i] = 0.0;
+      for (int i = 0; i < 6; ++i) {   // 96 bytes per pixel, 16 at a time
+        const double2 v = reinterpret_cast<const double2*>(acc12 + 12 * p)[i];
+        A[2 * i] = v.x;
+        A[2 * i + 1] = v.y;
+      }
+      double wi[6] = {0, 0, 0, 0, 0, 0}, mi[6] = {0, 0, 0, 0, 0, 0};
+      if (ok && !sym3_surely_kept(A, rcond_min)) {
+        double emin, emax;
+        sym3_eig(A, &emin, &emax);
+        ok = emax > 0.0 && emin / emax >= rcond_min;
+      }
+      if (ok) ok = sym3_inv(A, wi) && sym3_inv(A + 6, mi);
+      if (!ok)
+        for (int i = 0; i < 6; ++i) wi[i] = mi[i] = 0.0;
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      reinterpret_cast<double2*>(W + 6 * p)[i] = make_double2(wi[2 * i], wi[2 * i + 1]);
-      reinterpret_cast<double2*>(Minv + 6 * p)[i] = make_double2(mi[2 * i], mi[2 * i + 1]);
+      for (int i = 0; i < 3; ++i) {
+        reinterpret_cast<double2*>(W + 6 * p)[i] = make_double2(wi[2 * i], wi[2 * i + 1]);
+        reinterpret_cast<double2*>(Minv + 6 * p)[i] = make_double2(mi[2 * i], mi[2 * i + 1]);
+      }
     }
+    valid[p] = ok ? 1 : 0;
   }
-  valid[p] = ok ? 1 : 0;
-  const unsigned act = __activemask(), kept = __ballot_sync(act, ok);
+  // every lane votes, those past the map and those cut among them: after divergent branches a vote
+  // of the lanes that happen to be active could leave out lane 0, which adds
+  const unsigned kept = __ballot_sync(0xffffffffu, ok);
   if ((threadIdx.x & 31) == 0 && kept) atomicAdd(n_valid, (unsigned long long)__popc(kept));
 }
 
