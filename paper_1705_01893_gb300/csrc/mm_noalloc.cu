@@ -92,11 +92,14 @@ __global__ void k_noalloc_solve(const double* __restrict__ s, int64_t n_pix, int
   if (!(det > 0.0) && !(det < 0.0)) return;
   const double c11 = A * F - C * C, c12 = B * C - A * E, c22 = A * D - B * B;
   const double b0 = a[6], b1 = a[7], b2 = a[8];
-  // quotients by one reciprocal and a residual step each (FP64 divisions are several times that)
+  // quotients by one reciprocal and a residual step each (FP64 divisions are several times that);
+  // without the step where the quotient is not finite (an infinite sample: its residual is NaN).
+  // 1 / det is finite: det is far above FP64's smallest for weights and hits of FP32's range.
   const double id = 1.0 / det;
   auto over = [&](double v) {
     const double r = v * id;
-    return fma(fma(-r, det, v), id, r);
+    const double f = fma(fma(-r, det, v), id, r);
+    return (__double2hiint(r) & 0x7ff00000) == 0x7ff00000 ? r : f;
   };
   o[0] = over(c00 * b0 + c01 * b1 + c02 * b2);
   o[1] = over(c01 * b0 + c11 * b1 + c12 * b2);
