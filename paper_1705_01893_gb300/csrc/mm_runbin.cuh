@@ -35,7 +35,8 @@ constexpr int kBinWarps = 8, kBinThreads = 32 * kBinWarps;
 // Op: NF float streams per sample (load), NV sums per run (add), NO outputs per run (emit).
 // Samples [n0, n1); samples with a pixel outside [0, n_pix) are skipped.  Op::tile(first,
 // last, shared) prepares per-tile state (every thread, before a barrier); Op::cut(i) marks a tile
-// position that starts a run whatever its pixel.
+// position that starts a run whatever its pixel; Op::kPerSample, Op::one(pixel, s): a single sum
+// that may go out sample by sample.
 template <class Op>
 __global__ void __launch_bounds__(kBinThreads) k_run_bin(Op op, const int32_t* __restrict__ pix,
                                                          int64_t n0, int64_t n1, int64_t n_pix, int segs) {
@@ -54,6 +55,31 @@ __global__ void __launch_bounds__(kBinThreads) k_run_bin(Op op, const int32_t* _
   for (int g = 0; g < segs; ++g) {
     const int at = ((g * kBinWarps + warp) * 32 + lane) * 4;   // the lane's first sample in the tile
     if (tile + at - 4 * lane >= n1) break;   // warp-uniform
+    // One sum a run and short runs: a reduction per sample, 32 consecutive samples at a time, is
+    // the cheaper way (a run's sums of one word gain nothing from being handed out again).  P^T of
+    // 8 M T-only samples, by samples per pixel, so / by runs: 1: 26.0 / 47.4 us, 3: 26.1 / 30.9,
+    // 4: 26.3 / 29.0, 16: 43.4 / 31.0; hence from 24 runs in 128 samples on (the count makes long
+    // runs 2 us slower).
+    if constexpr (Op::kPerSample) {
+      int q[4], heads = 0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int64_t s = tile + at - 3 * lane + 32 * u;
+        q[u] = s < n1 ? pix[s] : -1;
+        if (q[u] >= n_pix) q[u] = -1;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int before = __shfl_up_sync(0xffffffffu, q[u], 1);
+        heads += __popc(__ballot_sync(0xffffffffu, q[u] >= 0 && (lane == 0 || q[u] != before)));
+      }
+      if (heads >= 24) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (q[u] >= 0) op.one(q[u], tile + at - 3 * lane + 32 * u);
+        continue;
+      }
+    }
     int p[5];
     float f[4][NF > 0 ? NF : 1];
 #pragma unroll
@@ -118,6 +144,7 @@ static cudaError_t launch_run_bin(const Op& op, const int32_t* pix, int64_t n0, 
 template <int NC>
 struct BinPT {
   static constexpr int NF = NC == 3 ? 3 : 1, NV = NC, NO = NC;
+  static constexpr bool kPerSample = NC == 1;
   const float* tod;
   const void *cosw, *sinw;
   int half_w;
@@ -139,6 +166,7 @@ struct BinPT {
   __device__ void emit(int p, int o, const double* v, int64_t, const double*) const {
     atomicAdd(out + (int64_t)NC * p + o, v[o]);
   }
+  __device__ void one(int p, int64_t s) const { atomicAdd(out + p, widen(tod[s])); }   // NC = 1
 };
 
 // Normal-equation sums of the unit-weight binned map, kStride doubles per pixel: hits, then
@@ -146,6 +174,7 @@ struct BinPT {
 template <int NC, int kStride>
 struct BinNormal {
   static constexpr int NF = NC == 3 ? 3 : 1, NV = NC == 3 ? 9 : 2, NO = NV;
+  static constexpr bool kPerSample = false;
   const float* tod;
   const void *cosw, *sinw;
   int half_w;
@@ -184,6 +213,7 @@ struct BinNormal {
 template <int NC>
 struct BinWeights {
   static constexpr int NF = NC == 3 ? 2 : 0, NV = NC == 3 ? 6 : 1, NO = 2 * NV;
+  static constexpr bool kPerSample = false;
   const ChunkDesc* desc;
   int n_chunks;
   const void *cosw, *sinw;
