@@ -204,11 +204,18 @@ __device__ __forceinline__ void gpass_rows(const float2* src, float2* dst, int L
 }
 
 #define GEN_RADICES(X) X(2) X(3) X(4) X(5) X(6) X(8) X(9) X(10) X(15) X(16)
+// kWide: the iterations' radices; otherwise those of the data transform's plan (radix_plan), whose
+// kernels then need 40 to 64 registers instead of 64 to 80: with the wide ones compiled in, the rfft
+// of 1000 chunks of 3000 samples took 80.2 us, 69.4 before them, 61.2 without.
+template <bool kWide>
+__device__ __forceinline__ constexpr bool gen_has_radix(int r) {
+  return kWide || r <= 5 || r == 8;
+}
 
 // All passes of the row DFTs of a job.  kFirst: the first pass reads the intermediate (nothing
 // is in the tiles), otherwise tile a holds the input; kLast: the last pass writes the
 // intermediate.  Returns the tile that holds the result (kLast smem).
-template <int DIR, int kFirst, int kLast>
+template <int DIR, int kFirst, int kLast, bool kWide = true>
 __device__ float2* gen_dft_rows(float2* a, float2* b, int L, int nr, const int8_t* rad, const float2* tw,
                                 int nseq, int T, const RowIO& io) {
   int Ns = 1;
@@ -225,19 +232,19 @@ __device__ float2* gen_dft_rows(float2* a, float2* b, int L, int nr, const int8_
     const bool g_in = kFirst == kGlobal && p == 0, g_out = kLast == kGlobal && p == nr - 1;
     if (g_in) {      // into b: the swap below makes it the next source
       switch (R) {
-#define X(r) case r: gpass_rows<r, DIR, kGlobal, kSmem>(a, b, L, Ns, nseq, tw, T, io); break;
+#define X(r) case r: if constexpr (gen_has_radix<kWide>(r)) gpass_rows<r, DIR, kGlobal, kSmem>(a, b, L, Ns, nseq, tw, T, io); break;
         GEN_RADICES(X)
 #undef X
       }
     } else if (g_out) {
       switch (R) {
-#define X(r) case r: gpass_rows<r, DIR, kSmem, kGlobal>(a, b, L, Ns, nseq, tw, T, io); break;
+#define X(r) case r: if constexpr (gen_has_radix<kWide>(r)) gpass_rows<r, DIR, kSmem, kGlobal>(a, b, L, Ns, nseq, tw, T, io); break;
         GEN_RADICES(X)
 #undef X
       }
     } else {
       switch (R) {
-#define X(r) case r: gpass_rows<r, DIR, kSmem, kSmem>(a, b, L, Ns, nseq, tw, T, io); break;
+#define X(r) case r: if constexpr (gen_has_radix<kWide>(r)) gpass_rows<r, DIR, kSmem, kSmem>(a, b, L, Ns, nseq, tw, T, io); break;
         GEN_RADICES(X)
 #undef X
       }
@@ -251,7 +258,7 @@ __device__ float2* gen_dft_rows(float2* a, float2* b, int L, int nr, const int8_
 }
 
 // All passes of the column DFTs of a tile, ends as above.
-template <int DIR, int kFirst, int kLast>
+template <int DIR, int kFirst, int kLast, bool kWide = true>
 __device__ float2* gen_dft_cols(float2* a, float2* b, int L, int nr, const int8_t* rad, const float2* tw,
                                 int NB, int lnb, int T, const ColIO& io) {
   int Ns = 1;
@@ -269,19 +276,19 @@ __device__ float2* gen_dft_cols(float2* a, float2* b, int L, int nr, const int8_
     const bool g_in = kFirst == kGlobal && p == 0, g_out = kLast == kGlobal && p == nr - 1;
     if (g_in) {
       switch (R) {
-#define X(r) case r: gpass_cols<r, DIR, kGlobal, kSmem>(a, b, L, Ns, NB, lnb, tw, T, io); break;
+#define X(r) case r: if constexpr (gen_has_radix<kWide>(r)) gpass_cols<r, DIR, kGlobal, kSmem>(a, b, L, Ns, NB, lnb, tw, T, io); break;
         GEN_RADICES(X)
 #undef X
       }
     } else if (g_out) {
       switch (R) {
-#define X(r) case r: gpass_cols<r, DIR, kSmem, kGlobal>(a, b, L, Ns, NB, lnb, tw, T, io); break;
+#define X(r) case r: if constexpr (gen_has_radix<kWide>(r)) gpass_cols<r, DIR, kSmem, kGlobal>(a, b, L, Ns, NB, lnb, tw, T, io); break;
         GEN_RADICES(X)
 #undef X
       }
     } else {
       switch (R) {
-#define X(r) case r: gpass_cols<r, DIR, kSmem, kSmem>(a, b, L, Ns, NB, lnb, tw, T, io); break;
+#define X(r) case r: if constexpr (gen_has_radix<kWide>(r)) gpass_cols<r, DIR, kSmem, kSmem>(a, b, L, Ns, NB, lnb, tw, T, io); break;
         GEN_RADICES(X)
 #undef X
       }
@@ -408,7 +415,7 @@ __device__ __forceinline__ void feed_put(GenChunk* dst, int lane, const int* w) 
 
 // ------------------------------------------------------------ kernel A: columns forward
 template <int NC, int SRC>
-__global__ void __launch_bounds__(512, 2) k_gen_col_forward(GenParams q) {
+__global__ void __launch_bounds__(512, SRC == kSrcTod ? 3 : 2) k_gen_col_forward(GenParams q) {
   extern __shared__ float2 gsm[];
   const int T = blockDim.x, NB = q.nb, lnb = NB == 16 ? 4 : 3;
   __shared__ TileFeed feed;
@@ -460,7 +467,7 @@ __global__ void __launch_bounds__(512, 2) k_gen_col_forward(GenParams q) {
     }
     const ColIO io{q.ybuf + (G.yoff - q.base_y), &G, M2, j2_0, width};
     if constexpr (SRC == kSrcTod)   // the data keep their own plan (see radix_plan)
-      gen_dft_cols<-1, kSmem, kGlobal>(a, b, M1, G.nr1d, G.rad1d, G.tw_col_d, NB, lnb, T, io);
+      gen_dft_cols<-1, kSmem, kGlobal, false>(a, b, M1, G.nr1d, G.rad1d, G.tw_col_d, NB, lnb, T, io);
     else
       gen_dft_cols<-1, kSmem, kGlobal>(a, b, M1, G.nr1, G.rad1, G.tw_col, NB, lnb, T, io);
   }
@@ -629,10 +636,12 @@ __global__ void __launch_bounds__(512, 2) k_gen_col_inverse(GenParams q) {
 // `count` consecutive pairs of rows (k1, M1 - k1), k1 = first .. first + count - 1; tile
 // sequence 2j holds row first + j and sequence 2j + 1 its partner.
 // MODE >= 0: the row mode folded in at compile time (the messenger step and its map-sized
-// form); -1: read from q.a.mode (set-up, PCG, chi^2, composite and the other modes).
-// MAXT: 256 (three CTAs an SM, 80 registers) or 1024 threads.
+// form); -1: read from q.a.mode (PCG, chi^2, composite and the other modes); kGenRowData: the
+// transform of the data (kRowSpectrum, kRowNatural).
+// MAXT: 256 (three CTAs an SM, 80 registers; the data transform four, 64) or 1024 threads.
+constexpr int kGenRowData = -2;
 template <int MODE, int MAXT>
-__global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1) k_gen_row(GenParams q) {
+__global__ void __launch_bounds__(MAXT, MAXT == 256 ? (MODE == kGenRowData ? 4 : 3) : 1) k_gen_row(GenParams q) {
   extern __shared__ float2 gsm[];
   __shared__ float red[32];
   // the current job and the next one: table entry, chunk record, tau, lambda tau, output scale.
@@ -643,12 +652,12 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1) k_gen_row(GenParams
   __shared__ float s_con[2][3];
   const int T = blockDim.x;
   const int mode = MODE >= 0 ? MODE : q.a.mode;
-  const bool fwd = mode != kRowPcgRhs && mode != kRowMd;
-  const bool mess = mode == kRowMessenger || mode == kRowMessengerF || mode == kRowMd;
-  const bool resid = mode == kRowResidual;
-  const bool inv = mess || resid || mode == kRowPcgApply || mode == kRowPcgRhs;
-  const bool load_d = mode != kRowSpectrum && mode != kRowNatural && mode != kRowPcgApply &&
-                      mode != kRowMessengerF;
+  constexpr bool data = MODE == kGenRowData;
+  const bool fwd = data || (mode != kRowPcgRhs && mode != kRowMd);
+  const bool mess = !data && (mode == kRowMessenger || mode == kRowMessengerF || mode == kRowMd);
+  const bool resid = !data && mode == kRowResidual;
+  const bool inv = !data && (mess || resid || mode == kRowPcgApply || mode == kRowPcgRhs);
+  const bool load_d = !data && mode != kRowPcgApply && mode != kRowMessengerF;
   double lambda = q.a.lambda;
   double* chi2 = q.a.chi2;
   if (q.a.lam_table) {          // graph mode: schedule and chi^2 slot from device memory
@@ -656,7 +665,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1) k_gen_row(GenParams
     lambda = q.a.lam_table[it];
     chi2 = q.a.chi2_base[0] ? q.a.chi2_base[0] + it : nullptr;
   }
-  const bool want_x2 = chi2 != nullptr &&
+  const bool want_x2 = !data && chi2 != nullptr &&
                        (mode == kRowMessenger || mode == kRowMessengerF || mode == kRowChi2 ||
                         mode == kRowPcgRhs || mode == kRowResidual);
   const bool lam_inf = (__double2hiint(lambda) & 0x7fffffff) == 0x7ff00000;
@@ -706,8 +715,8 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1) k_gen_row(GenParams
     float2* z = a;
     const RowIO io{y, &G, M1, M2, first, self};
     if (fwd) {
-      if (mode == kRowSpectrum || mode == kRowNatural)   // the data keep their own plan (see radix_plan)
-        z = gen_dft_rows<-1, kGlobal, kSmem>(a, b, M2, G.nr2d, G.rad2d, G.tw_row_d, nseq, T, io);
+      if constexpr (data)   // the data keep their own plan (see radix_plan)
+        z = gen_dft_rows<-1, kGlobal, kSmem, false>(a, b, M2, G.nr2d, G.rad2d, G.tw_row_d, nseq, T, io);
       else
         z = gen_dft_rows<-1, kGlobal, kSmem>(a, b, M2, G.nr2, G.rad2, G.tw_row, nseq, T, io);
     }
@@ -747,8 +756,8 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1) k_gen_row(GenParams
         const int k = r + M1 * p;
         const int ze = lay(e);
         const float2 X = fwd ? z[ze] : make_float2(0.f, 0.f);
-        if (mode == kRowSpectrum) { q.dtab[d.spec + slot] = X; continue; }
-        if (mode == kRowNatural) {
+        if (data && mode == kRowSpectrum) { q.dtab[d.spec + slot] = X; continue; }
+        if (data) {
           if (2 * k <= d.n) q.a.natural[d.nat + k] = X;
           continue;
         }
@@ -786,7 +795,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1) k_gen_row(GenParams
           act[u] = on; pv[u] = p; jv[u] = j; qv[u] = qi;
           Dk[u] = Dp[u] = make_float2(0.f, 0.f);
           nk[u] = np[u] = 0.f;
-          if (on && mode != kRowSpectrum && mode != kRowNatural) {
+          if (on && !data) {
             const int sk = (first + j) * M2 + p, sp = (self ? first : M1 - first - j) * M2 + qi;
             if (load_d) { Dk[u] = __ldcs(dt + sk); Dp[u] = __ldcs(dt + sp); }
             nk[u] = __ldcs(nb + sk);
@@ -804,8 +813,8 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1) k_gen_row(GenParams
           const float2 Zp = fwd ? z[ep] : make_float2(0.f, 0.f);
           if (rA == 0 && p == 0) {
             const float X0 = Zk.x + Zk.y, XM = Zk.x - Zk.y;
-            if (mode == kRowSpectrum) { q.dtab[d.spec] = make_float2(X0, XM); continue; }
-            if (mode == kRowNatural) {
+            if (data && mode == kRowSpectrum) { q.dtab[d.spec] = make_float2(X0, XM); continue; }
+            if (data) {
               q.a.natural[d.nat] = make_float2(X0, 0.f);
               q.a.natural[d.nat + M] = make_float2(XM, 0.f);
               continue;
@@ -829,12 +838,12 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1) k_gen_row(GenParams
           const float2 Xk = cadd(E, wO);
           const float2 Xp = cconj(csub(E, wO));
           const bool same = self && qi == p;                 // k == M - k
-          if (mode == kRowSpectrum) {
+          if (data && mode == kRowSpectrum) {
             q.dtab[d.spec + sk] = Xk;
             if (!same) q.dtab[d.spec + sp] = Xp;
             continue;
           }
-          if (mode == kRowNatural) {
+          if (data) {
             const int k = rA + M1 * p;
             q.a.natural[d.nat + k] = Xk;
             q.a.natural[d.nat + M - k] = Xp;
@@ -883,7 +892,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1) k_gen_row(GenParams
           // rows of general chunks need not start on 16 bytes: prefetch their aligned interior
           if (fwd) prefetch_l2_inner(yn + (int64_t)r * nM2, 8 * (size_t)nM2);
           if (load_d) prefetch_l2_inner(q.dtab + Gn.d.spec + (int64_t)r * nM2, 8 * (size_t)nM2);
-          prefetch_l2_inner(q.nbar + Gn.d.spec + (int64_t)r * nM2, 4 * (size_t)nM2);
+          if (!data) prefetch_l2_inner(q.nbar + Gn.d.spec + (int64_t)r * nM2, 4 * (size_t)nM2);
         }
       }
     }
@@ -1042,7 +1051,9 @@ cudaError_t launch_gen_row(const mm_plan_s* p, const Batch& b, const RowArgs& a,
   q.tile = emax + (emax >> 4) + 1;
   const size_t smem = 2 * sizeof(float2) * (size_t)q.tile;
   const bool narrow = p->gen_tune.row_threads <= 256;
-  auto k = a.mode == kRowMessenger    ? (narrow ? k_gen_row<kRowMessenger, 256> : k_gen_row<kRowMessenger, 1024>)
+  const bool data = a.mode == kRowSpectrum || a.mode == kRowNatural;
+  auto k = data                       ? (narrow ? k_gen_row<kGenRowData, 256> : k_gen_row<kGenRowData, 1024>)
+           : a.mode == kRowMessenger  ? (narrow ? k_gen_row<kRowMessenger, 256> : k_gen_row<kRowMessenger, 1024>)
            : a.mode == kRowMessengerF ? (narrow ? k_gen_row<kRowMessengerF, 256> : k_gen_row<kRowMessengerF, 1024>)
                                       : (narrow ? k_gen_row<-1, 256> : k_gen_row<-1, 1024>);
   return gen_launch(k, p->gen_tune.row_threads, smem, q.n_items, q, st);
