@@ -14,7 +14,11 @@ namespace mm {
 template <int M1, int CB, int T, int NC, int SRC, bool ROOMY>
 __global__ void __launch_bounds__(T, pass_ctas(T, 8, ROOMY)) k_col_forward(ColParams q) {
   extern __shared__ float2 sm[];
-  __shared__ float2 s4[SRC == kSrcTod ? 1 : four_step_n(M1, kColLo) * CB];
+  // the tile's four-step twiddles from shared memory, but for 32-point columns, which use each
+  // entry once (1000 x 2^12 samples, T-only: 4 iterations 266 us without, 276 with; 16 points, whose one
+  // pass hides the copy: 4000 x 2^10 328 / 311; 128 points and more: with)
+  constexpr bool kStage = SRC != kSrcTod && M1 != 32;
+  __shared__ float2 s4[kStage ? four_step_n(M1, kColLo) * CB : 1];
   const int M2 = q.g.M2;
   const int tpc = M2 / CB;
   const int ntiles = q.count * tpc;
@@ -25,12 +29,18 @@ __global__ void __launch_bounds__(T, pass_ctas(T, 8, ROOMY)) k_col_forward(ColPa
     const int j2_0 = cb * CB;
     if constexpr (SRC == kSrcTod) {
       smem_fft<M1, CB, ColLayout<CB>, T, -1>(sm, q.g.tw_col, SrcTod{q.tod, d.off + 2ll * j2_0, M2},
-                                             DstYData{q.ybuf + (int64_t)ci * d.M, &q.g, j2_0, M2});
+                                             DstYTable{q.ybuf + (int64_t)ci * d.M, &q.g, j2_0, M2});
     } else {
-      load_col_twiddles<M1, CB, T>(s4, q.g, cb);
       using Src = typename std::conditional<SRC == kSrcGather2, SrcGather2<NC, CB>, SrcGather<NC, CB>>::type;
-      smem_fft<M1, CB, ColLayout<CB>, T, -1>(sm, q.g.tw_col, Src{&q, d.off + (int64_t)cb * (2 * CB * M1)},
-                                             DstY<M1, CB, true>{q.ybuf + (int64_t)ci * d.M, s4, j2_0, M2});
+      const Src src{&q, d.off + (int64_t)cb * (2 * CB * M1)};
+      if constexpr (kStage) {
+        load_col_twiddles<M1, CB, T>(s4, q.g, cb);
+        smem_fft<M1, CB, ColLayout<CB>, T, -1>(sm, q.g.tw_col, src,
+                                               DstY<M1, CB, true>{q.ybuf + (int64_t)ci * d.M, s4, j2_0, M2});
+      } else {
+        smem_fft<M1, CB, ColLayout<CB>, T, -1>(sm, q.g.tw_col, src,
+                                               DstYTable{q.ybuf + (int64_t)ci * d.M, &q.g, j2_0, M2});
+      }
     }
     __syncthreads();
   }

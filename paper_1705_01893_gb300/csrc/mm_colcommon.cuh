@@ -49,14 +49,18 @@ __device__ __forceinline__ float4 load_w4(const void* w, int half_w, int64_t s) 
 // then one map load serves both: the gathers are short of L1 requests (a vertical sweep touches a line per
 // pixel), not of bytes.  256^2, 4 x 2^20: 1523 -> 1461 us per
 // 21 iterations; the 20-step gradient 6424 -> 6009 us; 512^2, 8 x 2^22: 435 -> 432 us an iteration.
-template <int NC>
+// kShare: on for IQU.  T-only loads are a quarter of the size, and the second one's wait for the
+// compare of the pixels costs more than it saves (forward columns of 250 x 2^14 samples 14.3 us
+// against 20.7, 1000 x 2^12 16.5 / 20.8; 16 x 2^18, 4 iterations: 220 / 228), but for the long columns
+// in narrower tiles (4 iterations of 2 x 2^24 samples 1369 us sharing, 1408 not; 4 x 2^23 1316 / 1324).
+template <int NC, bool kShare = NC == 3>
 __device__ __forceinline__ float2 gather_two(const ColParams& q, int p0, int p1, float c0, float c1,
                                              float s0, float s1) {
   if constexpr (NC == 1) {
     const float* map = reinterpret_cast<const float*>(q.map4);
     const float a = p0 < 0 ? 0.f : __ldg(map + p0);
     float b = a;
-    if (p1 != p0) b = p1 < 0 ? 0.f : __ldg(map + p1);
+    if (!kShare || p1 != p0) b = p1 < 0 ? 0.f : __ldg(map + p1);
     return make_float2(a, b);
   } else {
     const float4* map = reinterpret_cast<const float4*>(q.map4);
@@ -240,7 +244,7 @@ struct SrcGather {   // z = ((P m)_s, (P m)_s+1), Eq. 1; tile-ordered pointing f
         cw0 = c.x; cw1 = c.y; sw0 = w.x; sw1 = w.y;
       }
     }
-    return gather_two<NC>(*q, p.x, p.y, cw0, cw1, sw0, sw1);
+    return gather_two<NC, NC == 3 || (CB < kColCB)>(*q, p.x, p.y, cw0, cw1, sw0, sw1);
   }
 };
 
@@ -299,10 +303,10 @@ struct DstY {
   }
 };
 
-// The same with the plan-wide two-level table, for the transform of the data: it runs once per
+// The same with the plan-wide two-level table, for 32-point columns and the transform of the data: that runs once per
 // data set, and its rounding reaches every later iterate through d~ (1/f noise spreads it over
 // the high frequencies), so it stays as it was.
-struct DstYData {
+struct DstYTable {
   float2* y;
   const Group* g;
   int j2_0;
