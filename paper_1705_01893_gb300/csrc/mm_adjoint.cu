@@ -346,7 +346,7 @@ static cudaError_t row_adjoint_m2(const mm_plan_s* p, const Batch& b, float2* yV
   q.acc = acc;
   const bool theta = rspec != nullptr;
   const size_t smem = sizeof(float2) * (2 * M2 + tw_size(M2));
-  constexpr bool R = T != 512;
+  constexpr bool R = T < 512;
   auto roomy = theta ? k_row_adjoint<M2, T, true, R> : k_row_adjoint<M2, T, false, R>;
   auto k = theta ? k_row_adjoint<M2, T, true, false> : k_row_adjoint<M2, T, false, false>;
   int grid = 0;
@@ -397,7 +397,7 @@ static cudaError_t col_adjoint_m1(const mm_plan_s* p, const Batch& b, const AdjC
   const size_t smem = sizeof(float2) * M1 * kColCB;
   int grid = 0;
   cudaError_t e;
-  constexpr bool R = T != 512;
+  constexpr bool R = T < 512;
   auto roomy = p->ncomp == 3 ? k_col_inverse_adjoint<M1, kColCB, T, 3, THETA, R> : k_col_inverse_adjoint<M1, kColCB, T, 1, THETA, R>;
   auto k = p->ncomp == 3 ? k_col_inverse_adjoint<M1, kColCB, T, 3, THETA, false> : k_col_inverse_adjoint<M1, kColCB, T, 1, THETA, false>;
   if ((e = pass_grid(roomy, k, T, smem, ntiles, &k, &grid)) != cudaSuccess) return e;

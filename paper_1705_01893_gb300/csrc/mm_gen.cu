@@ -636,12 +636,11 @@ __global__ void __launch_bounds__(512, 2) k_gen_col_inverse(GenParams q) {
 // `count` consecutive pairs of rows (k1, M1 - k1), k1 = first .. first + count - 1; tile
 // sequence 2j holds row first + j and sequence 2j + 1 its partner.
 // MODE >= 0: the row mode folded in at compile time (the messenger step and its map-sized
-// form); -1: read from q.a.mode (PCG, chi^2, composite and the other modes); kGenRowData: the
+// form); -1: read from q.a.mode (PCG, chi^2, composite and the other modes); kRowDataModes: the
 // transform of the data (kRowSpectrum, kRowNatural).
 // MAXT: 256 (three CTAs an SM, 80 registers; the data transform four, 64) or 1024 threads.
-constexpr int kGenRowData = -2;
 template <int MODE, int MAXT>
-__global__ void __launch_bounds__(MAXT, MAXT == 256 ? (MODE == kGenRowData ? 4 : 3) : 1) k_gen_row(GenParams q) {
+__global__ void __launch_bounds__(MAXT, MAXT == 256 ? (MODE == kRowDataModes ? 4 : 3) : 1) k_gen_row(GenParams q) {
   extern __shared__ float2 gsm[];
   __shared__ float red[32];
   // the current job and the next one: table entry, chunk record, tau, lambda tau, output scale.
@@ -652,7 +651,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? (MODE == kGenRowData ? 4 :
   __shared__ float s_con[2][3];
   const int T = blockDim.x;
   const int mode = MODE >= 0 ? MODE : q.a.mode;
-  constexpr bool data = MODE == kGenRowData;
+  constexpr bool data = MODE == kRowDataModes;
   const bool fwd = data || (mode != kRowPcgRhs && mode != kRowMd);
   const bool mess = !data && (mode == kRowMessenger || mode == kRowMessengerF || mode == kRowMd);
   const bool resid = !data && mode == kRowResidual;
@@ -1052,7 +1051,7 @@ cudaError_t launch_gen_row(const mm_plan_s* p, const Batch& b, const RowArgs& a,
   const size_t smem = 2 * sizeof(float2) * (size_t)q.tile;
   const bool narrow = p->gen_tune.row_threads <= 256;
   const bool data = a.mode == kRowSpectrum || a.mode == kRowNatural;
-  auto k = data                       ? (narrow ? k_gen_row<kGenRowData, 256> : k_gen_row<kGenRowData, 1024>)
+  auto k = data                       ? (narrow ? k_gen_row<kRowDataModes, 256> : k_gen_row<kRowDataModes, 1024>)
            : a.mode == kRowMessenger  ? (narrow ? k_gen_row<kRowMessenger, 256> : k_gen_row<kRowMessenger, 1024>)
            : a.mode == kRowMessengerF ? (narrow ? k_gen_row<kRowMessengerF, 256> : k_gen_row<kRowMessengerF, 1024>)
                                       : (narrow ? k_gen_row<-1, 256> : k_gen_row<-1, 1024>);

@@ -713,6 +713,10 @@ struct RowArgs {
   double* const* chi2_base = nullptr;
 };
 
+// Row kernel instances: MODE >= 0 one mode, -1 any but the data transform's, kRowDataModes its two
+// (kRowSpectrum, kRowNatural).
+constexpr int kRowDataModes = -2;
+
 // Source of the forward column pass.
 enum ColSrc { kSrcGather = 0, kSrcTod = 1, kSrcGather2 = 2 /* composite pointing */ };
 
@@ -760,7 +764,7 @@ __host__ __device__ constexpr int col_cb(int M1) { return M1 <= 512 ? kColCB : 8
 // at most 50 bytes of spills.  The roomy one runs launches that it holds in one wave anyway (2
 // chunks of 2^18 samples, 3 iterations: 145 us, capped 150); beyond, the full SM pays (256^2,
 // 4 x 2^20 iteration, rows of 1024 points: 83 -> 73 us; the 20-step gradient on the same data 7.21
-// -> 6.39 ms).  The 512-thread shapes have one instance.
+// -> 6.39 ms).  The shapes of 512 and more threads have one instance.
 __host__ __device__ constexpr int pass_ctas(int threads, int below128, bool roomy) {
   return threads > 512 ? 1 : threads == 512 || roomy ? 2 : threads >= 128 ? 1024 / threads : below128;
 }

@@ -86,11 +86,12 @@ __device__ __forceinline__ void kernel_body_job(const RowParams& q, float2* sm, 
   const bool self = rA == rB;
   const int mode = MODE >= 0 ? MODE : q.a.mode;   // compile-time for the hot mode
   float2* y = q.ybuf + (int64_t)ci * d.M;
-  const bool fwd = mode != kRowPcgRhs && mode != kRowMd;
-  const bool mess = mode == kRowMessenger || mode == kRowMessengerF || mode == kRowMd ||
-                    mode == kRowMessengerKeep;
-  const bool resid = mode == kRowResidual;
-  const bool inv = mess || resid || mode == kRowPcgApply || mode == kRowPcgRhs;
+  constexpr bool data = MODE == kRowDataModes;    // the other instances have none of these modes
+  const bool fwd = data || (mode != kRowPcgRhs && mode != kRowMd);
+  const bool mess = !data && (mode == kRowMessenger || mode == kRowMessengerF || mode == kRowMd ||
+                              mode == kRowMessengerKeep);
+  const bool resid = !data && mode == kRowResidual;
+  const bool inv = !data && (mess || resid || mode == kRowPcgApply || mode == kRowPcgRhs);
 
   // The job's constants come from thread 0: FP64 products and conversions in every warp, and a
   // chain of them in thread 0 that all others wait for, held up each job by 2 to 3 of 46
@@ -98,7 +99,7 @@ __device__ __forceinline__ void kernel_body_job(const RowParams& q, float2* sm, 
   __shared__ float s_con[3];    // tau, lambda tau, lambda
   double* chi2 = q.a.chi2;
   bool lam_inf = false;
-  {
+  if constexpr (!data) {
     double lambda = q.a.lambda;
     if (q.a.lam_table) {          // graph mode: schedule and chi^2 slot from device memory
       const int it = *q.a.iter;
@@ -121,7 +122,7 @@ __device__ __forceinline__ void kernel_body_job(const RowParams& q, float2* sm, 
   }
 
   // per-mode constants
-  const float tau = s_con[0], lt = s_con[1];
+  const float tau = data ? 1.f : s_con[0], lt = data ? 0.f : s_con[1];
   const float inv_n = 1.0f / (float)d.n;
   if (!mess && !resid) lam_inf = false;
   // N' = Nbar + cn for chi^2: tau (Eq. 3) or lambda tau (chi^2(m, lambda))
@@ -145,12 +146,11 @@ __device__ __forceinline__ void kernel_body_job(const RowParams& q, float2* sm, 
     if (mode == kRowPcgApply) return cscale(X, __fdividef(sc, nbv + tau));
     return cscale(D, __fdividef(sc, nbv + tau));  // kRowPcgRhs
   };
-  const bool want_x2 = chi2 != nullptr &&
+  const bool want_x2 = !data && chi2 != nullptr &&
                        (mode == kRowMessenger || mode == kRowMessengerF || mode == kRowChi2 ||
                         mode == kRowChi2Modes || resid ||
                         mode == kRowPcgRhs);
-  const bool spec_out = mode == kRowSpectrum || mode == kRowNatural;
-  const bool load_d = !spec_out && mode != kRowPcgApply && mode != kRowMessengerF;
+  const bool load_d = !data && mode != kRowPcgApply && mode != kRowMessengerF;
 
   // Pairs (k, M - k): p in row rA with partner qi in row rB (or in row rA itself when the
   // row pairs with itself).  PB pairs per thread have their d~ / Nbar loads in flight at once.
@@ -173,7 +173,7 @@ __device__ __forceinline__ void kernel_body_job(const RowParams& q, float2* sm, 
       act[u] = a; qsv[u] = qs; qiv[u] = qi;
       Dk[u] = Dp[u] = make_float2(0.f, 0.f);
       nk[u] = np[u] = 0.f;
-      if (a && !spec_out) {
+      if (a && !data) {
         const int sk = rA * M2 + p, sp = (qs ? rB : rA) * M2 + qi;
         if (load_d) { Dk[u] = __ldcs(dt + sk); Dp[u] = __ldcs(dt + sp); }
         nk[u] = __ldcs(nb + sk);
@@ -194,8 +194,8 @@ __device__ __forceinline__ void kernel_body_job(const RowParams& q, float2* sm, 
         // k = 0 and k = M (both real): X_0 = Re Z_0 + Im Z_0, X_M = Re Z_0 - Im Z_0;
         // slot 0 of d~ holds (d~_0, d~_M) and the Nyquist Nbar is kept per chunk
         const float X0 = Zk.x + Zk.y, XM = Zk.x - Zk.y;
-        if (mode == kRowSpectrum) { q.dtab[d.spec] = make_float2(X0, XM); continue; }
-        if (mode == kRowNatural) {
+        if (data && mode == kRowSpectrum) { q.dtab[d.spec] = make_float2(X0, XM); continue; }
+        if (data) {
           float2* o = q.a.natural + d.nat;
           o[0] = make_float2(X0, 0.f);
           o[M] = make_float2(XM, 0.f);
@@ -229,12 +229,12 @@ __device__ __forceinline__ void kernel_body_job(const RowParams& q, float2* sm, 
       const float2 Xk = cadd(E, wO);
       const float2 Xp = cconj(csub(E, wO));
       const bool same = (qs == 0 && qi == p);   // k == M - k (k = M/2)
-      if (mode == kRowSpectrum) {
+      if (data && mode == kRowSpectrum) {
         q.dtab[d.spec + sk] = Xk;
         if (!same) q.dtab[d.spec + sp] = Xp;
         continue;
       }
-      if (mode == kRowNatural) {
+      if (data) {
         float2* o = q.a.natural + d.nat;
         const int k = rA + M1 * p;
         o[k] = Xk;
