@@ -573,7 +573,7 @@ struct NoiseArgs {
 // 1 <= m < 2, and m's leading 11 bits t (1024 <= t < 2048), m = (t / 1024) (1 + d), d < 2^-10:
 //   sigma^2 (f_knee / f)^alpha = A_e B_t (1 + d)^-alpha,
 //   A_e = sigma^2 (f_knee / (2^e f_1))^alpha,  B_t = (t / 1024)^-alpha,  f_1 = f_sample / n,
-// and (1 + d)^-alpha by its binomial series to d^5 (the next term is below 3e-17 for
+// and (1 + d)^-alpha by its binomial series to d^5 (the next term is at most 84 d^6 < 8e-17 for
 // |alpha| <= 4, the range the tables are used in).  A chunk's table: 1024 pairs
 // (B_t, 1024 / t), then A_e for e = 0 .. 31 in the x parts of 32 more.  A pow and two
 // divisions per mode on the narrow FP64 pipe took 4.13 ms for 8 x 2^22 samples.
