@@ -224,6 +224,9 @@ static size_t tw_count(int M, int M1, int M2, bool general) {
 
 // Pairs in a chunk's power-law table (see k_noise_table).
 constexpr int kNoiseTable = 1024 + 32;
+// Bins of the longest chunk from which a plan keeps tables (17 KB a chunk): they pay from about
+// their own length on, 1056 pow a chunk.
+constexpr int kNoiseTableBins = 8 * kNoiseTable;
 
 // -------------------------------------------------------------------- workspace layout
 struct Layout {
@@ -232,6 +235,7 @@ struct Layout {
       adapt, queue, fitems, fctr, fault, small, total, ybytes;
   int64_t gen_ccap, gen_rcap;
   int lam_cap;
+  bool tables;             // power-law tables of the noise model are kept
   int n_groups;
   int gM[kMaxGroups], gM1[kMaxGroups], gM2[kMaxGroups], gcount[kMaxGroups], gbatch[kMaxGroups];
   int gn[kMaxGroups], ggen[kMaxGroups], gcplx[kMaxGroups];
@@ -367,7 +371,10 @@ static mm_status make_layout(int n_chunks, const int64_t* off, int64_t n_pix, in
   L->desc = take(sizeof(ChunkDesc) * n_chunks);
   L->chunks = take(sizeof(int) * n_chunks);
   L->params = take(sizeof(double) * 4 * n_chunks);
-  L->ntab = take(sizeof(double2) * kNoiseTable * (size_t)n_chunks);
+  int max_m = 0;
+  for (int g = 0; g < L->n_groups; ++g) max_m = L->gM[g] > max_m ? L->gM[g] : max_m;
+  L->tables = max_m >= kNoiseTableBins;
+  L->ntab = take(L->tables ? sizeof(double2) * kNoiseTable * (size_t)n_chunks : 0);
   L->tw = take(sizeof(float2) * tw);
   L->hits = take(sizeof(int32_t) * np);
   L->valid = take(np);
@@ -1397,7 +1404,7 @@ static mm_status plan_create(mm_plan* out, int n_chunks, const int64_t* offsets,
   p->params = reinterpret_cast<double*>(ws + L.params);
   p->small_bar = reinterpret_cast<unsigned*>(ws + L.small);
   p->small_rec = reinterpret_cast<GenChunk*>(ws + L.small + 256);
-  p->noise_tab = reinterpret_cast<double2*>(ws + L.ntab);
+  p->noise_tab = L.tables ? reinterpret_cast<double2*>(ws + L.ntab) : nullptr;
   p->tpix = reinterpret_cast<int32_t*>(ws + L.tpix);
   p->tcos = ncomp == 3 ? static_cast<void*>(ws + L.tcos) : nullptr;
   p->tsin = ncomp == 3 ? static_cast<void*>(ws + L.tsin) : nullptr;
@@ -1684,8 +1691,7 @@ extern "C" mm_status mm_set_noise_psd(mm_plan p, const double* psd_dev, const do
     for (int c = 0; c < C; ++c) maxM = p->h_desc[c].M > maxM ? p->h_desc[c].M : maxM;
     const int per = 256 * 16;
     const dim3 grid((maxM + per - 1) / per, C);
-    // tables pay from about their own length on (1056 pow a chunk)
-    if (d_params && maxM >= 8 * kNoiseTable) {
+    if (d_params && p->noise_tab) {
       k_noise_table<<<dim3(blocks_for(kNoiseTable, 64), C), 64, 0, s>>>(p->d_desc, d_params, p->noise_tab);
       LAUNCHED("k_noise_table");
       k_noise<true><<<grid, 256, 0, s>>>(na);

@@ -194,7 +194,7 @@ struct mm_plan_s {
   int check_on_return; // 1: the solver calls synchronise and report an expired wait
   double* scal;     // [64] scalars (see kScal*)
   double* params;   // [n_chunks][4] noise parameters (device copy)
-  double2* noise_tab;  // power-law tables of the chunks (set-up)
+  double2* noise_tab;  // power-law tables of the chunks (set-up), or nullptr
   float2* tw_pool;
   // general path: chunk list in plan order and per-chunk prefix sums over it (column tiles,
   // row jobs, intermediate elements), device and host copies; device copy of the groups
