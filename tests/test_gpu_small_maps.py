@@ -50,3 +50,15 @@ def test_both_sides_of_the_limit(ncomp, limit, over):
     plan.messenger(m, [math.inf, 5.0, 1.0])
     ref, _ = O.run_messenger(prob, [math.inf, 5.0, 1.0])
     assert np.linalg.norm(m.cpu().numpy() - ref) <= 1e-5 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("ncomp", [1, 3])
+@pytest.mark.parametrize("over", [0, 1, 255, 511])
+def test_two_pixels_a_thread(ncomp, over):
+    """The map step's two-pixel form, from 2^19 pixels on, at the ends of its last block."""
+    npix = (1 << 19) + over
+    plan, prob = _plan([1 << 12], npix, ncomp, seed=over)
+    m = torch.ones(npix, ncomp, dtype=torch.float64, device="cuda")
+    plan.messenger(m, [math.inf, 5.0])
+    ref, _ = O.run_messenger(prob, [math.inf, 5.0])
+    assert np.linalg.norm(m.cpu().numpy() - ref) <= 1e-5 * np.linalg.norm(ref)
