@@ -17,7 +17,7 @@
  *    `workspace`, sized by mm_plan_workspace_size.
  *  - `stream` is a cudaStream_t passed as void* (NULL = legacy default stream).  Calls are
  *    asynchronous on that stream unless documented otherwise.
- *  - Pointing: pix int32 [n] (-1 = sample excluded), and for IQU maps cos 2psi / sin 2psi
+ *  - Pointing: pix int32 [n] (-1 = sample excluded, whatever its weights), and for IQU maps cos 2psi / sin 2psi
  *    [n] in FP32 (MM_W_F32) or FP16 (MM_W_F16).  Pointing weights of a sample are
  *    (1, cos 2psi, sin 2psi) (single pencil beam, Sec. 2.1).  The plan keeps the pointing
  *    pointers: they must stay valid and unchanged for the plan's lifetime.
@@ -171,8 +171,9 @@ mm_status mm_plan_batches(mm_plan p, int* n_batches);
  * (mm_plan_fused_batches), else GATHER_FFT(b), FILTER(b), IFFT_BIN(b); then MAP.  The same
  * sequence through this entry point gives identical results, and the three separate stages
  * on a fused batch the same up to the order of the FP64 pixel additions.  Small plans (a few
- * short chunks) run mm_messenger_iterate and mm_messenger_graph as one launch for the whole
- * schedule instead; these stages then give its results up to FP32 rounding.
+ * short chunks on a map of at most some thousand pixels per CTA) run mm_messenger_iterate and
+ * mm_messenger_graph as one launch for the whole schedule instead; these stages then give its
+ * results up to FP32 rounding.
  *   MM_STAGE_LOAD:       map_inout (device float64 [n_pix][ncomp]) -> internal FP32 map;
  *   MM_STAGE_GATHER_FFT: P m gathered from the internal map, packed, column DFTs (Eq. 1);
  *   MM_STAGE_FILTER:     row DFTs, per-mode messenger filter at `lambda` (>= 1 or INFINITY),
@@ -357,6 +358,8 @@ mm_status mm_chi2_modes(mm_plan p, const double* map, double lambda, double* chi
  * iteration graph (recaptured on the next mm_messenger_graph).  mm_set_tune sets a schedule
  * explicitly (MM_ERR_ARG for values outside those sets); mm_get_tune reads it (NULL
  * outputs are skipped).  Results do not depend on the schedule beyond FP32 rounding.
+ * Small plans (mm_messenger_stage) take only the order of the radices from it in the solver's one
+ * launch, and all of it in their other calls.
  * Plans with only power-of-two chunks ignore all three. */
 mm_status mm_autotune(mm_plan p, void* stream);
 mm_status mm_set_tune(mm_plan p, int col_nb, int col_threads, int row_threads, int radix_order,

@@ -9,7 +9,7 @@
 // over all CTAs between two grid barriers (one cluster: the cluster's own barrier), and one
 // launch runs the whole schedule.  What bounds an iteration is then the chain of barriers,
 // exchanges and L2 round trips.  Measured: one chunk of 2^15 samples, T-only, 101 iterations
-// 2.10 -> 1.16 ms; 12 ragged IQU chunks of 1500 to 12000 samples, 21 iterations 844 -> 328 us.
+// 2.10 -> 1.16 ms; 12 ragged IQU chunks of 1500 to 12000 samples, 21 iterations 844 -> 321 us.
 //
 // Lengths are general (radices 2, 3, 4, 5, 8, 16 at run time), with the layouts and scales of
 // the other paths: row layout of d~ and Nbar, sums scaled by 1 / (n tau).
