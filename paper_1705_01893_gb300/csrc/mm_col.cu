@@ -15,8 +15,8 @@ template <int M1, int CB, int T, int NC, int SRC, bool ROOMY>
 __global__ void __launch_bounds__(T, pass_ctas(T, 8, ROOMY)) k_col_forward(ColParams q) {
   extern __shared__ float2 sm[];
   // the tile's four-step twiddles from shared memory, but for 32-point columns, which use each
-  // entry once (1000 x 2^12 samples, T-only: 4 iterations 266 us without, 276 with; 16 points, whose one
-  // pass hides the copy: 4000 x 2^10 328 / 311; 128 points and more: with)
+  // entry once (4 T-only iterations of 1000 x 2^12 samples 266 us without, 276 with; 16 points, whose
+  // one pass hides the copy, 4000 x 2^10: 328 / 311; longer columns use entries many times)
   constexpr bool kStage = SRC != kSrcTod && M1 != 32;
   __shared__ float2 s4[kStage ? four_step_n(M1, kColLo) * CB : 1];
   const int M2 = q.g.M2;

@@ -45,14 +45,15 @@ __device__ __forceinline__ float4 load_w4(const void* w, int half_w, int64_t s) 
 }
 
 // (P m) of two consecutive samples; the weights of an excluded one (pixel -1) must be finite, as
-// those of the tile-order copies are (included_w).  They share a pixel more often than not, and
-// then one map load serves both: the gathers are short of L1 requests (a vertical sweep touches a line per
-// pixel), not of bytes.  256^2, 4 x 2^20: 1523 -> 1461 us per
-// 21 iterations; the 20-step gradient 6424 -> 6009 us; 512^2, 8 x 2^22: 435 -> 432 us an iteration.
+// those of the tile-order copies are (included_w).  The two share a pixel more often than not, and
+// then one map load serves both: the gathers are short of L1 requests (a vertical sweep touches a
+// line per pixel), not of bytes.  256^2, 4 x 2^20: 1523 -> 1461 us per 21 iterations; the 20-step
+// gradient 6424 -> 6009 us; 512^2, 8 x 2^22: 435 -> 432 us an iteration.
 // kShare: on for IQU.  T-only loads are a quarter of the size, and the second one's wait for the
 // compare of the pixels costs more than it saves (forward columns of 250 x 2^14 samples 14.3 us
-// against 20.7, 1000 x 2^12 16.5 / 20.8; 16 x 2^18, 4 iterations: 220 / 228), but for the long columns
-// in narrower tiles (4 iterations of 2 x 2^24 samples 1369 us sharing, 1408 not; 4 x 2^23 1316 / 1324).
+// against 20.7, 1000 x 2^12 16.5 / 20.8; 4 iterations of 16 x 2^18 220 / 228), but for the long
+// columns in narrower tiles (4 iterations of 2 x 2^24 samples 1369 us sharing, 1408 not; 4 x 2^23
+// 1316 / 1324).
 template <int NC, bool kShare = NC == 3>
 __device__ __forceinline__ float2 gather_two(const ColParams& q, int p0, int p1, float c0, float c1,
                                              float s0, float s1) {
@@ -303,9 +304,9 @@ struct DstY {
   }
 };
 
-// The same with the plan-wide two-level table, for 32-point columns and the transform of the data: that runs once per
-// data set, and its rounding reaches every later iterate through d~ (1/f noise spreads it over
-// the high frequencies), so it stays as it was.
+// The same with the plan-wide two-level table, for 32-point columns (see k_col_forward) and the
+// transform of the data: that runs once per data set, and its rounding reaches every later iterate
+// through d~ (1/f noise spreads it over the high frequencies), so it stays as it was.
 struct DstYTable {
   float2* y;
   const Group* g;

@@ -96,9 +96,9 @@ static cudaError_t row_m2(const mm_plan_s* p, const Batch& b, const RowArgs& a,
   const RowParams q = make_row_params(p, b, a);
   const size_t smem = sizeof(float2) * (2 * M2 + tw_size(M2));
   // the per-iteration modes (messenger step, its map-sized form) get their own instances
-  // with the mode folded in, the two of the data transform one of their own (no filter and no inverse
-  // DFTs, hence fewer registers: rfft of 2000 x 2^11 samples 53.9 -> 48.5 us, 40 x 2^16 32.6 -> 27.1, 8 x 2^22
-  // 257 -> 246); the others share one
+  // with the mode folded in, the two of the data transform one of their own (no filter and no
+  // inverse DFTs, hence fewer registers: rfft of 2000 x 2^11 samples 53.9 -> 48.5 us, 40 x 2^16
+  // 32.6 -> 27.1, 8 x 2^22 257 -> 246); the others share one
   constexpr bool R = T < 512;   // one instance only from 512 threads on
   const bool data = a.mode == kRowSpectrum || a.mode == kRowNatural;
   auto roomy = data                       ? k_row<M2, T, kRowDataModes, R>
